@@ -1,12 +1,14 @@
 // FP64 kernels of the RI-MP2 hot path: grouped persistent DFMA GEMM for the four
 // contractions (Eq. MP2_ints for V; Appendix Gamma, D^MP2_ab, D^MP2_ij), the amplitude
 // pass (T -> Tt = 2T - T^T and the pair energies), the compensated energy reduction,
-// and input checks.  CUDA-core FP64 on sm_103a: the GEMM keeps a 64x64 tile per CTA
-// with a 4x4 register block per thread; work tiles come from a device queue (an
-// atomic counter) in the order the host sorted them (largest K first).
+// and input checks.  CUDA-core FP64 on sm_103a: the GEMM's work items (fp64_gemm.cuh) come
+// from a device queue (an atomic counter) in the order the host sorted them (largest
+// first).
 #include <math.h>
 
-#include "rimp2_internal.cuh"
+#include <algorithm>
+
+#include "fp64_gemm.cuh"
 
 namespace rimp2 {
 
@@ -18,15 +20,6 @@ __device__ __forceinline__ int find_prob(const GemmProb* __restrict__ probs, int
     if (probs[mid].tile_begin <= t) lo = mid; else hi = mid - 1;
   }
   return lo;
-}
-
-// Upper-triangle enumeration, column by column: t -> (r, c) with r <= c.
-__device__ __forceinline__ void tri_index(long long t, int& r, int& c) {
-  long long cc = (long long)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
-  while (cc * (cc + 1) / 2 > t) --cc;
-  while ((cc + 1) * (cc + 2) / 2 <= t) ++cc;
-  c = (int)cc;
-  r = (int)(t - cc * (cc + 1) / 2);
 }
 
 template <typename F>
@@ -45,117 +38,95 @@ __device__ __forceinline__ int find_frag(const FragDev* __restrict__ frags, int 
 __global__ void __launch_bounds__(256, 2)
 k_gemm_f64(const GemmProb* __restrict__ probs, int nprobs, long long total, Bases bs,
            unsigned* __restrict__ counter, const int* __restrict__ skip) {
-  __shared__ double As[F64_BK][F64_BM + 1];
-  __shared__ double Bs[F64_BK][F64_BN + 1];
-  __shared__ long long s_tile;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  __shared__ F64Smem sm;
+  __shared__ GemmProb P;
+  __shared__ int s_tm, s_tn, s_ks, s_done;
   if (skip && *(volatile const int*)skip) return;
-
   for (;;) {
-    if (tid == 0) s_tile = (long long)atomicAdd(counter, 1u);
+    if (threadIdx.x < 32) {
+      // the first warp takes the next item, finds its problem and copies the descriptor
+      long long t = 0;
+      int pi = 0;
+      if (threadIdx.x == 0) {
+        t = (long long)atomicAdd(counter, 1u);
+        s_done = t >= total;
+        if (t < total) pi = find_prob(probs, nprobs, t);
+      }
+      pi = __shfl_sync(0xffffffffu, pi, 0);
+      static_assert(sizeof(GemmProb) % 8 == 0, "copied in 8-byte words");
+      for (int w = threadIdx.x; w < (int)(sizeof(GemmProb) / 8); w += 32)
+        ((long long*)&P)[w] = ((const long long*)(probs + pi))[w];
+      __syncwarp();
+      if (threadIdx.x == 0 && t < total) f64_decode(P, t - P.tile_begin, s_tm, s_tn, s_ks);
+    }
     __syncthreads();
-    const long long t = s_tile;
-    if (t >= total) break;
-    const GemmProb P = probs[find_prob(probs, nprobs, t)];
-    const long long lt = t - P.tile_begin;
-    const int ks = (int)(lt % P.ksplit);
-    const long long tt = lt / P.ksplit;
-    int tm, tn;
-    if (P.kind == PK_V) tri_index(tt, tm, tn);
-    else { tm = (int)(tt / P.tiles_n); tn = (int)(tt % P.tiles_n); }
-    const int m0 = tm * F64_BM, n0 = tn * F64_BN;
-    const double* __restrict__ A =
-        P.kind == PK_GEN ? P.pa : (P.kind == PK_V ? bs.B : bs.ws) + P.a_off;
-    const double* __restrict__ Bo = P.kind == PK_GEN ? P.pb : (P.b_from_B ? bs.B : bs.ws) + P.b_off;
-    const bool a_kc = (P.sAk == 1), b_kc = (P.sBk == 1);
+    if (s_done) break;
+    f64_item(P, bs, s_tm, s_tn, s_ks, sm);
+    __syncthreads();  // the shared tile and descriptor are rewritten for the next item
+  }
+}
 
-    double acc[4][4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[r][c] = 0.0;
-
-    const int k1b = ks * P.k1_chunk;
-    const int k1e = min(P.K1, k1b + P.k1_chunk);
-    for (int k1 = k1b; k1 < k1e; ++k1) {
-      for (int k0 = 0; k0 < P.K0; k0 += F64_BK) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int e = tid + 256 * q;
-          int mm, kk;
-          if (a_kc) { kk = e & 15; mm = e >> 4; } else { mm = e & 63; kk = e >> 6; }
-          const int gm = m0 + mm, gk = k0 + kk;
-          double val = 0.0;
-          if (gm < P.M && gk < P.K0)
-            val = A[(long long)gm * P.sAm + (long long)gk * P.sAk + (long long)k1 * P.sA1];
-          As[kk][mm] = val;
-          int nn, kb;
-          if (b_kc) { kb = e & 15; nn = e >> 4; } else { nn = e & 63; kb = e >> 6; }
-          const int gn = n0 + nn, gkb = k0 + kb;
-          double vb = 0.0;
-          if (gn < P.N && gkb < P.K0)
-            vb = Bo[(long long)gn * P.sBn + (long long)gkb * P.sBk + (long long)k1 * P.sB1];
-          Bs[kb][nn] = vb;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < F64_BK; ++kk) {
-          double a[4], b[4];
-#pragma unroll
-          for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) b[c] = Bs[kk][tx + 16 * c];
-#pragma unroll
-          for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[r][c] = fma(a[r], b[c], acc[r][c]);
-        }
-        __syncthreads();
-      }
+// Tile width, K pieces and queue position of every problem of one launch (sorted longest
+// item first).  An item should hold about 1 / per_sm of an SM's share of the launch: large
+// enough to amortise its start (queue, descriptor, first loads), small enough that the last
+// items end together.  At nocc=10 nvir=40 naux=150 fixed 64 x 64 tiles put V on 28 of the
+// 152 SMs and P_ij (10 x 10) into a tile with 1 / 41 of it filled: 1020 us for both GEMM
+// launches.
+void plan_f64_tiles(std::vector<GemmProb>& v, int grid, int per_sm, long long& total) {
+  auto up16 = [](long long x) { return (x + 15) / 16 * 16; };
+  auto work = [&](const GemmProb& P) {
+    return (double)P.M * P.N * (double)std::max(1LL, P.k_total) * (P.sym ? 0.5 : 1.0);
+  };
+  double all = 0.0;
+  for (const auto& P : v) all += work(P);
+  const int sms = std::max(1, grid / 2);   // two CTAs per SM
+  const double unit = std::max(all / ((double)sms * per_sm), 1.0);
+  // FMAs a symmetric problem spends with tiles of width bt (triangle of tiles, edges in 16s)
+  auto padded = [&](const GemmProb& P, int bt) {
+    double s = 0.0;
+    for (long long c = 0; c * bt < P.N; ++c) {
+      const double w = (double)std::min<long long>(bt, up16(P.N - c * bt));
+      s += w * (double)std::min<long long>((c + 1) * bt, up16(P.M));
     }
-
-    // epilogue
-    if (P.kind == PK_V) {
-      double* __restrict__ C = bs.ws + P.c_off;
-      const double* eo = bs.eps + P.eo_off;
-      const double* ev = bs.eps + P.ev_off;
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int m = m0 + ty + 16 * r;
-        if (m >= P.M) continue;
-        const int i = m / P.v, a = m - i * P.v;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int n = n0 + tx + 16 * c;
-          if (n >= P.N) continue;
-          const int j = n / P.v, b = n - j * P.v;
-          const double D = eo[i] + eo[j] - ev[a] - ev[b];
-          const double T = acc[r][c] / D;
-          C[(long long)m * P.ldc + n] = T;
-          if (tm != tn) C[(long long)n * P.ldc + m] = T;
-        }
-      }
+    return s;
+  };
+  for (auto& P : v) {
+    const bool split = P.kind == PK_PAB || P.kind == PK_PIJ || (P.kind == PK_GEN && P.accumulate);
+    const double K = (double)std::max(1LL, P.k_total);
+    auto ext = [&](int bt, int n) { return (double)std::min<long long>(bt, up16(n)); };
+    int bt = F64_T;
+    if (split) {
+      // K pieces give the balance; narrower tiles only where they save padding above the
+      // diagonal or the pieces would get short
+      if (P.sym)
+        while (bt > 16 && padded(P, bt) > 1.06 * padded(P, bt / 2)) bt /= 2;
+      while (bt > 16 && unit / (ext(bt, P.M) * ext(bt, P.N)) < 256.0 && ext(bt, P.M) * ext(bt, P.N) > 256.0) bt /= 2;
+      long long ch = up16((long long)(unit / (ext(bt, P.M) * ext(bt, P.N))) + 1);
+      // P sums terms of one sign: bounded pieces also keep the rounding of their running
+      // sums where it was (a single 45,000-long chain quadrupled P_ij's 1e-15 error)
+      ch = std::min<long long>(std::max<long long>(ch, 128), bt == F64_T ? 32768 : 4096);
+      P.k_chunk = std::min<long long>(ch, std::max<long long>(up16(P.k_total), 16));
     } else {
-      double* __restrict__ C =
-          P.kind == PK_GEN ? P.pc
-                           : (P.kind == PK_GAMMA ? bs.gamma : P.kind == PK_PAB ? bs.pab : bs.pij) +
-                                 P.c_off;
-      const bool store = P.ksplit == 1 && (P.kind == PK_GAMMA || (P.kind == PK_GEN && !P.accumulate));
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int m = m0 + ty + 16 * r;
-        if (m >= P.M) continue;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int n = n0 + tx + 16 * c;
-          if (n >= P.N) continue;
-          const double val = P.alpha * acc[r][c];
-          if (store) C[(long long)m * P.ldc + n] = val;
-          else atomicAdd(C + (long long)m * P.ldc + n, val);
-        }
-      }
+      while (bt > 16 && ext(bt, P.M) * ext(bt, P.N) * K > unit) bt /= 2;
+      P.k_chunk = std::max<long long>(up16(P.k_total), 16);
     }
-    __syncthreads();  // s_tile is rewritten at the top of the next iteration
+    P.bt = bt;
+    P.ksplit = (int)std::max<long long>(1, (P.k_total + P.k_chunk - 1) / P.k_chunk);
+    P.tiles_m = (P.M + bt - 1) / bt;
+    P.tiles_n = (P.N + bt - 1) / bt;
+    P.ntiles = (P.sym ? (long long)P.tiles_m * (P.tiles_m + 1) / 2 : (long long)P.tiles_m * P.tiles_n) * P.ksplit;
+  }
+  std::stable_sort(v.begin(), v.end(), [&](const GemmProb& a, const GemmProb& b) {
+    auto cost = [&](const GemmProb& P) {
+      return (double)std::min<long long>(P.bt, up16(P.M)) * (double)std::min<long long>(P.bt, up16(P.N)) *
+             (double)std::min<long long>(P.k_chunk, std::max(1LL, P.k_total));
+    };
+    return cost(a) > cost(b);
+  });
+  total = 0;
+  for (auto& P : v) {
+    P.tile_begin = total;
+    total += P.ntiles;
   }
 }
 

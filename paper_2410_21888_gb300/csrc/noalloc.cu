@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include <mutex>
+#include <vector>
 
 #include "rimp2_internal.cuh"
 
@@ -109,16 +110,14 @@ extern "C" int rimp2_energy_fp64_noalloc(int32_t nocc, int32_t nvir, int32_t nau
   long long tiles = 0;
   if (ov > 0) {
     P.kind = PK_V; P.frag = 0;
-    P.M = P.N = (int)ov; P.K0 = naux; P.K1 = 1;
-    P.tiles_m = P.tiles_n = (int)((ov + F64_BM - 1) / F64_BM);
-    P.ksplit = 1; P.k1_chunk = 1;
-    P.ntiles = (long long)P.tiles_m * (P.tiles_m + 1) / 2;
-    P.tile_begin = 0;
+    P.M = P.N = (int)ov; P.K0 = naux; P.k_total = naux; P.sym = 1;
     P.a_off = 0; P.b_off = 0; P.c_off = fd.t_off;
     P.sAm = naux; P.sAk = 1; P.sA1 = 0; P.sBn = naux; P.sBk = 1; P.sB1 = 0;
     P.ldc = (long long)ov; P.alpha = 1.0;
     P.eo_off = 0; P.ev_off = nocc; P.v = nvir; P.b_from_B = 1;
-    tiles = P.ntiles;
+    std::vector<GemmProb> one(1, P);
+    plan_f64_tiles(one, grid, F64_ITEMS_V, tiles);
+    P = one[0];
   }
   k_noalloc_header<<<1, 32, 0, s>>>((unsigned char*)scratch, fd, P);
   cudaError_t e = cudaGetLastError();

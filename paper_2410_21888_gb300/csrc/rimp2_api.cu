@@ -151,31 +151,6 @@ int check_frag_shapes(const rimp2_frag* frags, int nfrag) {
   return RIMP2_OK;
 }
 
-// split-K factor over the outer K index so that small M x N problems fill the GPU
-void choose_split(GemmProb& P, int grid, int mul) {
-  const long long tiles = (long long)P.tiles_m * P.tiles_n;
-  long long want = std::max(1LL, ((long long)mul * grid + tiles - 1) / tiles);
-  want = std::min<long long>(want, P.K1);
-  int chunk = (int)((P.K1 + want - 1) / want);
-  if (chunk < 1) chunk = 1;
-  P.k1_chunk = chunk;
-  P.ksplit = (P.K1 + chunk - 1) / chunk;
-  if (P.ksplit < 1) P.ksplit = 1;
-}
-
-void finish_probs(std::vector<GemmProb>& v, long long& total) {
-  // largest work per tile first (LPT order of the device queue)
-  std::stable_sort(v.begin(), v.end(), [](const GemmProb& a, const GemmProb& b) {
-    const double ca = (double)a.K0 * a.k1_chunk, cb = (double)b.K0 * b.k1_chunk;
-    return ca > cb;
-  });
-  total = 0;
-  for (auto& P : v) {
-    P.tile_begin = total;
-    total += P.ntiles;
-  }
-}
-
 int build_fp64_wave(rimp2_plan* p, const rimp2_frag* frags, WaveDesc& w) {
   size_t ws = 0;
   long long pairs = 0;
@@ -199,14 +174,11 @@ int build_fp64_wave(rimp2_plan* p, const rimp2_frag* frags, WaveDesc& w) {
     w.max_b = std::max<long long>(w.max_b, (long long)ov * f.naux);
     if (ov == 0) continue;
     const int o = f.nocc, v = f.nvir, X = f.naux;
-    // V: rows (i,a), cols (j,b), K = Q; upper triangle of tiles
+    // V: rows (i,a), cols (j,b), K = Q; upper triangle of tiles, mirrored
     {
       GemmProb P{};
       P.kind = PK_V; P.frag = idx;
-      P.M = P.N = (int)ov; P.K0 = X; P.K1 = 1;
-      P.tiles_m = P.tiles_n = (int)((ov + F64_BM - 1) / F64_BM);
-      P.ksplit = 1; P.k1_chunk = 1;
-      P.ntiles = (long long)P.tiles_m * (P.tiles_m + 1) / 2;
+      P.M = P.N = (int)ov; P.K0 = X; P.k_total = X; P.sym = 1;
       P.a_off = f.b_off; P.b_off = f.b_off; P.c_off = d.t_off;
       P.sAm = X; P.sAk = 1; P.sA1 = 0; P.sBn = X; P.sBk = 1; P.sB1 = 0; P.ldc = (long long)ov;
       P.alpha = 1.0; P.eo_off = f.eo_off; P.ev_off = f.ev_off; P.v = v; P.b_from_B = 1;
@@ -215,10 +187,7 @@ int build_fp64_wave(rimp2_plan* p, const rimp2_frag* frags, WaveDesc& w) {
     if (f.gamma_off >= 0 && X > 0) {  // Gamma[(i,a)][Q] = sum_(j,b) Tt[(i,a)][(j,b)] B[(j,b)][Q]
       GemmProb P{};
       P.kind = PK_GAMMA; P.frag = idx;
-      P.M = (int)ov; P.N = X; P.K0 = (int)ov; P.K1 = 1;
-      P.tiles_m = (int)((ov + F64_BM - 1) / F64_BM); P.tiles_n = (X + F64_BN - 1) / F64_BN;
-      P.ksplit = 1; P.k1_chunk = 1;
-      P.ntiles = (long long)P.tiles_m * P.tiles_n;
+      P.M = (int)ov; P.N = X; P.K0 = (int)ov; P.k_total = (long long)ov;
       P.a_off = d.tt_off; P.b_off = f.b_off; P.c_off = f.gamma_off;
       P.sAm = (long long)ov; P.sAk = 1; P.sA1 = 0;
       P.sBn = 1; P.sBk = X; P.sB1 = 0; P.ldc = X;
@@ -228,33 +197,27 @@ int build_fp64_wave(rimp2_plan* p, const rimp2_frag* frags, WaveDesc& w) {
     if (f.pab_off >= 0) {  // P_ab = sum_i Tt[i][a][:] . T[i][b][:]
       GemmProb P{};
       P.kind = PK_PAB; P.frag = idx;
-      P.M = P.N = v; P.K0 = (int)ov; P.K1 = o;
-      P.tiles_m = P.tiles_n = (v + F64_BM - 1) / F64_BM;
+      P.M = P.N = v; P.K0 = (int)ov; P.k_total = (long long)ov * o; P.sym = 1;
       P.a_off = d.tt_off; P.b_off = d.t_off; P.c_off = f.pab_off;
       P.sAm = (long long)ov; P.sAk = 1; P.sA1 = (long long)v * ov;
       P.sBn = (long long)ov; P.sBk = 1; P.sB1 = (long long)v * ov; P.ldc = v;
       P.alpha = 1.0; P.v = v; P.b_from_B = 0;
-      choose_split(P, p->gemm_grid, 2 << p->variant);
-      P.ntiles = (long long)P.tiles_m * P.tiles_n * P.ksplit;
       w.probs_c.push_back(P);
     }
     if (f.pij_off >= 0) {  // P_ij = -sum_(k,b) sum_a Tt[k][b][i][a] T[k][b][j][a]
       GemmProb P{};
       P.kind = PK_PIJ; P.frag = idx;
-      P.M = P.N = o; P.K0 = v; P.K1 = (int)ov;
-      P.tiles_m = P.tiles_n = (o + F64_BM - 1) / F64_BM;
+      P.M = P.N = o; P.K0 = v; P.k_total = (long long)ov * v; P.sym = 1;
       P.a_off = d.tt_off; P.b_off = d.t_off; P.c_off = f.pij_off;
       P.sAm = v; P.sAk = 1; P.sA1 = (long long)ov;
       P.sBn = v; P.sBk = 1; P.sB1 = (long long)ov; P.ldc = o;
       P.alpha = -1.0; P.v = v; P.b_from_B = 0;
-      choose_split(P, p->gemm_grid, 2 << p->variant);
-      P.ntiles = (long long)P.tiles_m * P.tiles_n * P.ksplit;
       w.probs_c.push_back(P);
     }
   }
   w.total_pairs = pairs;
-  finish_probs(w.probs_v, w.tiles_v);
-  finish_probs(w.probs_c, w.tiles_c);
+  plan_f64_tiles(w.probs_v, p->gemm_grid, F64_ITEMS_V, w.tiles_v);
+  plan_f64_tiles(w.probs_c, p->gemm_grid, F64_ITEMS_C << p->variant, w.tiles_c);
   // the layout must fit the workspace the plan sized with frag_ws_elems_fp64
   if (ws * sizeof(double) + 256 > p->ws_bytes) return RIMP2_ERR_WORKSPACE;
   return RIMP2_OK;
@@ -380,7 +343,7 @@ void drop_graph(rimp2_plan* p) {
   p->graph = nullptr;
 }
 
-constexpr int kFp64Variants = 3;   // FP64 path: split-K target 2, 4, 8 x grid
+constexpr int kFp64Variants = 3;   // FP64 path: 8, 16, 32 work items per SM in the Gamma / P launch
 
 uint64_t fnv(uint64_t h, uint64_t x) {
   for (int b = 0; b < 8; ++b) {

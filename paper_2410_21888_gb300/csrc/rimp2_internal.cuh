@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "rimp2.h"
 
 namespace rimp2 {
@@ -91,12 +93,14 @@ struct Bases {
   unsigned* status;
 };
 
-// One GEMM-shaped problem C(m,n) = alpha * sum_{k1,k0} A(m,k0,k1) Bop(n,k0,k1).
-// A(m,k0,k1) = A[a_off + m*sAm + k0*sAk + k1*sA1]; Bop likewise with n.
+// One GEMM-shaped problem C(m,n) = alpha * sum_k A(m,k) Bop(n,k) over the flat index
+// k = k1 K0 + k0 < k_total: A(m,k) = A[a_off + m*sAm + k0*sAk + k1*sA1]; Bop likewise with n.
+// Tiles, K pieces and queue positions are set by plan_f64_tiles.
 struct GemmProb {
   int kind, frag;
-  int M, N, K0, K1;
-  int tiles_m, tiles_n, ksplit, k1_chunk;
+  int M, N, K0, sym;         // sym: C is symmetric, only tiles on or above the diagonal
+  int tiles_m, tiles_n, ksplit, bt;   // bt: tile width, 16, 32 or 64
+  long long k_total, k_chunk;
   long long tile_begin, ntiles;  // position in the flattened work queue
   long long a_off, b_off, c_off; // a from B (PK_V) or ws; b from B (PK_V, PK_GAMMA) or ws
   long long sAm, sAk, sA1, sBn, sBk, sB1, ldc;
@@ -128,14 +132,14 @@ cudaError_t launch_gemm_f64(const GemmProb* d_probs, int nprobs, long long total
                             Bases bs, unsigned* counter, int grid, cudaStream_t s,
                             const int* skip = nullptr);
 int gemm_f64_occupancy_grid();
+// Work items per SM a launch is cut into (more: better balance, shorter items).  V, whose
+// tiles cannot be cut along K, takes 16 (nocc=29 nvir=117 naux=437: 4.59 ms with 8, 4.37
+// with 16 or 32), the other contractions 8 (10.61 ms, 10.77 with 16).
+constexpr int F64_ITEMS_V = 16, F64_ITEMS_C = 8;
+void plan_f64_tiles(std::vector<GemmProb>& probs, int grid, int per_sm, long long& total);
 cudaError_t launch_amplitude_f64(const FragDev* d_frags, int nfrag, long long total_pairs,
                                  Bases bs, cudaStream_t s);
 cudaError_t launch_energy_reduce(const FragDev* d_frags, int nfrag, Bases bs, cudaStream_t s);
 cudaError_t launch_zero_p(const FragDev* d_frags, int nfrag, Bases bs, cudaStream_t s);
-
-// tile sizes of the FP64 grouped GEMM
-constexpr int F64_BM = 64;
-constexpr int F64_BN = 64;
-constexpr int F64_BK = 16;
 
 }  // namespace rimp2

@@ -195,32 +195,15 @@ __global__ void k_cg_finish(const CgState* st, int max_iter, double* info) {
 // C(m,n) = alpha sum_{k1,k0} A[m sAm + k0 sAk + k1 sA1] Bop[n sBn + k0 sBk + k1 sB1]
 GemmProb gen(int M, int N, int K0, int K1, const double* a, long long sAm, long long sAk,
              long long sA1, const double* b, long long sBn, long long sBk, long long sB1,
-             double* c, long long ldc, double alpha, bool accumulate, int grid) {
+             double* c, long long ldc, double alpha, bool accumulate) {
   GemmProb P{};
   P.kind = PK_GEN;
-  P.M = M; P.N = N; P.K0 = K0; P.K1 = std::max(K1, 1);
-  P.tiles_m = (M + F64_BM - 1) / F64_BM;
-  P.tiles_n = (N + F64_BN - 1) / F64_BN;
+  P.M = M; P.N = N; P.K0 = K0; P.k_total = (long long)K0 * K1;
   P.pa = a; P.sAm = sAm; P.sAk = sAk; P.sA1 = sA1;
   P.pb = b; P.sBn = sBn; P.sBk = sBk; P.sB1 = sB1;
   P.pc = c; P.ldc = ldc; P.alpha = alpha;
   P.accumulate = accumulate ? 1 : 0;
-  const long long tiles = (long long)P.tiles_m * P.tiles_n;
-  long long want = 1;
-  if (accumulate && tiles > 0) want = std::max(1LL, (2LL * grid + tiles - 1) / tiles);
-  want = std::min<long long>(want, P.K1);
-  P.k1_chunk = (int)((P.K1 + want - 1) / want);
-  P.ksplit = (P.K1 + P.k1_chunk - 1) / P.k1_chunk;
-  P.ntiles = tiles * P.ksplit;
   return P;
-}
-
-void finish(std::vector<GemmProb>& v, long long& total) {
-  std::stable_sort(v.begin(), v.end(), [](const GemmProb& a, const GemmProb& b) {
-    return (double)a.K0 * a.k1_chunk > (double)b.K0 * b.k1_chunk;
-  });
-  total = 0;
-  for (auto& P : v) { P.tile_begin = total; total += P.ntiles; }
 }
 
 struct Layout {
@@ -315,36 +298,36 @@ int rimp2_zvec_solve(const rimp2_zvec_args* A, void* workspace, size_t ws_bytes,
   // 0: Gamma^P[(i,a)][P] = sum_Q Gamma[(i,a)][Q] J^{-1/2}[P][Q]
   if (A->jmh && A->gamma_p)
     lists[0].push_back(gen((int)ov, X, X, 1, A->gamma, X, 1, 0, A->jmh, X, 1, 0, A->gamma_p, X,
-                           1.0, false, grid));
+                           1.0, false));
   // 1: L'[i][q] = sum_(a,Q) Gamma[i][a][Q] B[q][o+a][Q]; L''[a][q] = sum_(i,Q) Gamma[i][a][Q] B[i][q][Q]
   lists[1].push_back(gen(o, n, X, v, A->gamma, (long long)v * X, 1, X, Bf + oX, nX, 1, X, A->lp, n,
-                         1.0, true, grid));
+                         1.0, true));
   lists[1].push_back(gen(v, n, X, o, A->gamma, X, 1, (long long)v * X, Bf, X, 1, nX, A->lpp, n,
-                         1.0, true, grid));
+                         1.0, true));
   // 2: U[i][l][Q] = sum_k D_kl B[i][k][Q];  V[i][c][Q] = sum_b D_bc B[i][o+b][Q]
   for (int i = 0; i < o; ++i) {
     lists[2].push_back(gen(o, X, o, 1, A->pij, o, 1, 0, Bf + (long long)i * nX, 1, X, 0,
-                           W + (long long)i * oX, X, 1.0, false, grid));
+                           W + (long long)i * oX, X, 1.0, false));
     lists[2].push_back(gen(v, X, v, 1, A->pab, v, 1, 0, Bf + (long long)i * nX + oX, 1, X, 0,
-                           Vv + (long long)i * v * X, X, 1.0, false, grid));
+                           Vv + (long long)i * v * X, X, 1.0, false));
   }
   // 3: rhs[i][a] += sum_(l,Q) B[l][o+a][Q] U[i][l][Q] + sum_(c,Q) B[o+a][o+c][Q] V[i][c][Q]
-  lists[3].push_back(gen(o, v, X, o, W, oX, 1, X, Bf + oX, X, 1, nX, rhs, v, 1.0, true, grid));
+  lists[3].push_back(gen(o, v, X, o, W, oX, 1, X, Bf + oX, X, 1, nX, rhs, v, 1.0, true));
   lists[3].push_back(gen(o, v, X, v, Vv, (long long)v * X, 1, X, Bf + (long long)o * nX + oX, nX, 1,
-                         X, rhs, v, 1.0, true, grid));
+                         X, rhs, v, 1.0, true));
   // 4: W[i][j][Q] = sum_b p[j][b] B[i][o+b][Q]
   for (int i = 0; i < o; ++i)
     lists[4].push_back(gen(o, X, v, 1, p, v, 1, 0, Bf + (long long)i * nX + oX, 1, X, 0,
-                           W + (long long)i * oX, X, 1.0, false, grid));
+                           W + (long long)i * oX, X, 1.0, false));
   // 5: Ap[i][a] -= sum_(j,Q) B[j][o+a][Q] W[i][j][Q]
-  lists[5].push_back(gen(o, v, X, o, W, oX, 1, X, Bf + oX, X, 1, nX, Ap, v, -1.0, true, grid));
+  lists[5].push_back(gen(o, v, X, o, W, oX, 1, X, Bf + oX, X, 1, nX, Ap, v, -1.0, true));
 
   std::vector<char> host(kDescBytes, 0);
   size_t doff[kDescLists];
   long long tiles[kDescLists];
   size_t off = 0;
   for (int k = 0; k < kDescLists; ++k) {
-    finish(lists[k], tiles[k]);
+    plan_f64_tiles(lists[k], grid, F64_ITEMS_C, tiles[k]);
     doff[k] = off;
     const size_t bytes = lists[k].size() * sizeof(GemmProb);
     if (off + bytes > kDescBytes) return RIMP2_ERR_UNSUPPORTED;
