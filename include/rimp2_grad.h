@@ -54,12 +54,12 @@ int rimp2_zvec_workspace_size(int32_t nocc, int32_t nvir, int32_t naux, int32_t 
 /* Enqueues the step on `stream`.  Outputs are overwritten.  The problem descriptors are
  * staged from host memory into the workspace during the call, which therefore waits for
  * the work already queued on the stream and is not stream-capturable; the step itself
- * runs asynchronously (the conjugate-gradient iterations are all enqueued; those after
- * convergence return at once on the device).  Errors: RIMP2_ERR_BAD_ARG for negative
- * sizes or a NULL required pointer, RIMP2_ERR_WORKSPACE when the workspace is NULL, not
- * 256-byte aligned or below rimp2_zvec_workspace_size, RIMP2_ERR_UNSUPPORTED when the
- * descriptor lists outgrow their 1 MB region (nocc above ~2000), RIMP2_ERR_CUDA for a
- * failed launch or copy. */
+ * runs asynchronously (the conjugate-gradient iterations are one cooperative launch, whose
+ * grid barriers have bounded waits: on expiry it ends as not converged).  Errors:
+ * RIMP2_ERR_BAD_ARG for negative sizes or a NULL required pointer, RIMP2_ERR_WORKSPACE when
+ * the workspace is NULL, not 256-byte aligned or below rimp2_zvec_workspace_size,
+ * RIMP2_ERR_UNSUPPORTED when the descriptor lists outgrow their 1.25 MB region (nocc above
+ * ~2000), RIMP2_ERR_CUDA for a failed launch or copy. */
 int rimp2_zvec_solve(const rimp2_zvec_args* args, void* workspace, size_t ws_bytes,
                      cudaStream_t stream);
 

@@ -12,16 +12,6 @@
 
 namespace rimp2 {
 
-__device__ __forceinline__ int find_prob(const GemmProb* __restrict__ probs, int nprobs,
-                                         long long t) {
-  int lo = 0, hi = nprobs - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (probs[mid].tile_begin <= t) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 template <typename F>
 __device__ __forceinline__ int find_frag(const FragDev* __restrict__ frags, int nfrag,
                                          long long t, F key) {
@@ -35,33 +25,16 @@ __device__ __forceinline__ int find_frag(const FragDev* __restrict__ frags, int 
 
 // ------------------------------------------------------------------ grouped GEMM
 
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, F64_CTAS)
 k_gemm_f64(const GemmProb* __restrict__ probs, int nprobs, long long total, Bases bs,
-           unsigned* __restrict__ counter, const int* __restrict__ skip) {
+           unsigned* __restrict__ counter) {
   __shared__ F64Smem sm;
-  __shared__ GemmProb P;
-  __shared__ int s_tm, s_tn, s_ks, s_done;
-  if (skip && *(volatile const int*)skip) return;
+  __shared__ F64Entry e;
   for (;;) {
-    if (threadIdx.x < 32) {
-      // the first warp takes the next item, finds its problem and copies the descriptor
-      long long t = 0;
-      int pi = 0;
-      if (threadIdx.x == 0) {
-        t = (long long)atomicAdd(counter, 1u);
-        s_done = t >= total;
-        if (t < total) pi = find_prob(probs, nprobs, t);
-      }
-      pi = __shfl_sync(0xffffffffu, pi, 0);
-      static_assert(sizeof(GemmProb) % 8 == 0, "copied in 8-byte words");
-      for (int w = threadIdx.x; w < (int)(sizeof(GemmProb) / 8); w += 32)
-        ((long long*)&P)[w] = ((const long long*)(probs + pi))[w];
-      __syncwarp();
-      if (threadIdx.x == 0 && t < total) f64_decode(P, t - P.tile_begin, s_tm, s_tn, s_ks);
-    }
+    if (threadIdx.x < 32) f64_next(probs, nprobs, total, counter, e);
     __syncthreads();
-    if (s_done) break;
-    f64_item(P, bs, s_tm, s_tn, s_ks, sm);
+    if (e.t >= total) break;
+    f64_item(e.P, bs, e.tm, e.tn, e.ks, sm);
     __syncthreads();  // the shared tile and descriptor are rewritten for the next item
   }
 }
@@ -72,21 +45,22 @@ k_gemm_f64(const GemmProb* __restrict__ probs, int nprobs, long long total, Base
 // items end together.  At nocc=10 nvir=40 naux=150 fixed 64 x 64 tiles put V on 28 of the
 // 152 SMs and P_ij (10 x 10) into a tile with 1 / 41 of it filled: 1020 us for both GEMM
 // launches.
-void plan_f64_tiles(std::vector<GemmProb>& v, int grid, int per_sm, long long& total) {
+int plan_f64_tiles(std::vector<GemmProb>& v, int grid, int per_sm, long long& total) {
   auto up16 = [](long long x) { return (x + 15) / 16 * 16; };
   auto work = [&](const GemmProb& P) {
     return (double)P.M * P.N * (double)std::max(1LL, P.k_total) * (P.sym ? 0.5 : 1.0);
   };
   double all = 0.0;
   for (const auto& P : v) all += work(P);
-  const int sms = std::max(1, grid / 2);   // two CTAs per SM
+  const int sms = std::max(1, grid / F64_CTAS);
   const double unit = std::max(all / ((double)sms * per_sm), 1.0);
-  // FMAs a symmetric problem spends with tiles of width bt (triangle of tiles, edges in 16s)
+  // FMAs per K element of a symmetric problem with tiles of width bt: whole columns of tiles
+  // above the diagonal (edges in 16s) and 8 x 8 blocks on it
   auto padded = [&](const GemmProb& P, int bt) {
     double s = 0.0;
     for (long long c = 0; c * bt < P.N; ++c) {
-      const double w = (double)std::min<long long>(bt, up16(P.N - c * bt));
-      s += w * (double)std::min<long long>((c + 1) * bt, up16(P.M));
+      const long long w = std::min<long long>(bt, P.N - c * bt), nb = (w + 7) / 8;
+      s += (double)(c * bt) * (double)up16(w) + 64.0 * (double)(nb * (nb + 1) / 2);
     }
     return s;
   };
@@ -99,12 +73,17 @@ void plan_f64_tiles(std::vector<GemmProb>& v, int grid, int per_sm, long long& t
       // K pieces give the balance; narrower tiles only where they save padding above the
       // diagonal or the pieces would get short
       if (P.sym)
-        while (bt > 16 && padded(P, bt) > 1.06 * padded(P, bt / 2)) bt /= 2;
+        if (padded(P, bt) > 1.03 * padded(P, bt / 2)) bt /= 2;
       while (bt > 16 && unit / (ext(bt, P.M) * ext(bt, P.N)) < 256.0 && ext(bt, P.M) * ext(bt, P.N) > 256.0) bt /= 2;
       long long ch = up16((long long)(unit / (ext(bt, P.M) * ext(bt, P.N))) + 1);
       // P sums terms of one sign: bounded pieces also keep the rounding of their running
       // sums where it was (a single 45,000-long chain quadrupled P_ij's 1e-15 error)
-      ch = std::min<long long>(std::max<long long>(ch, 128), bt == F64_T ? 32768 : 4096);
+      // At least 128 K elements amortise an item's start, or fewer where all pieces then still
+      // run at once (a chain of 64 is half as long; 32 cost more in additions to C)
+      const long long t = (P.M + bt - 1) / bt * (long long)((P.N + bt - 1) / bt);
+      const long long once = up16(P.k_total * t / std::max(grid, 1) + 1);
+      ch = std::max(ch, std::min<long long>(128, std::max<long long>(64, once)));
+      ch = std::min<long long>(ch, 4096);
       P.k_chunk = std::min<long long>(ch, std::max<long long>(up16(P.k_total), 16));
     } else {
       while (bt > 16 && ext(bt, P.M) * ext(bt, P.N) * K > unit) bt /= 2;
@@ -116,18 +95,22 @@ void plan_f64_tiles(std::vector<GemmProb>& v, int grid, int per_sm, long long& t
     P.tiles_n = (P.N + bt - 1) / bt;
     P.ntiles = (P.sym ? (long long)P.tiles_m * (P.tiles_m + 1) / 2 : (long long)P.tiles_m * P.tiles_n) * P.ksplit;
   }
-  std::stable_sort(v.begin(), v.end(), [&](const GemmProb& a, const GemmProb& b) {
-    auto cost = [&](const GemmProb& P) {
-      return (double)std::min<long long>(P.bt, up16(P.M)) * (double)std::min<long long>(P.bt, up16(P.N)) *
-             (double)std::min<long long>(P.k_chunk, std::max(1LL, P.k_total));
-    };
-    return cost(a) > cost(b);
-  });
+  auto cost = [&](const GemmProb& P) {
+    return (double)std::min<long long>(P.bt, up16(P.M)) * (double)std::min<long long>(P.bt, up16(P.N)) *
+           (double)std::min<long long>(P.k_chunk, std::max(1LL, P.k_total));
+  };
+  std::stable_sort(v.begin(), v.end(), [&](const GemmProb& a, const GemmProb& b) { return cost(a) > cost(b); });
   total = 0;
   for (auto& P : v) {
     P.tile_begin = total;
     total += P.ntiles;
   }
+  // The CTAs of an SM share its FP64 unit, so short items taken beside a long one only delay
+  // it: where the longest item is more than a quarter of an SM's share, fewer CTAs run
+  // (Gamma and P at nocc=10 nvir=40 naux=150: 115 us with four, 78 with two)
+  const double longest = v.empty() ? 0.0 : cost(v[0]), share = all / sms;
+  const int ctas = longest * F64_CTAS <= share ? F64_CTAS : longest * 3 <= share ? 3 : 2;
+  return sms * std::min(ctas, F64_CTAS);
 }
 
 int gemm_f64_occupancy_grid() {
@@ -140,11 +123,10 @@ int gemm_f64_occupancy_grid() {
 }
 
 cudaError_t launch_gemm_f64(const GemmProb* d_probs, int nprobs, long long total_tiles,
-                            Bases bs, unsigned* counter, int grid, cudaStream_t s,
-                            const int* skip) {
+                            Bases bs, unsigned* counter, int grid, cudaStream_t s) {
   if (total_tiles <= 0) return cudaSuccess;
   const long long g = total_tiles < grid ? total_tiles : grid;
-  k_gemm_f64<<<(unsigned)g, 256, 0, s>>>(d_probs, nprobs, total_tiles, bs, counter, skip);
+  k_gemm_f64<<<(unsigned)g, 256, 0, s>>>(d_probs, nprobs, total_tiles, bs, counter);
   return cudaGetLastError();
 }
 

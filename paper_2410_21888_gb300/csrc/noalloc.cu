@@ -116,7 +116,7 @@ extern "C" int rimp2_energy_fp64_noalloc(int32_t nocc, int32_t nvir, int32_t nau
     P.ldc = (long long)ov; P.alpha = 1.0;
     P.eo_off = 0; P.ev_off = nocc; P.v = nvir; P.b_from_B = 1;
     std::vector<GemmProb> one(1, P);
-    plan_f64_tiles(one, grid, F64_ITEMS_V, tiles);
+    grid = plan_f64_tiles(one, grid, F64_ITEMS_PER_SM, tiles);
     P = one[0];
   }
   k_noalloc_header<<<1, 32, 0, s>>>((unsigned char*)scratch, fd, P);

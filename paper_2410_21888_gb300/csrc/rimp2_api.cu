@@ -33,6 +33,7 @@ struct WaveDesc {
   std::vector<GemmProb> probs_v;      // stage 1: V (+ T epilogue)
   std::vector<GemmProb> probs_c;      // stage 2: Gamma, P_ab, P_ij
   long long tiles_v = 0, tiles_c = 0, total_pairs = 0, max_b = 0;
+  int grid_v = 0, grid_c = 0;         // FP64: CTAs of the two GEMM launches
   size_t off_fdev = 0, off_pv = 0, off_pc = 0;  // byte offsets into the plan device block
   SplitWave split;                    // split-path descriptors (split_path.cu)
 };
@@ -216,8 +217,8 @@ int build_fp64_wave(rimp2_plan* p, const rimp2_frag* frags, WaveDesc& w) {
     }
   }
   w.total_pairs = pairs;
-  plan_f64_tiles(w.probs_v, p->gemm_grid, F64_ITEMS_V, w.tiles_v);
-  plan_f64_tiles(w.probs_c, p->gemm_grid, F64_ITEMS_C << p->variant, w.tiles_c);
+  w.grid_v = plan_f64_tiles(w.probs_v, p->gemm_grid, F64_ITEMS_PER_SM, w.tiles_v);
+  w.grid_c = plan_f64_tiles(w.probs_c, p->gemm_grid, p->variant == 0 ? F64_ITEMS_PER_SM : (F64_ITEMS_PER_SM / 4) << (p->variant == 1 ? 1 : 3), w.tiles_c);
   // the layout must fit the workspace the plan sized with frag_ws_elems_fp64
   if (ws * sizeof(double) + 256 > p->ws_bytes) return RIMP2_ERR_WORKSPACE;
   return RIMP2_OK;
@@ -305,7 +306,7 @@ int enqueue(rimp2_plan* p, const rimp2_batch* b, void* ws, cudaStream_t s) {
     if (p->precision == RIMP2_FP64) {
       if (ev) cudaEventRecordWithFlags(ev[1], s, cudaEventRecordExternal);
       e = launch_gemm_f64((const GemmProb*)(p->dblk + w.off_pv), (int)w.probs_v.size(), w.tiles_v,
-                          bs, ctr + 0, p->gemm_grid, s);
+                          bs, ctr + 0, w.grid_v, s);
       launches += w.tiles_v > 0;
       if (ev) cudaEventRecordWithFlags(ev[2], s, cudaEventRecordExternal);
       if (e == cudaSuccess) { e = launch_amplitude_f64(dfd, nf, w.total_pairs, bs, s); launches += w.total_pairs > 0; }
@@ -314,7 +315,7 @@ int enqueue(rimp2_plan* p, const rimp2_batch* b, void* ws, cudaStream_t s) {
       if (ev) cudaEventRecordWithFlags(ev[3], s, cudaEventRecordExternal);
       if (e == cudaSuccess) {
         e = launch_gemm_f64((const GemmProb*)(p->dblk + w.off_pc), (int)w.probs_c.size(), w.tiles_c,
-                            bs, ctr + 1, p->gemm_grid, s);
+                            bs, ctr + 1, w.grid_c, s);
         launches += w.tiles_c > 0;
       }
       tiles += w.tiles_v + w.tiles_c;
@@ -343,7 +344,7 @@ void drop_graph(rimp2_plan* p) {
   p->graph = nullptr;
 }
 
-constexpr int kFp64Variants = 3;   // FP64 path: 8, 16, 32 work items per SM in the Gamma / P launch
+constexpr int kFp64Variants = 3;   // FP64 path: 16, 8 or 32 work items per SM in the Gamma / P launch
 
 uint64_t fnv(uint64_t h, uint64_t x) {
   for (int b = 0; b < 8; ++b) {

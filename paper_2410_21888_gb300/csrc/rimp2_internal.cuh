@@ -99,7 +99,7 @@ struct Bases {
 struct GemmProb {
   int kind, frag;
   int M, N, K0, sym;         // sym: C is symmetric, only tiles on or above the diagonal
-  int tiles_m, tiles_n, ksplit, bt;   // bt: tile width, 16, 32 or 64
+  int tiles_m, tiles_n, ksplit, bt;   // bt: tile width, 16 or 32
   long long k_total, k_chunk;
   long long tile_begin, ntiles;  // position in the flattened work queue
   long long a_off, b_off, c_off; // a from B (PK_V) or ws; b from B (PK_V, PK_GAMMA) or ws
@@ -127,16 +127,15 @@ struct FragDev {
 // ---- launchers (fp64_kernels.cu) ----
 cudaError_t launch_check_inputs(const FragDev* d_frags, int nfrag, long long max_bx,
                                 Bases bs, cudaStream_t s);
-// skip (device, may be null): when *skip != 0 at launch time every CTA returns at once
 cudaError_t launch_gemm_f64(const GemmProb* d_probs, int nprobs, long long total_tiles,
-                            Bases bs, unsigned* counter, int grid, cudaStream_t s,
-                            const int* skip = nullptr);
+                            Bases bs, unsigned* counter, int grid, cudaStream_t s);
 int gemm_f64_occupancy_grid();
-// Work items per SM a launch is cut into (more: better balance, shorter items).  V, whose
-// tiles cannot be cut along K, takes 16 (nocc=29 nvir=117 naux=437: 4.59 ms with 8, 4.37
-// with 16 or 32), the other contractions 8 (10.61 ms, 10.77 with 16).
-constexpr int F64_ITEMS_V = 16, F64_ITEMS_C = 8;
-void plan_f64_tiles(std::vector<GemmProb>& probs, int grid, int per_sm, long long& total);
+// Work items per SM a launch is cut into (more: better balance, shorter items): nocc=29
+// nvir=117 naux=437 takes 10.35 ms for Gamma and P with 16, 11.1 with 8, 10.5 with 32.
+constexpr int F64_ITEMS_PER_SM = 16;
+// Sets the tiles, K pieces and queue positions of one launch's problems; grid: CTAs that
+// fit the GPU.  Returns the CTAs to launch.
+int plan_f64_tiles(std::vector<GemmProb>& probs, int grid, int per_sm, long long& total);
 cudaError_t launch_amplitude_f64(const FragDev* d_frags, int nfrag, long long total_pairs,
                                  Bases bs, cudaStream_t s);
 cudaError_t launch_energy_reduce(const FragDev* d_frags, int nfrag, Bases bs, cudaStream_t s);
