@@ -59,14 +59,6 @@ __device__ __forceinline__ dfl d_add(dfl a, dfl b) {
   s.l += a.l + b.l;
   return d_fast(s.h, s.l);
 }
-__device__ __forceinline__ dfl d_neg(dfl a) { return {-a.h, -a.l}; }
-// (__fmul_rn: the rounded product must not be contracted into d_fast's addition)
-__device__ __forceinline__ dfl d_mul(dfl a, dfl b) {
-  const float p = __fmul_rn(a.h, b.h);
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, fmaf(a.l, b.h, e));
-  return d_fast(p, e);
-}
 __device__ __forceinline__ dfl d_from(double x) {
   const float h = (float)x;
   return {h, (float)(x - (double)h)};
@@ -173,6 +165,26 @@ __device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c) {
   return d;
 }
 
+__device__ __forceinline__ f2x f2_neg(f2x a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ f2x f2_two(float a) { return f2_pack(a, a); }
+// Double-float sum and product on two lanes (the f32x2 forms round each lane like the scalar
+// instruction and are never contracted)
+__device__ __forceinline__ void d_add2(f2x ah, f2x al, f2x bh, f2x bl, f2x& h, f2x& l) {
+  const f2x s = f2_add(ah, bh);
+  const f2x bb = f2_sub(s, ah);
+  const f2x e = f2_add(f2_sub(ah, f2_sub(s, bb)), f2_sub(bh, bb));
+  const f2x t = f2_add(e, f2_add(al, bl));
+  h = f2_add(s, t);
+  l = f2_sub(t, f2_sub(h, s));
+}
+__device__ __forceinline__ void d_mul2(f2x ah, f2x al, f2x bh, f2x bl, f2x& h, f2x& l) {
+  const f2x p = f2_mul(ah, bh);
+  f2x e = f2_fma(ah, bh, f2_neg(p));
+  e = f2_fma(ah, bl, f2_fma(al, bh, e));
+  h = f2_add(p, e);
+  l = f2_sub(e, f2_sub(h, p));
+}
+
 // digit_step on two elements at once, with the scaling by 2^LB folded into the Fast2Sum
 // (seven packed operations instead of eight, bit-identical): with a = xh - d and
 // s = a + xl as in digit_step, 2^LB s = RN(2^LB a + 2^LB xl) is one FMA; 2^LB (s - a) is
@@ -191,18 +203,16 @@ __device__ __forceinline__ f2x digit_step2(f2x& xh, f2x& xl) {
   return d;
 }
 
-// Digits of four consecutive elements (double-floats x[k] already scaled to the slice
-// frame), one packed store per slice plane; the digit steps run on element pairs.  NS > 0:
+// Digits of four consecutive elements (double-floats in element pairs, already scaled to the
+// slice frame), one packed store per slice plane; the digit steps run on element pairs.  NS > 0:
 // the plane count is NS, known at compile time (the loop unrolls; st is not read).
 // STREAM: the stores carry the evict-first hint (the amplitude kernel's digit planes are
 // far larger than L2 and are read back by later launches only).
 template <bool F8, int NS = 0, bool STREAM = false>
-__device__ __forceinline__ void put4(dfl x[4], int st, typename Digit<F8>::T* out,
-                                     long long plane) {
+__device__ __forceinline__ void put4(f2x h01, f2x l01, f2x h23, f2x l23, int st,
+                                     typename Digit<F8>::T* out, long long plane) {
   constexpr int LB = Digit<F8>::LB;
   using PT = typename Pack4<F8>::T;
-  f2x h01 = f2_pack(x[0].h, x[1].h), l01 = f2_pack(x[0].l, x[1].l);
-  f2x h23 = f2_pack(x[2].h, x[3].h), l23 = f2_pack(x[2].l, x[3].l);
   auto one = [&](int p) {
     float d0, d1, d2, d3;
     f2_unpack(digit_step2<LB>(h01, l01), d0, d1);
@@ -216,6 +226,12 @@ __device__ __forceinline__ void put4(dfl x[4], int st, typename Digit<F8>::T* ou
   } else {
     for (int p = 0; p < st; ++p) one(p);
   }
+}
+template <bool F8>
+__device__ __forceinline__ void put4(const dfl (&x)[4], int st, typename Digit<F8>::T* out,
+                                     long long plane) {
+  put4<F8>(f2_pack(x[0].h, x[1].h), f2_pack(x[0].l, x[1].l), f2_pack(x[2].h, x[3].h),
+           f2_pack(x[2].l, x[3].l), st, out, plane);
 }
 
 // 2^e as two normal powers of two (e clamped to [-252, 254])
@@ -402,6 +418,7 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
   const int v = F.v, o = F.o, vpad = F.vpad;
   const int i = (int)((gp - F.pair_begin) / o), j = (int)((gp - F.pair_begin) % o);
   const bool tr = i > j;                  // the stored block is (j, i)
+  if (tr && F.st_out == 0) return;        // energies only: (j, i) has this pair's
   const int i0 = tr ? j : i, j0 = tr ? i : j;
   const long long ldd = F.ldd, ldt = F.ldt;
   st = F.st_out;              // Tt digit planes (0: energy only)
@@ -428,7 +445,8 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
   const long long colJ = (long long)j * vpad;                            // output columns
   const long long rowS = (long long)i0 * v, colS = (long long)j0 * F.vpadt; // stored T block
   const int nt = (v + 31) / 32;
-  dfl e_acc = {0.f, 0.f}, e_os = {0.f, 0.f};   // pair energy and its opposite-spin part
+  // pair energy and its opposite-spin part, two running sums each (even and odd columns)
+  f2x e_h = 0ull, e_l = 0ull, o_h = 0ull, o_l = 0ull;
 
   float4 xh, xl, yh, yl;
   auto load = [&](int ta, int tb) {
@@ -448,42 +466,59 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
     }
   };
 
+  const f2x k2 = f2_two(2.f);
   // one output tile row segment: t_k and its transposed partner y_k for the four columns
-  // col0 + k (local column index lc0 + k of the output block), written at global row orow
-  auto emit = [&](const dfl t_in[4], const dfl y_in[4], long long orow, long long ocol0, int lc0,
-                  bool energy, long long drow_r, long long drow_c0) {
-    dfl t[4], tt[4];
-    float2 dm = make_float2(0.f, 0.f), dn[4];
-    if (energy) {   // the D terms of the row and the four columns, issued together
-      dm = dr[drow_r];
+  // col0 + k (local column index lc0 + k of the output block), written at global row orow;
+  // all arithmetic on element pairs (columns past nvir are zeroed first: t = Tt = 0 there)
+  auto emit = [&](dfl (&t_in)[4], dfl (&y_in)[4], long long orow, long long ocol0, int lc0,
+                  long long drow_r, long long drow_c0) {
+    if (lc0 + 4 > v) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) dn[k] = lc0 + k < v ? dr[drow_c0 + k] : make_float2(0.f, 0.f);
+      for (int k = 0; k < 4; ++k)
+        if (lc0 + k >= v) t_in[k] = y_in[k] = dfl{0.f, 0.f};
     }
+    f2x th[2], tl[2], uh[2], ul[2];   // T and Tt
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const bool ok = lc0 + k < v;
-      t[k] = ok ? t_in[k] : dfl{0.f, 0.f};
-      tt[k] = ok ? d_add({2.f * t_in[k].h, 2.f * t_in[k].l}, d_neg(y_in[k])) : dfl{0.f, 0.f};
-      if (energy && ok) {
-        const dfl D = d_add({dm.x, dm.y}, {dn[k].x, dn[k].y});
-        const dfl V = d_mul(t[k], D);
-        e_acc = d_add(e_acc, d_mul(tt[k], V));
-        e_os = d_add(e_os, d_mul(t[k], V));
+    for (int g = 0; g < 2; ++g) {
+      th[g] = f2_pack(t_in[2 * g].h, t_in[2 * g + 1].h);
+      tl[g] = f2_pack(t_in[2 * g].l, t_in[2 * g + 1].l);
+      const f2x yh2 = f2_pack(y_in[2 * g].h, y_in[2 * g + 1].h);
+      const f2x yl2 = f2_pack(y_in[2 * g].l, y_in[2 * g + 1].l);
+      d_add2(f2_mul(th[g], k2), f2_mul(tl[g], k2), f2_neg(yh2), f2_neg(yl2), uh[g], ul[g]);
+    }
+    if (!tr) {   // pair energy: D terms of the row and the four columns
+      const float2 dm = dr[drow_r];
+      const f2x dmh = f2_two(dm.x), dml = f2_two(dm.y);
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        const float2 z = make_float2(0.f, 0.f);
+        const float2 n0 = lc0 + 2 * g < v ? dr[drow_c0 + 2 * g] : z;
+        const float2 n1 = lc0 + 2 * g + 1 < v ? dr[drow_c0 + 2 * g + 1] : z;
+        f2x Dh, Dl, Vh, Vl, ph, pl;
+        d_add2(dmh, dml, f2_pack(n0.x, n1.x), f2_pack(n0.y, n1.y), Dh, Dl);
+        d_mul2(th[g], tl[g], Dh, Dl, Vh, Vl);
+        d_mul2(uh[g], ul[g], Vh, Vl, ph, pl);
+        d_add2(e_h, e_l, ph, pl, e_h, e_l);
+        d_mul2(th[g], tl[g], Vh, Vl, ph, pl);
+        d_add2(o_h, o_l, ph, pl, o_h, o_l);
       }
     }
     if (st == 0) return;
     const long long o_ = orow * ldd + ocol0;
+    const f2x a1 = f2_two(s1t), a2 = f2_two(s2t), b1 = f2_two(s1tt), b2 = f2_two(s2tt);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      t[k] = {(t[k].h * s1t) * s2t, (t[k].l * s1t) * s2t};
-      tt[k] = {(tt[k].h * s1tt) * s2tt, (tt[k].l * s1tt) * s2tt};
+    for (int g = 0; g < 2; ++g) {
+      th[g] = f2_mul(f2_mul(th[g], a1), a2);
+      tl[g] = f2_mul(f2_mul(tl[g], a1), a2);
+      uh[g] = f2_mul(f2_mul(uh[g], b1), b2);
+      ul[g] = f2_mul(f2_mul(ul[g], b1), b2);
     }
     if (ns) {
-      put4<F8, NS, true>(t, stt, ts + o_, plane);
-      put4<F8, NS, true>(tt, st, tts + o_, plane);
+      put4<F8, NS, true>(th[0], tl[0], th[1], tl[1], stt, ts + o_, plane);
+      put4<F8, NS, true>(uh[0], ul[0], uh[1], ul[1], st, tts + o_, plane);
     } else {
-      put4<F8, 0, true>(t, stt, ts + o_, plane);
-      put4<F8, 0, true>(tt, st, tts + o_, plane);
+      put4<F8, 0, true>(th[0], tl[0], th[1], tl[1], stt, ts + o_, plane);
+      put4<F8, 0, true>(uh[0], ul[0], uh[1], ul[1], st, tts + o_, plane);
     }
   };
 
@@ -512,7 +547,7 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
           t4[k] = tr ? y : x;
           y4[k] = tr ? x : y;
         }
-        emit(t4, y4, rowI + la, colJ + lb, lb, !tr, rowI + la, rowJ + lb);
+        emit(t4, y4, rowI + la, colJ + lb, lb, rowI + la, rowJ + lb);
       }
     }
     if (cta != ctb) {   // output tile (ctb, cta): Y[r][c] (stored (i,j)) or X[c][r]
@@ -524,7 +559,7 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
           t4[k] = tr ? y : x;
           y4[k] = tr ? x : y;
         }
-        emit(t4, y4, rowI + la, colJ + lb, lb, !tr, rowI + la, rowJ + lb);
+        emit(t4, y4, rowI + la, colJ + lb, lb, rowI + la, rowJ + lb);
       }
     }
   }
@@ -544,7 +579,16 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
       ((U4*)row)[c] = make_uint4(0u, 0u, 0u, 0u);
     }
   }
-  // pair energy: warp, then block, in double-float; one FP64 value per pair
+  if (tr) return;
+  // pair energy: the two running sums, then warp and block, in double-float; one FP64 value
+  // per pair
+  auto join = [](f2x h, f2x l) {
+    float h0, h1, l0, l1;
+    f2_unpack(h, h0, h1);
+    f2_unpack(l, l0, l1);
+    return d_add({h0, l0}, {h1, l1});
+  };
+  dfl e_acc = join(e_h, e_l), e_os = join(o_h, o_l);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     const dfl o2 = {__shfl_down_sync(0xffffffffu, e_acc.h, off),
@@ -559,7 +603,7 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
     ros_h[tid >> 5] = e_os.h; ros_l[tid >> 5] = e_os.l;
   }
   __syncthreads();
-  if (tid == 0 && !tr) {
+  if (tid == 0) {
     double e = 0.0, eos = 0.0;
     for (int w = 0; w < 8; ++w) {
       e += (double)red_h[w] + (double)red_l[w];
