@@ -167,22 +167,33 @@ __device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c) {
 
 __device__ __forceinline__ f2x f2_neg(f2x a) { return a ^ 0x8000000080000000ull; }
 __device__ __forceinline__ f2x f2_two(float a) { return f2_pack(a, a); }
-// Double-float sum and product on two lanes (the f32x2 forms round each lane like the scalar
-// instruction and are never contracted)
-__device__ __forceinline__ void d_add2(f2x ah, f2x al, f2x bh, f2x bl, f2x& h, f2x& l) {
-  const f2x s = f2_add(ah, bh);
-  const f2x bb = f2_sub(s, ah);
-  const f2x e = f2_add(f2_sub(ah, f2_sub(s, bb)), f2_sub(bh, bb));
-  const f2x t = f2_add(e, f2_add(al, bl));
+// Double-float arithmetic on two lanes (the f32x2 forms round each lane like the scalar
+// instruction and are never contracted).  s + e = a + b exactly:
+__device__ __forceinline__ void f2_two_sum(f2x a, f2x b, f2x& s, f2x& e) {
+  s = f2_add(a, b);
+  const f2x bb = f2_sub(s, a);
+  e = f2_add(f2_sub(a, f2_sub(s, bb)), f2_sub(b, bb));
+}
+// a - b, normalised
+__device__ __forceinline__ void d_sub2(f2x ah, f2x al, f2x bh, f2x bl, f2x& h, f2x& l) {
+  const f2x s = f2_sub(ah, bh);
+  const f2x bb = f2_sub(ah, s);                                     // b as seen in s
+  const f2x e = f2_add(f2_sub(bb, bh), f2_sub(ah, f2_add(s, bb)));   // two-difference
+  const f2x t = f2_add(e, f2_sub(al, bl));
   h = f2_add(s, t);
   l = f2_sub(t, f2_sub(h, s));
 }
-__device__ __forceinline__ void d_mul2(f2x ah, f2x al, f2x bh, f2x bl, f2x& h, f2x& l) {
-  const f2x p = f2_mul(ah, bh);
-  f2x e = f2_fma(ah, bh, f2_neg(p));
-  e = f2_fma(ah, bl, f2_fma(al, bh, e));
-  h = f2_add(p, e);
-  l = f2_sub(e, f2_sub(h, p));
+// a b as h + l with |l| of the order of an ulp of h (not normalised); na = -ah
+__device__ __forceinline__ void d_mul2(f2x ah, f2x na, f2x al, f2x bh, f2x bl, f2x& h, f2x& l) {
+  h = f2_mul(ah, bh);
+  const f2x ne = f2_fma(na, bh, h);                                 // h - ah bh, exact
+  l = f2_sub(f2_fma(ah, bl, f2_mul(al, bh)), ne);
+}
+// sum (sh, sl) += (h, l): sh takes h without error, sl collects the errors and the low parts
+__device__ __forceinline__ void d_acc2(f2x& sh, f2x& sl, f2x h, f2x l) {
+  f2x e;
+  f2_two_sum(sh, h, sh, e);
+  sl = f2_add(sl, f2_add(e, l));
 }
 
 // digit_step on two elements at once, with the scaling by 2^LB folded into the Fast2Sum
@@ -248,6 +259,7 @@ __global__ void k_split_reset(const SplitFragDev* __restrict__ f, int n, Bases b
   const SplitFragDev& F = f[blockIdx.x];
   char* ws = (char*)bs.ws;
   if (threadIdx.x == 0) ((unsigned*)(ws + F.scal))[1] = 0u;
+  for (int i = threadIdx.x; i < F.o; i += blockDim.x) ((unsigned*)(ws + F.ecnt))[i] = 0u;
   if (F.sg_out > 0) {
     unsigned long long* cm = (unsigned long long*)(ws + F.ecolm);
     for (int q = threadIdx.x; q < F.X; q += blockDim.x) cm[q] = 0ull;
@@ -304,6 +316,13 @@ k_slice_b1(const SplitFragDev* __restrict__ f, int nf, long long rows, int sv, B
     const int i = r / F.v, a = r - i * F.v;
     const dfl d = d_from(bs.eps[F.eo_off + i] - bs.eps[F.ev_off + a]);
     ((float2*)(ws + F.drow))[r] = make_float2(d.h, d.l);
+    // the same terms by padded j blocks for the amplitude kernel's 16-byte loads
+    float* dnh = (float*)(ws + F.dnh) + (long long)i * F.vpadt;
+    float* dnl = (float*)(ws + F.dnl) + (long long)i * F.vpadt;
+    dnh[a] = d.h;
+    dnl[a] = d.l;
+    if (a == F.v - 1)
+      for (int k = F.v; k < F.vpadt; ++k) dnh[k] = dnl[k] = 0.f;
     const dfl vd = d_from(ss);
     ((float2*)(ws + F.vdrow))[r] = make_float2(vd.h, vd.l);
   }
@@ -391,230 +410,235 @@ k_slice_b2(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
   }
 }
 
-// One CTA per ordered pair (i, j), i-major, so that the CTAs in flight fill the same rows
-// of the digit planes.  The CTA writes the (i,j) block only; it reads the stored block
+// Amplitude stage: Tt = 2T - T^T, digits of T and Tt (one scale per fragment each), pair
+// energies e_ij = sum_ab Tt_ij(a,b) V_ij(a,b) (V = T D) and their opposite-spin part
+// sum_ab T_ij(a,b) V_ij(a,b) for i <= j.
+//
+// A CTA takes a strip of ROWS rows (i, a0 ..) and a range of j; per step it forms C = 4 LPR
+// columns of one j block, a group of LPR lanes per row, four columns a lane.  The stored block
 // (min(i,j), max(i,j)) of the double-float T planes (rows (i,a), columns j*vpadt + b;
-// T_ij(a,b) = T_ji(b,a)) in pairs of 32 x 32 tiles (ta <= tb): X = tile (ta, tb) and
-// Y = tile (tb, ta), 16-byte loads prefetched into registers while the previous pair is
-// processed.  Every thread forms, for one row and four consecutive columns of the output
-// tiles (ta, tb) and (tb, ta), Tt = 2T - T^T and the digits of T and Tt (one scale per
-// fragment each; one packed store per slice; columns in [nvir, vpad) get zero digits).
-// CTAs with i <= j also accumulate
-// the pair energy e_ij = sum_ab Tt_ij(a,b) V_ij(a,b) (V = T D) and its opposite-spin
-// part sum_ab T_ij(a,b) V_ij(a,b) in double-float (D from the double-float row terms
-// d_m = e_i - e_a).
-template <bool F8>
+// T_ij(a,b) = T_ji(b,a)) gives both operands: a direct tile (rows a, columns b) the lanes read
+// for themselves, and a transposed tile (rows b, columns a) that goes through shared memory.
+// For i <= j the direct tile is T and the other its partner T_ij(b,a), for i > j the reverse.
+//
+// The write pattern bounds this kernel: 24 (BF16) or 20 (FP8) bytes an element in 12 or 20
+// planes.  HBM and L2 take full rate only when a warp's store covers whole 128-byte lines of a
+// row, and neighbouring lines follow soon: as pairs of 32 x 32 tiles (64 or 32 bytes a row and
+// store) the same bytes moved at 3.1 TB/s (BF16) and 1.3 TB/s (FP8), in these strips at 6.2
+// and 4.8 (copies of both patterns without the arithmetic, nocc=40 nvir=400), although the
+// strips read T twice.
+// LPR: lanes per row, 32, or fewer where the rows are short (amp_lanes).
+template <bool F8, int LPR>
 __global__ void __launch_bounds__(256, 3)
-k_amp_split(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
+k_amp_split(const SplitFragDev* __restrict__ f, int nf, Bases bs) {
   using DT = typename Digit<F8>::T;
   constexpr int LB = Digit<F8>::LB;
-  // hi and lo parts of the tile pair in separate planes: with rows of 33 floats both the
-  // row-wise and the transposed reads of a warp (4 rows x 8 column groups) hit 32 banks
-  __shared__ float Xh[32][33], Xl[32][33], Yh[32][33], Yl[32][33];
-  __shared__ float red_h[8], red_l[8], ros_h[8], ros_l[8];
-  const int tid = threadIdx.x, r = tid >> 3, c0 = (tid & 7) * 4;
-  const long long gp = blockIdx.x;
-  const SplitFragDev& F = f[find_sfd(f, nf, gp, 2)];
-  const int v = F.v, o = F.o, vpad = F.vpad;
-  const int i = (int)((gp - F.pair_begin) / o), j = (int)((gp - F.pair_begin) % o);
-  const bool tr = i > j;                  // the stored block is (j, i)
-  if (tr && F.st_out == 0) return;        // energies only: (j, i) has this pair's
-  const int i0 = tr ? j : i, j0 = tr ? i : j;
-  const long long ldd = F.ldd, ldt = F.ldt;
-  st = F.st_out;              // Tt digit planes (0: energy only)
-  const int stt = F.st_t;     // T digit planes (0: no P)
-  // BF16: the usual plane count (6) unrolled; FP8's ten planes stay a loop (unrolled,
-  // they cost more registers than the loop saves: 33.4 against 32.3 ms at nocc=100 nvir=500 naux=1500)
+  constexpr int GROUPS = 32 / LPR, ROWS = 8 * GROUPS, C = 4 * LPR;
+  constexpr int LDY = C + 4;   // 16-byte rows; the transposing writes of a warp then hit all banks
+  __shared__ __align__(16) float Yh[2][ROWS * LDY], Yl[2][ROWS * LDY];
+  __shared__ int s_last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const SplitFragDev& F = f[find_sfd(f, nf, blockIdx.x, 2)];
+  const int v = F.v, o = F.o, vpad = F.vpad, vpadt = F.vpadt;
+  const int strips = max(1, (v + ROWS - 1) / ROWS);
+  // CTA -> (i, j range, strip): neighbouring CTAs take neighbouring strips of the same i
+  int q = (int)(blockIdx.x - F.pair_begin);
+  const int strip = q % strips;
+  q /= strips;
+  const int jranges = (o + F.amp_jchunk - 1) / F.amp_jchunk;
+  const int i = q / jranges;
+  const int st = F.st_out, stt = F.st_t;   // digit planes of Tt (0: energies only) and T (0: no P)
+  const int jb0 = (q % jranges) * F.amp_jchunk, je = min(o, jb0 + F.amp_jchunk);
+  const int jb = st == 0 ? max(jb0, i) : jb0;   // energies only: the pairs i <= j
+  // BF16: the usual plane count (6) unrolled; FP8's ten planes stay a loop (unrolled, they
+  // cost more registers than the loop saves)
   constexpr int NS = F8 ? 0 : 6;
   const bool ns = NS > 0 && st == NS && stt == NS;
   char* ws = (char*)bs.ws;
   const float* Th = (const float*)(ws + F.thi);
   const float* Tl = (const float*)(ws + F.tlo);
-  const float2* __restrict__ dr = (const float2*)(ws + F.drow);
+  const float* __restrict__ Dh = (const float*)(ws + F.dnh);   // e_j - e_b at j*vpadt + b
+  const float* __restrict__ Dl = (const float*)(ws + F.dnl);
   const unsigned emax = *(const unsigned*)(ws + F.scal + 4);
-  float s1t, s2t, s1tt, s2tt;   // 2^(LB - E) as two normal factors, for T and Tt
-  // |T| < 2^(emax - 126) and |Tt| <= 3 max |T| < 2^(emax - 124): the scales keep both
-  // within 2^(E - 2 - HEAD) and 2^(E - 1 - HEAD)
-  constexpr int HEAD = Digit<F8>::HEAD;
-  pow2_factors(LB - ((int)emax - 124 + HEAD), s1t, s2t);
-  pow2_factors(LB - ((int)emax - 123 + HEAD), s1tt, s2tt);
+  // |T| < 2^(emax - 126) and |Tt| <= 3 max |T| < 2^(emax - 124): the scales 2^kt of T and
+  // 2^(kt - 1) of Tt keep both within 2^(E - 2 - HEAD) and 2^(E - 1 - HEAD).  T_ij(b,a) is
+  // scaled by the latter, so that Tt = 2T - T^T is a plain difference of scaled values, and the
+  // energies are formed from the scaled T and Tt (all exact powers of two).
+  const int kt = LB - ((int)emax - 124 + Digit<F8>::HEAD);
+  const bool one = kt <= 126 && kt >= -125;   // 2^kt is a normal float (unless |T| < 2^-121)
+  float sa, sb;
+  pow2_factors(kt, sa, sb);
+  if (one) { sa = __int_as_float((kt + 127) << 23); sb = 1.f; }
+  const f2x sc_t = f2_two(sa), sc_y = f2_two(0.5f * sa), sc_2 = f2_two(sb);
   DT* tts = (DT*)(ws + F.tts);
   DT* ts = (DT*)(ws + F.ts);
-  const long long plane = (long long)o * v * ldd;
-  const long long rowI = (long long)i * v, rowJ = (long long)j * v;      // output rows, D terms
-  const long long colJ = (long long)j * vpad;                            // output columns
-  const long long rowS = (long long)i0 * v, colS = (long long)j0 * F.vpadt; // stored T block
-  const int nt = (v + 31) / 32;
-  // pair energy and its opposite-spin part, two running sums each (even and odd columns)
-  f2x e_h = 0ull, e_l = 0ull, o_h = 0ull, o_l = 0ull;
+  const long long ldd = F.ldd, ldt = F.ldt, plane = (long long)o * v * ldd;
+  const int nb = (vpad + C - 1) / C, steps = max(0, je - jb) * nb;
+  const int a0 = strip * ROWS;
+  // this lane's row and columns of the direct tile, and its float4 of the transposed one
+  const int row = warp * GROUPS + lane / LPR, a = a0 + row, c0 = 4 * (lane % LPR);
+  const int yq = 4 * (tid % (ROWS / 4)), yb = tid / (ROWS / 4);
 
-  float4 xh, xl, yh, yl;
-  auto load = [&](int ta, int tb) {
-    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-    xh = xl = yh = yl = z;
-    const int ax = ta * 32 + r, bx = tb * 32 + c0;
-    if (ax < v && bx < F.vpadt) {
-      const long long ix = (rowS + ax) * ldt + colS + bx;
+  // the next step's direct and transposed elements; their offsets advance within a j block
+  float4 dh, dl, xh, xl;
+  long long id = 0, ix = 0;
+  const long long xstep = (long long)C * ldt;
+  auto load = [&](int j, int b0) {
+    if (b0 == 0) {
+      const long long rows = (long long)min(i, j) * v, cols = (long long)max(i, j) * vpadt;
+      id = (rows + a) * ldt + cols + c0;
+      ix = (rows + yb) * ldt + cols + a0 + yq;
+    }
+    dh = dl = xh = xl = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (a < v && b0 + c0 < vpadt) {
+      dh = __ldg((const float4*)(Th + id));
+      dl = __ldg((const float4*)(Tl + id));
+    }
+    if (b0 + yb < v && a0 + yq < vpadt) {
       xh = __ldg((const float4*)(Th + ix));
       xl = __ldg((const float4*)(Tl + ix));
     }
-    const int ay = tb * 32 + r, by = ta * 32 + c0;
-    if (ay < v && by < F.vpadt) {
-      const long long iy = (rowS + ay) * ldt + colS + by;
-      yh = __ldg((const float4*)(Th + iy));
-      yl = __ldg((const float4*)(Tl + iy));
-    }
+    id += C;
+    ix += xstep;
   };
 
-  const f2x k2 = f2_two(2.f);
-  // one output tile row segment: t_k and its transposed partner y_k for the four columns
-  // col0 + k (local column index lc0 + k of the output block), written at global row orow;
-  // all arithmetic on element pairs (columns past nvir are zeroed first: t = Tt = 0 there)
-  auto emit = [&](dfl (&t_in)[4], dfl (&y_in)[4], long long orow, long long ocol0, int lc0,
-                  long long drow_r, long long drow_c0) {
-    if (lc0 + 4 > v) {
+  // pair energy and its opposite-spin part, two running sums each (even and odd columns)
+  f2x e_h = 0ull, e_l = 0ull, o_h = 0ull, o_l = 0ull;
+  const float dmh1 = a < v ? Dh[(long long)i * vpadt + a] : 0.f, dml1 = a < v ? Dl[(long long)i * vpadt + a] : 0.f;
+  const f2x dmh = f2_two(dmh1), dml = f2_two(dml1);
+  int j = jb, b0 = 0;
+  if (steps > 0) load(j, 0);
+  for (int s = 0; s < steps; ++s) {
+    float* const Sh = Yh[s & 1];
+    float* const Sl = Yl[s & 1];
+    Sh[(yq + 0) * LDY + yb] = xh.x; Sh[(yq + 1) * LDY + yb] = xh.y;
+    Sh[(yq + 2) * LDY + yb] = xh.z; Sh[(yq + 3) * LDY + yb] = xh.w;
+    Sl[(yq + 0) * LDY + yb] = xl.x; Sl[(yq + 1) * LDY + yb] = xl.y;
+    Sl[(yq + 2) * LDY + yb] = xl.z; Sl[(yq + 3) * LDY + yb] = xl.w;
+    f2x th[2] = {f2_pack(dh.x, dh.y), f2_pack(dh.z, dh.w)};
+    f2x tl[2] = {f2_pack(dl.x, dl.y), f2_pack(dl.z, dl.w)};
+    __syncthreads();   // the other buffer's readers are past it: two buffers, one barrier a step
+    const int cj = j, b = b0 + c0;
+    b0 += C;
+    if (b0 >= vpad) { b0 = 0; ++j; }
+    if (s + 1 < steps) load(j, b0);   // in flight while this step is processed
+    if (a < v && b < vpad) {
+      const float4 ph = *(const float4*)(Sh + row * LDY + c0), pl = *(const float4*)(Sl + row * LDY + c0);
+      f2x yh[2] = {f2_pack(ph.x, ph.y), f2_pack(ph.z, ph.w)};
+      f2x yl[2] = {f2_pack(pl.x, pl.y), f2_pack(pl.z, pl.w)};
+      if (i > cj) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (lc0 + k >= v) t_in[k] = y_in[k] = dfl{0.f, 0.f};
-    }
-    f2x th[2], tl[2], uh[2], ul[2];   // T and Tt
+        for (int g = 0; g < 2; ++g) {
+          f2x t = th[g]; th[g] = yh[g]; yh[g] = t;
+          t = tl[g]; tl[g] = yl[g]; yl[g] = t;
+        }
+      }
+      if (b + 4 > v) {   // columns in [nvir, vpad) get zero digits
 #pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      th[g] = f2_pack(t_in[2 * g].h, t_in[2 * g + 1].h);
-      tl[g] = f2_pack(t_in[2 * g].l, t_in[2 * g + 1].l);
-      const f2x yh2 = f2_pack(y_in[2 * g].h, y_in[2 * g + 1].h);
-      const f2x yl2 = f2_pack(y_in[2 * g].l, y_in[2 * g + 1].l);
-      d_add2(f2_mul(th[g], k2), f2_mul(tl[g], k2), f2_neg(yh2), f2_neg(yl2), uh[g], ul[g]);
-    }
-    if (!tr) {   // pair energy: D terms of the row and the four columns
-      const float2 dm = dr[drow_r];
-      const f2x dmh = f2_two(dm.x), dml = f2_two(dm.y);
+        for (int g = 0; g < 2; ++g) {
+          const f2x m = (b + 2 * g < v ? 0xffffffffull : 0ull) |
+                        (b + 2 * g + 1 < v ? 0xffffffff00000000ull : 0ull);
+          th[g] &= m; tl[g] &= m; yh[g] &= m; yl[g] &= m;
+        }
+      }
+      f2x uh[2], ul[2];   // Tt
 #pragma unroll
       for (int g = 0; g < 2; ++g) {
-        const float2 z = make_float2(0.f, 0.f);
-        const float2 n0 = lc0 + 2 * g < v ? dr[drow_c0 + 2 * g] : z;
-        const float2 n1 = lc0 + 2 * g + 1 < v ? dr[drow_c0 + 2 * g + 1] : z;
-        f2x Dh, Dl, Vh, Vl, ph, pl;
-        d_add2(dmh, dml, f2_pack(n0.x, n1.x), f2_pack(n0.y, n1.y), Dh, Dl);
-        d_mul2(th[g], tl[g], Dh, Dl, Vh, Vl);
-        d_mul2(uh[g], ul[g], Vh, Vl, ph, pl);
-        d_add2(e_h, e_l, ph, pl, e_h, e_l);
-        d_mul2(th[g], tl[g], Vh, Vl, ph, pl);
-        d_add2(o_h, o_l, ph, pl, o_h, o_l);
-      }
-    }
-    if (st == 0) return;
-    const long long o_ = orow * ldd + ocol0;
-    const f2x a1 = f2_two(s1t), a2 = f2_two(s2t), b1 = f2_two(s1tt), b2 = f2_two(s2tt);
-#pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      th[g] = f2_mul(f2_mul(th[g], a1), a2);
-      tl[g] = f2_mul(f2_mul(tl[g], a1), a2);
-      uh[g] = f2_mul(f2_mul(uh[g], b1), b2);
-      ul[g] = f2_mul(f2_mul(ul[g], b1), b2);
-    }
-    if (ns) {
-      put4<F8, NS, true>(th[0], tl[0], th[1], tl[1], stt, ts + o_, plane);
-      put4<F8, NS, true>(uh[0], ul[0], uh[1], ul[1], st, tts + o_, plane);
-    } else {
-      put4<F8, 0, true>(th[0], tl[0], th[1], tl[1], stt, ts + o_, plane);
-      put4<F8, 0, true>(uh[0], ul[0], uh[1], ul[1], st, tts + o_, plane);
-    }
-  };
-
-  int ta = 0, tb = 0;
-  if (nt > 0) load(0, 0);
-  while (ta < nt) {
-    __syncthreads();   // the previous pair is no longer read from shared memory
-    Xh[r][c0 + 0] = xh.x; Xh[r][c0 + 1] = xh.y; Xh[r][c0 + 2] = xh.z; Xh[r][c0 + 3] = xh.w;
-    Xl[r][c0 + 0] = xl.x; Xl[r][c0 + 1] = xl.y; Xl[r][c0 + 2] = xl.z; Xl[r][c0 + 3] = xl.w;
-    Yh[r][c0 + 0] = yh.x; Yh[r][c0 + 1] = yh.y; Yh[r][c0 + 2] = yh.z; Yh[r][c0 + 3] = yh.w;
-    Yl[r][c0 + 0] = yl.x; Yl[r][c0 + 1] = yl.y; Yl[r][c0 + 2] = yl.z; Yl[r][c0 + 3] = yl.w;
-    __syncthreads();
-    const int cta = ta, ctb = tb;
-    if (++tb == nt) { ++ta; tb = ta; }
-    if (ta < nt) load(ta, tb);   // next pair in flight while this one is processed
-
-    dfl t4[4], y4[4];
-    // output tile (cta, ctb): T_ij(a,b) = X[r][c] (stored (i,j)) or Y[c][r] (stored (j,i));
-    // the partner T_ij(b,a) is the other one of the two
-    {
-      const int la = cta * 32 + r, lb = ctb * 32 + c0;
-      if (la < v && lb < vpad) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const dfl x = {Xh[r][c0 + k], Xl[r][c0 + k]}, y = {Yh[c0 + k][r], Yl[c0 + k][r]};
-          t4[k] = tr ? y : x;
-          y4[k] = tr ? x : y;
+        th[g] = f2_mul(th[g], sc_t);
+        tl[g] = f2_mul(tl[g], sc_t);
+        yh[g] = f2_mul(yh[g], sc_y);
+        yl[g] = f2_mul(yl[g], sc_y);
+        if (!one) {
+          th[g] = f2_mul(th[g], sc_2);
+          tl[g] = f2_mul(tl[g], sc_2);
+          yh[g] = f2_mul(yh[g], sc_2);
+          yl[g] = f2_mul(yl[g], sc_2);
         }
-        emit(t4, y4, rowI + la, colJ + lb, lb, rowI + la, rowJ + lb);
+        d_sub2(th[g], tl[g], yh[g], yl[g], uh[g], ul[g]);
       }
-    }
-    if (cta != ctb) {   // output tile (ctb, cta): Y[r][c] (stored (i,j)) or X[c][r]
-      const int la = ctb * 32 + r, lb = cta * 32 + c0;
-      if (la < v && lb < vpad) {
+      if (i <= cj && b < v) {
+        const float4 nh = __ldg((const float4*)(Dh + (long long)cj * vpadt + b));
+        const float4 nl = __ldg((const float4*)(Dl + (long long)cj * vpadt + b));
+        const f2x dnh[2] = {f2_pack(nh.x, nh.y), f2_pack(nh.z, nh.w)};
+        const f2x dnl[2] = {f2_pack(nl.x, nl.y), f2_pack(nl.z, nl.w)};
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const dfl x = {Yh[r][c0 + k], Yl[r][c0 + k]}, y = {Xh[c0 + k][r], Xl[c0 + k][r]};
-          t4[k] = tr ? y : x;
-          y4[k] = tr ? x : y;
+        for (int g = 0; g < 2; ++g) {
+          const f2x nt = f2_neg(th[g]);
+          f2x dh2, dl2, vh, vl, qh, ql;
+          f2_two_sum(dmh, dnh[g], dh2, dl2);
+          dl2 = f2_add(dl2, f2_add(dml, dnl[g]));
+          d_mul2(th[g], nt, tl[g], dh2, dl2, vh, vl);
+          d_mul2(uh[g], f2_neg(uh[g]), ul[g], vh, vl, qh, ql);
+          d_acc2(e_h, e_l, qh, ql);
+          d_mul2(th[g], nt, tl[g], vh, vl, qh, ql);
+          d_acc2(o_h, o_l, qh, ql);
         }
-        emit(t4, y4, rowI + la, colJ + lb, lb, rowI + la, rowJ + lb);
+      }
+      if (st > 0) {
+        const long long out = ((long long)i * v + a) * ldd + (long long)cj * vpad + b;
+        if (ns) {
+          put4<F8, NS, true>(th[0], tl[0], th[1], tl[1], stt, ts + out, plane);
+          put4<F8, NS, true>(uh[0], ul[0], uh[1], ul[1], st, tts + out, plane);
+        } else {
+          put4<F8, 0, true>(th[0], tl[0], th[1], tl[1], stt, ts + out, plane);
+          put4<F8, 0, true>(uh[0], ul[0], uh[1], ul[1], st, tts + out, plane);
+        }
       }
     }
-  }
-  // digit columns [32 nt, vpad) that no tile reaches (the padded row segment is longer
-  // than the tiles, e.g. nvir = 1500 with 1536-element segments): zero in every row
-  if (st > 0 && vpad > nt * 32) {
-    using U4 = uint4;
-    const int w16 = (vpad - nt * 32) * (int)sizeof(DT) / 16;   // 16-byte units per row
-    const long long units = (long long)(st + stt) * v * w16;
-    for (long long u = tid; u < units; u += blockDim.x) {
-      long long x = u;
-      const int c = (int)(x % w16); x /= w16;
-      const int a = (int)(x % v);
-      const int p = (int)(x / v);
-      DT* base = p < stt ? ts + p * plane : tts + (p - stt) * plane;
-      DT* row = base + (rowI + a) * ldd + colJ + nt * 32;
-      ((U4*)row)[c] = make_uint4(0u, 0u, 0u, 0u);
+    if (i <= cj && b0 == 0) {   // the block (i, cj) is done: this warp's share of its energy
+      auto join = [](f2x h, f2x l) {
+        float h0, h1, l0, l1;
+        f2_unpack(h, h0, h1);
+        f2_unpack(l, l0, l1);
+        return d_add({h0, l0}, {h1, l1});
+      };
+      // lanes 0..15 go on with the energy, 16..31 with its opposite-spin part
+      const dfl e = join(e_h, e_l), eo = join(o_h, o_l);
+      const bool up = lane >= 16;
+      const dfl give = up ? e : eo, keep = up ? eo : e;
+      dfl w = d_add(keep, {__shfl_xor_sync(0xffffffffu, give.h, 16), __shfl_xor_sync(0xffffffffu, give.l, 16)});
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1)
+        w = d_add(w, {__shfl_xor_sync(0xffffffffu, w.h, off), __shfl_xor_sync(0xffffffffu, w.l, off)});
+      if ((lane & 15) == 0)
+        ((float2*)(ws + F.epart))[2 * (((long long)i * o + cj) * (strips * 8) + strip * 8 + warp) + up] =
+            make_float2(w.h, w.l);
+      e_h = e_l = o_h = o_l = 0ull;
     }
   }
-  if (tr) return;
-  // pair energy: the two running sums, then warp and block, in double-float; one FP64 value
-  // per pair
-  auto join = [](f2x h, f2x l) {
-    float h0, h1, l0, l1;
-    f2_unpack(h, h0, h1);
-    f2_unpack(l, l0, l1);
-    return d_add({h0, l0}, {h1, l1});
-  };
-  dfl e_acc = join(e_h, e_l), e_os = join(o_h, o_l);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const dfl o2 = {__shfl_down_sync(0xffffffffu, e_acc.h, off),
-                    __shfl_down_sync(0xffffffffu, e_acc.l, off)};
-    e_acc = d_add(e_acc, o2);
-    const dfl o3 = {__shfl_down_sync(0xffffffffu, e_os.h, off),
-                    __shfl_down_sync(0xffffffffu, e_os.l, off)};
-    e_os = d_add(e_os, o3);
-  }
-  if ((tid & 31) == 0) {
-    red_h[tid >> 5] = e_acc.h; red_l[tid >> 5] = e_acc.l;
-    ros_h[tid >> 5] = e_os.h; ros_l[tid >> 5] = e_os.l;
-  }
+  // the last CTA of row i sums the warps' shares of e_ij, j >= i, in a fixed order (FP64)
+  __threadfence();
   __syncthreads();
-  if (tid == 0) {
-    double e = 0.0, eos = 0.0;
-    for (int w = 0; w < 8; ++w) {
-      e += (double)red_h[w] + (double)red_l[w];
-      eos += (double)ros_h[w] + (double)ros_l[w];
+  if (tid == 0)
+    s_last = atomicAdd((unsigned*)(ws + F.ecnt) + i, 1u) + 1u == (unsigned)(strips * jranges);
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double* ep = (double*)(ws + F.ep);
+  const int parts = v > 0 ? strips * 8 : 0;
+  for (int jj = i + warp; jj < o; jj += 8) {
+    const float4* p = (const float4*)(ws + F.epart) + ((long long)i * o + jj) * (strips * 8);
+    double e = 0.0, eo = 0.0;
+#pragma unroll 4
+    for (int k = lane; k < parts; k += 32) {
+      const float4 w = __ldcg(p + k);
+      e += (double)w.x + (double)w.y;
+      eo += (double)w.z + (double)w.w;
     }
-    double* ep = (double*)(ws + F.ep);
-    ep[(long long)i * o + j] = e;
-    ep[(long long)j * o + i] = e;
-    ep += (long long)o * o;          // opposite-spin pair energies
-    ep[(long long)i * o + j] = eos;
-    ep[(long long)j * o + i] = eos;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      e += __shfl_xor_sync(0xffffffffu, e, off);
+      eo += __shfl_xor_sync(0xffffffffu, eo, off);
+    }
+    if (lane == 0) {
+      e = ldexp(e, 1 - 2 * kt);   // the scales of T and Tt
+      eo = ldexp(eo, -2 * kt);
+      ep[(long long)i * o + jj] = e;
+      ep[(long long)jj * o + i] = e;
+      double* eq = ep + (long long)o * o;   // opposite-spin pair energies
+      eq[(long long)i * o + jj] = eo;
+      eq[(long long)jj * o + i] = eo;
+    }
   }
 }
 
@@ -699,7 +723,7 @@ void split_plan_release(SplitPlan&) {}
 namespace {
 
 struct Layout {
-  size_t bs1, bs2, erow, drow, vdrow, thi, tlo, tts, ts, ecolm, ecol, ep, scal, total;
+  size_t bs1, bs2, erow, drow, vdrow, dnh, dnl, thi, tlo, tts, ts, ecolm, ecol, ep, epart, ecnt, scal, total;
 };
 
 // element size of the digit planes and the padding that keeps every row 16-byte aligned
@@ -747,6 +771,8 @@ Layout frag_layout(const SplitPlan& sp, const rimp2_frag& f) {
   L.erow = off; off += al256(ov * 4);
   L.drow = off; off += al256(ov * 8);
   L.vdrow = off; off += al256(ov * 8);
+  L.dnh = off; off += al256(o * rup((int)v, 32) * 4);
+  L.dnl = off; off += al256(o * rup((int)v, 32) * 4);
   L.thi = off; off += al256(ov * ldt * 4);   // T planes: rows (i,a), columns j*vpadt + b
   L.tlo = off; off += al256(ov * ldt * 4);
   L.tts = off; off += al256(st_tt * ov * ldd * esz);
@@ -754,6 +780,8 @@ Layout frag_layout(const SplitPlan& sp, const rimp2_frag& f) {
   L.ecolm = off; off += al256(X * 8);
   L.ecol = off; off += al256(X * 4);
   L.ep = off; off += al256(2 * o * o * 8);   // pair energies, opposite-spin pair energies
+  L.epart = off; off += al256(o * o * 8 * ((v + 7) / 8) * 16);   // warps' shares, at most
+  L.ecnt = off; off += al256(o * 4);
   L.scal = off; off += 256;
   L.total = off;
   return L;
@@ -782,6 +810,24 @@ double prob_mma_flops(const SplitProb& P, int slices, int bk) {
     }
   const double K = (double)P.k1_count * P.k0_blocks * bk;
   return (double)tiles * 2.0 * SG_BM * P.n_tile * K * (slices * (slices + 1) / 2);
+}
+
+// Lanes per row of the amplitude kernel: a step takes 1024 element slots whatever the width,
+// so the width that wastes fewest on rows and columns past nvir, weighted by what a full step
+// costs.  Measured per step relative to 16 lanes (nocc=100 nvir=500, MBE3 dimers, nocc=42
+// nvir=168 in FP8): BF16 1.06 with 32 lanes (its 64 columns already fill 128-byte lines with
+// 16), 1.05 with 8 (64-byte runs); FP8 0.96 and 1.25 (32 lanes are what fills its lines).
+int amp_lanes(const std::vector<SplitFragDev>& fr, bool fp8) {
+  int best = 0;
+  double cost = 0.0;
+  for (int lpr : {16, 32, 8}) {
+    double c = 0.0;
+    for (const auto& s : fr)
+      c += (double)s.o * s.o * ((s.v + 256 / lpr - 1) / (256 / lpr)) * ((s.vpad + 4 * lpr - 1) / (4 * lpr));
+    c *= lpr == 16 ? 1.0 : lpr == 32 ? (fp8 ? 0.96 : 1.06) : (fp8 ? 1.25 : 1.05);
+    if (best == 0 || c < cost) { best = lpr; cost = c; }
+  }
+  return best;
 }
 
 void finish(std::vector<SplitProb>& v, long long& total) {
@@ -842,12 +888,11 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
     s.st_out = std::max(s.st_t, s.sg_out);
     s.b_off = f.b_off; s.eo_off = f.eo_off; s.ev_off = f.ev_off;
     s.bs1 = off + L.bs1; s.bs2 = off + L.bs2; s.erow = off + L.erow; s.drow = off + L.drow;
-    s.vdrow = off + L.vdrow;
+    s.vdrow = off + L.vdrow; s.dnh = off + L.dnh; s.dnl = off + L.dnl;
     s.thi = off + L.thi; s.tlo = off + L.tlo; s.tts = off + L.tts; s.ts = off + L.ts;
     s.ecolm = off + L.ecolm; s.ecol = off + L.ecol;
-    s.ep = off + L.ep; s.scal = off + L.scal;
-    s.pair_begin = pairs; s.row_begin = rows; s.b2_tile_begin = b2t; s.qblk_begin = qbl;
-    pairs += (long long)o * o;   // amplitude stage: one CTA per ordered pair
+    s.ep = off + L.ep; s.epart = off + L.epart; s.ecnt = off + L.ecnt; s.scal = off + L.scal;
+    s.row_begin = rows; s.b2_tile_begin = b2t; s.qblk_begin = qbl;
     rows += ov;
     if (g) {
       b2t += (long long)((X + 31) / 32) * ((RL + 127) / 128);
@@ -863,7 +908,7 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
     d.ep_off = (long long)(s.ep / 8);
     d.epos_off = d.ep_off + (long long)o * o;
     d.gamma_off = f.gamma_off; d.pij_off = f.pij_off; d.pab_off = f.pab_off;
-    d.epair_off = f.epair_off; d.pair_begin = s.pair_begin;
+    d.epair_off = f.epair_off;
     fdev.push_back(d);
     max_b = std::max<long long>(max_b, (long long)ov * X);
     off += L.total;
@@ -1021,6 +1066,22 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
     for (const auto& s : w.sfd) max_x = std::max(max_x, s.X);
     w.epi_warps = max_x <= 1024 ? 16 : 8;
   }
+  // Amplitude stage: CTAs (i, j range, strip).  One range of all j where the strips alone make
+  // eight rounds of three CTAs per SM (a shorter last round costs less of the whole); shorter
+  // ranges, down to one j, for smaller waves
+  w.amp_lpr = amp_lanes(w.sfd, sp.fp8);
+  {
+    const int R = 8 * (32 / w.amp_lpr);
+    auto strips = [&](const SplitFragDev& s) { return (long long)std::max(1, (s.v + R - 1) / R); };
+    long long ctas = 0;
+    for (const auto& s : w.sfd) ctas += s.o * strips(s);
+    const long long split = ctas > 0 ? (24LL * sp.grid + ctas - 1) / ctas : 1;
+    for (auto& s : w.sfd) {
+      s.amp_jchunk = std::max(1, (int)((s.o + split - 1) / split));
+      s.pair_begin = pairs;
+      pairs += (long long)s.o * strips(s) * ((s.o + s.amp_jchunk - 1) / s.amp_jchunk);
+    }
+  }
   total_pairs = pairs;
   w.rows = rows;
   w.b2_tiles = b2t;
@@ -1111,8 +1172,12 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, const FragDev* d
   }
   if (ev) cudaEventRecordWithFlags(ev[2], s, cudaEventRecordExternal);
   if (e == cudaSuccess && total_pairs > 0) {
-    if (sp.fp8) k_amp_split<true><<<(unsigned)total_pairs, 256, 0, s>>>(sfd, nf, sp.slices_t, bs);
-    else k_amp_split<false><<<(unsigned)total_pairs, 256, 0, s>>>(sfd, nf, sp.slices_t, bs);
+    auto amp = [&](auto kernel) { kernel<<<(unsigned)total_pairs, 256, 0, s>>>(sfd, nf, bs); };
+    switch (w.amp_lpr) {
+      case 8: sp.fp8 ? amp(k_amp_split<true, 8>) : amp(k_amp_split<false, 8>); break;
+      case 16: sp.fp8 ? amp(k_amp_split<true, 16>) : amp(k_amp_split<false, 16>); break;
+      default: sp.fp8 ? amp(k_amp_split<true, 32>) : amp(k_amp_split<false, 32>); break;
+    }
     ++nl;
     e = cudaGetLastError();
   }

@@ -22,6 +22,7 @@ struct SplitFragDev {
   long long bs2;    // B digits for Gamma: [s_g][X][ldd], one scale 2^E_Q per aux index Q
   long long erow;   // int32 [o*v] row exponents of bs1
   long long drow;   // float2 [o*v]: e_i - e_a as a double-float
+  long long dnh, dnl;  // float [o][vpadt]: the same terms, hi and lo planes, zero for b >= nvir
   long long vdrow;  // float2 [o*v]: V_ii(a,a) = sum_Q (B^Q_ia)^2 (FP64 sum) as a double-float
   long long thi, tlo;  // float [o*v][ldt]: T as a double-float pair of planes, column j*vpadt + b
   long long tts, ts;   // Tt [st_out] and T [st_t] digit planes [s][o*v][ldd], one scale each
@@ -30,7 +31,10 @@ struct SplitFragDev {
   long long ecol;   // int32 [X]: exponent of each aux index of B for Gamma
   long long ep;     // double [o][o] pair energies, then [o][o] opposite-spin pair energies
   long long scal;   // uint32 [1]: max |T| exponent ([0] unused)
-  long long pair_begin;   // first amplitude CTA of the fragment (o * o ordered pairs each)
+  long long pair_begin;   // first amplitude CTA of the fragment
+  int amp_jchunk, pad3;   // j blocks per amplitude CTA
+  long long epart;  // float4 [o][o][..]: the amplitude warps' shares of e_ij and its os part
+  long long ecnt;   // uint32 [o]: amplitude CTAs done per i
   long long row_begin, b2_tile_begin;
   long long qblk_begin;   // first block (32 Q x 256 rows) of the fragment in the column maxima pass
   int sg_out, pad2;       // slices of Gamma's operands (0: no Gamma)
@@ -67,6 +71,7 @@ struct SplitWave {
   std::vector<SplitProb> probs_v, probs_c, probs_g;   // V; P_ab / P_ij; Gamma
   long long tiles_v = 0, tiles_c = 0, tiles_g = 0, rows = 0, b2_tiles = 0, qblks = 0;
   bool want_gamma = false;
+  int amp_lpr = 32;    // lanes per row of the amplitude kernel
   int epi_warps = 8;   // epilogue warps of the wave's contraction launches (see build)
   double mma_v = 0, mma_c = 0, mma_g = 0;   // tensor-core FLOPs issued per launch
   size_t off_sfd = 0, off_pv = 0, off_pc = 0, off_pg = 0;  // byte offsets in the device block
