@@ -408,6 +408,25 @@ __device__ __forceinline__ void pow2_pair(int e, float& s1, float& s2) {
   s2 = __int_as_float((e2 + 127) << 23);
 }
 
+// (h + l) 2^e in FP64.  The FP64 unit issues two operations a clock and SM, conversions
+// included, and converting, adding and scaling every element of a 128 x 80 tile there took
+// 20 us, as long as a short contraction itself: the two doubles are put together from the
+// FP32 bit patterns with integer instructions, which leaves one FP64 addition.  Values whose
+// FP32 or FP64 exponents leave the normal range take the conversions.
+__device__ __forceinline__ bool f64_bits(float x, int e, double& d) {
+  const unsigned u = __float_as_uint(x), m = u & 0x7FFFFFu;
+  const int ex = (int)((u >> 23) & 0xFFu);
+  if ((u & 0x7FFFFFFFu) == 0u) { d = 0.0; return true; }
+  const int f = ex - 127 + 1023 + e;
+  d = __hiloint2double((int)((u & 0x80000000u) | ((unsigned)f << 20) | (m >> 3)), (int)(m << 29));
+  return ex >= 1 && ex <= 254 && f >= 1 && f <= 2046;
+}
+__device__ __forceinline__ double df_scaled(float h, float l, int e) {
+  double a, b;
+  const bool ok = f64_bits(h, e, a) & f64_bits(l, e, b);
+  return ok ? a + b : ldexp((double)h + (double)l, e);
+}
+
 // ------------------------------------------------------------------ tile decode
 
 struct TileInfo {
@@ -934,17 +953,19 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
             const int n = nbase + c;
             if (n >= P->N) continue;
             const int e = ea + (P->eb_rows ? EB[n] : EB[0]) + P->eb_add - 2 * LB;
-            const double val = ldexp((double)acc_h[c] + (double)acc_l[c], e);
+            // alpha is +1 or -1: applied to the two parts, exactly
+            const float sg = (float)P->alpha;
+            const double val = df_scaled(sg * acc_h[c], sg * acc_l[c], e);
             if ((P->kind == PK_GAMMA || P->kind == PK_RAW) && P->ksplit == 1) {
-              C[(long long)m * P->ldc + n] = P->alpha * val;
+              C[(long long)m * P->ldc + n] = val;
             } else if (P->sym) {
               // each unordered pair once: (m,n) and its mirror for m < n, the diagonal once;
               // m > n is covered by the mirror of a computed tile
               if (m > n) continue;
-              atomicAdd(C + (long long)m * P->ldc + n, P->alpha * val);
-              if (m < n) atomicAdd(C + (long long)n * P->ldc + m, P->alpha * val);
+              atomicAdd(C + (long long)m * P->ldc + n, val);
+              if (m < n) atomicAdd(C + (long long)n * P->ldc + m, val);
             } else {
-              atomicAdd(C + (long long)m * P->ldc + n, P->alpha * val);
+              atomicAdd(C + (long long)m * P->ldc + n, val);
             }
           }
         }
@@ -953,6 +974,356 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
         emax = __reduce_max_sync(0xffffffffu, emax);
         if (lane == 0 && emax) atomicMax((unsigned*)((char*)bs.ws + P->et_off), emax);
       }
+    }
+  }
+
+  // ---------------------------------------------------------------- teardown
+  tc_fence_before();
+  __syncthreads();
+  if (*abort_flag && threadIdx.x == 0) atomicOr(bs.status, ST_TIMEOUT);
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u)
+                 : "memory");
+  }
+}
+
+// ------------------------------------------------------------------ slice-stacked kernel
+//
+// P_ij and P_ab of small fragments: symmetric results of a few tens of rows and columns with a
+// very long K.  In 128 x 64 tiles nocc = 28 rows fill 10 % of the tensor-core work.  Here the
+// digit slices fill the tile instead: rows (p, i) and columns (q, j), R = nocc or nvir of them
+// a slice, S R <= 256.  One MMA of 128 rows against N = S R columns forms every product
+// A_p B_q^T of those rows at once (also a few with p + q >= S, which are kept: they only
+// lengthen the sum), a second one the rows from 128 on against the slices q they need, so a
+// K step of S = 6, R = 28 takes 240 accumulator columns instead of 1344.  The operands' way
+// from L2 bounds it then (2 S R rows of 64 bytes a step).  Every (p, q) has accumulators of
+// its own, so the level sums that must be exact (see split_gemm.cuh) are shorter than in the
+// kernel above.  A thread folds its row's slices q per chunk like that kernel's levels; at the
+// end of a tile the slices p of an element meet in shared memory.
+// Roles, barriers, bounded waits and abort path as in k_split_gemm.
+constexpr int kStackEpi = 8;     // epilogue warps: two per TMEM lane quadrant, half the j each
+constexpr int kStackCols = 20;   // columns j a thread holds at most (R <= 40)
+
+struct StackTile { const SplitProb* P; int tm, tn, k1b, nK; };
+
+__device__ __forceinline__ StackTile stack_tile(const SplitProb* __restrict__ probs, int pi, long long t) {
+  StackTile ti;
+  ti.P = probs + pi;
+  const int tri = ti.P->tiles_m * (ti.P->tiles_m + 1) / 2;
+  const long long lt = t - ti.P->tile_begin;
+  const int ks = (int)(lt / tri);
+  int r = (int)(lt - (long long)ks * tri), c = 0;
+  while (r > c) { ++c; r -= c; }   // column by column: r <= c
+  ti.tm = r;
+  ti.tn = c;
+  ti.k1b = ks * ti.P->k1_chunk;
+  ti.nK = max(0, min(ti.P->k1_count, ti.k1b + ti.P->k1_chunk) - ti.k1b) * ti.P->k0_blocks;
+  return ti;
+}
+
+template <bool F8>
+__global__ void __launch_bounds__((2 + kStackEpi) * 32, 1)
+k_split_stack(const SplitProb* __restrict__ probs, const long long* __restrict__ begins, int nprobs,
+              long long total, Bases bs, unsigned* __restrict__ counter, int slices, int stages,
+              uint32_t half_bytes) {
+  constexpr int ROWB = 64, BKE = F8 ? 64 : 32;
+  constexpr int CHUNK_STAGES = (F8 ? SG_CHUNK_K_FP8 : SG_CHUNK_K_BF16) / BKE;
+  constexpr int LB = F8 ? SG_LB_FP8 : SG_LB_BF16;
+  constexpr int EXACT = F8 ? 5 : 3;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const uint32_t stage_bytes = 2 * half_bytes;   // A, then B, each 1024-byte aligned
+  uint64_t* full = (uint64_t*)(smem + (size_t)stages * stage_bytes);
+  uint64_t* empty = full + 8;
+  uint64_t* tmem_full = empty + 8;      // [2]: one per accumulator set
+  uint64_t* tmem_empty = tmem_full + 2; // [2]
+  uint64_t* tile_full = tmem_empty + 2; // [2]
+  uint64_t* tile_empty = tile_full + 2; // [2]
+  uint64_t* red_full = tile_empty + 2;  // the slices p of a tile are in shared memory
+  uint64_t* red_empty = red_full + 1;   // ... and have been summed
+  uint64_t* mma_drain = red_empty + 1;
+  long long* tile_idx = (long long*)(mma_drain + 1);   // [2]
+  int* tile_prob = (int*)(tile_idx + 2);               // [2]
+  uint32_t* tmem_base_slot = (uint32_t*)(tile_prob + 2);
+  volatile int* abort_flag = (volatile int*)(tmem_base_slot + 1);
+  float2* red = (float2*)(smem + (size_t)stages * stage_bytes + 512);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(full + s, 1);
+      mbar_init(empty + s, 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(tmem_full + s, 1);
+      mbar_init(tmem_empty + s, kStackEpi);
+      mbar_init(tile_full + s, 1);
+      mbar_init(tile_empty + s, 1 + kStackEpi);
+    }
+    mbar_init(red_full, kStackEpi);
+    mbar_init(red_empty, kStackEpi);
+    mbar_init(mma_drain, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_base_slot)),
+                 "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_base_slot;
+  const uint64_t cwait = g_sg_consumer_wait_ns;
+  // Row groups of a tile with R rows a slice: group 0 is rows 0..127 against all slices q,
+  // group 1 the rows from 128 on, whose smallest slice is p1 = 128 / R, against q < S - p1.
+  // Accumulator columns: N0, then N1 (multiples of 16).  Two sets when both fit.
+  auto cols0 = [&](int R) { return (slices * R + 15) & ~15; };
+  auto cols1 = [&](int R) { return slices * R <= 128 ? 0 : ((slices - 128 / R) * R + 15) & ~15; };
+  auto sets = [&](int R) { return 2 * (cols0(R) + cols1(R)) <= 512 ? 2u : 1u; };
+
+  if (warp == 0) {
+    // ---------------------------------------------------------------- TMA producer
+    if (lane == 0) {
+      uint32_t st = 0, ph = 0, tph = 0;
+      int tslot = 0;
+      bool pending[8] = {false, false, false, false, false, false, false, false};
+      uint32_t pend_ph[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+      for (;;) {
+        const long long t = (long long)atomicAdd(counter, 1u);
+        const int pi = t < total ? find_problem(probs, begins, nprobs, t) : 0;
+        if (!mbar_wait(tile_empty + tslot, tph ^ 1u, abort_flag)) break;
+        tile_idx[tslot] = t;
+        tile_prob[tslot] = pi;
+        mbar_arrive(tile_full + tslot);
+        tslot ^= 1;
+        if (tslot == 0) tph ^= 1u;
+        if (t >= total) break;
+        const StackTile ti = stack_tile(probs, pi, t);
+        const SplitProb* P = ti.P;
+        const int R = P->n_tile;
+        const uint32_t bytes = 2u * (uint32_t)(slices * R * ROWB);
+        bool ok = true;
+        for (int kk = 0; kk < ti.nK; ++kk) {
+          if (!mbar_wait(empty + st, ph ^ 1u, abort_flag)) { ok = false; break; }
+          pending[st] = false;
+          mbar_arrive_expect_tx(full + st, bytes);
+          pending[st] = true;
+          pend_ph[st] = ph;
+          const int k1 = ti.k1b + kk / P->k0_blocks;
+          const int x = (kk % P->k0_blocks) * BKE;
+          const uint32_t base = smem_u32(smem + (size_t)st * stage_bytes);
+          tma_operand(base, &P->tmA, full + st, P->a_mode, x, ti.tm * R, k1, P->div5, 0);
+          tma_operand(base + half_bytes, &P->tmB, full + st, P->b_mode, x, ti.tn * R, k1, P->div5, 0);
+          if (++st == (uint32_t)stages) { st = 0; ph ^= 1u; }
+        }
+        if (!ok) break;
+      }
+      if (*abort_flag) {
+        for (int s = 0; s < stages; ++s)
+          if (pending[s]) {
+            const uint64_t t0 = global_ns();
+            while (!mbar_try_wait(full + s, pend_ph[s]) && global_ns() - t0 < kWaitLimitNs) { }
+          }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ---------------------------------------------------------------- MMA issuer
+    if (lane == 0) {
+      constexpr uint32_t kFmt = F8 ? 0u : 1u;
+      const uint32_t idesc_m = (1u << 4) | (kFmt << 7) | (kFmt << 10) | ((uint32_t)(SG_BM >> 4) << 24);
+      uint32_t st = 0, ph = 0, tph = 0, use[2] = {0, 0}, set = 0;
+      bool wide = false;   // the last use of set 0 reached into set 1's columns
+      int tslot = 0;
+      for (;;) {
+        if (!mbar_wait(tile_full + tslot, tph, abort_flag, cwait)) break;
+        const long long t = tile_idx[tslot];
+        const int pi = tile_prob[tslot];
+        mbar_arrive(tile_empty + tslot);
+        tslot ^= 1;
+        if (tslot == 0) tph ^= 1u;
+        if (t >= total) break;
+        const StackTile ti = stack_tile(probs, pi, t);
+        const int R = ti.P->n_tile;
+        const uint32_t n0 = (uint32_t)cols0(R), n1 = (uint32_t)cols1(R);
+        const int chunks = (ti.nK + CHUNK_STAGES - 1) / CHUNK_STAGES;
+        bool ok = true;
+        for (int c = 0; c < chunks && ok; ++c) {
+          // set 1 only where two sets fit; a problem with one set uses set 0 for every chunk
+          set = sets(R) == 2u ? set ^ 1u : 0u;
+          const uint32_t acc = tmem_base + set * 256u;
+          if (!mbar_wait(tmem_empty + set, (use[set] & 1u) ^ 1u, abort_flag, cwait)) { ok = false; break; }
+          // a one-set problem's accumulators reach into set 1's columns: the two are never in
+          // use together
+          const uint32_t other = set ^ 1u;
+          if ((sets(R) == 1u || (set == 1u && wide)) && use[other] > 0 &&
+              !mbar_wait(tmem_empty + other, (use[other] & 1u) ^ 1u, abort_flag, cwait)) { ok = false; break; }
+          if (set == 0u) wide = sets(R) == 1u;
+          ++use[set];
+          tc_fence_after();
+          const int kend = min(ti.nK, (c + 1) * CHUNK_STAGES);
+          for (int kk = c * CHUNK_STAGES; kk < kend; ++kk) {
+            if (!mbar_wait(full + st, ph, abort_flag, cwait)) { ok = false; break; }
+            tc_fence_after();
+            const uint64_t desc = smem_desc<ROWB>(smem_u32(smem + (size_t)st * stage_bytes));
+            const uint64_t bdesc = desc + (half_bytes >> 4);
+#pragma unroll
+            for (int k16 = 0; k16 < 2; ++k16) {
+              const uint32_t add = (kk == c * CHUNK_STAGES && k16 == 0) ? 0u : 1u;
+              const uint32_t i0 = idesc_m | ((n0 >> 3) << 17), i1 = idesc_m | ((n1 >> 3) << 17);
+              if (F8) umma_f8(acc, desc + k16 * 2, bdesc + k16 * 2, i0, add);
+              else umma_bf16(acc, desc + k16 * 2, bdesc + k16 * 2, i0, add);
+              if (n1) {
+                const uint64_t a1 = desc + ((128 * ROWB) >> 4) + k16 * 2;
+                if (F8) umma_f8(acc + n0, a1, bdesc + k16 * 2, i1, add);
+                else umma_bf16(acc + n0, a1, bdesc + k16 * 2, i1, add);
+              }
+            }
+            umma_commit(empty + st);
+            if (++st == (uint32_t)stages) { st = 0; ph ^= 1u; }
+          }
+          if (ok) umma_commit(tmem_full + set);
+        }
+        if (!ok) break;
+      }
+      if (*abort_flag) {
+        umma_commit(mma_drain);
+        const uint64_t t0 = global_ns();
+        while (!mbar_try_wait(mma_drain, 0) && global_ns() - t0 < kWaitLimitNs) { }
+      }
+    }
+    __syncwarp();
+  } else {
+    // ---------------------------------------------------------------- epilogue
+    const int ew = warp - 2, quad = warp & 3, half = ew >> 2;
+    const int row = quad * 32 + lane;
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
+    uint32_t use[2] = {0, 0}, set = 0, tph = 0, rph = 0;
+    int tslot = 0;
+    for (;;) {
+      if (!mbar_wait_warp(tile_full + tslot, tph, abort_flag, cwait)) break;
+      const long long t = tile_idx[tslot];
+      const int pi = tile_prob[tslot];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tile_empty + tslot);
+      tslot ^= 1;
+      if (tslot == 0) tph ^= 1u;
+      if (t >= total) break;
+      const StackTile ti = stack_tile(probs, pi, t);
+      const SplitProb* P = ti.P;
+      const int R = P->n_tile;                        // a multiple of 4
+      const int jh = ((R >> 1) + 3) & ~3;             // columns of the first half
+      const int j0 = half ? jh : 0, nj = half ? R - jh : jh;   // multiples of 4
+      const int n0 = cols0(R), n1 = cols1(R);
+      const int chunks = (ti.nK + CHUNK_STAGES - 1) / CHUNK_STAGES;
+      f2x acc_h[2][kStackCols / 2], acc_l[2][kStackCols / 2];
+#pragma unroll
+      for (int g = 0; g < 2; ++g)
+#pragma unroll
+        for (int c = 0; c < kStackCols / 2; ++c) acc_h[g][c] = acc_l[g][c] = 0ull;
+      bool ok = true;
+      for (int ch = 0; ch < chunks; ++ch) {
+        set = sets(R) == 2u ? set ^ 1u : 0u;
+        if (!mbar_wait_warp(tmem_full + set, use[set] & 1u, abort_flag, cwait)) { ok = false; break; }
+        ++use[set];
+        tc_fence_after();
+        const uint32_t set_addr = lane_addr + set * 256u + (uint32_t)j0;
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          if (g == 1 && n1 == 0) break;
+          const int nq = g == 0 ? slices : slices - 128 / R;
+          for (int q = nq - 1; q >= 0; --q) {
+            float v[kStackCols];
+#pragma unroll
+            for (int u = 0; u < kStackCols / 4; ++u)
+              if (4 * u < nj)
+                tmem_ld4(set_addr + (uint32_t)((g ? n0 : 0) + q * R + 4 * u), v + 4 * u);
+            tmem_wait_ld();
+            tmem_hold<kStackCols>(v);
+            const float sc = __int_as_float((127 - LB * q) << 23);   // 2^(-LB q)
+            const f2x sc2 = f2_pack(sc, sc);
+            if (q >= EXACT) {
+#pragma unroll
+              for (int c = 0; c < kStackCols / 2; ++c)
+                if (2 * c < nj) acc_l[g][c] = f2_fma(f2_pack(v[2 * c], v[2 * c + 1]), sc2, acc_l[g][c]);
+            } else {
+#pragma unroll
+              for (int c = 0; c < kStackCols / 2; ++c)
+                if (2 * c < nj) {
+                  f2x s2, e2;
+                  f2_two_sum(acc_h[g][c], f2_mul(f2_pack(v[2 * c], v[2 * c + 1]), sc2), s2, e2);
+                  acc_h[g][c] = s2;
+                  acc_l[g][c] = f2_add(acc_l[g][c], e2);
+                }
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tmem_empty + set);
+#pragma unroll
+        for (int g = 0; g < 2; ++g)
+#pragma unroll
+          for (int c = 0; c < kStackCols / 2; ++c) {
+            f2x s2, e2;
+            f2_two_sum(acc_h[g][c], acc_l[g][c], s2, e2);
+            acc_h[g][c] = s2;
+            acc_l[g][c] = e2;
+          }
+      }
+      if (!ok) break;
+      // the rows (p, i), scaled by 2^(-LB p), to shared memory (free once the previous
+      // tile's sums are done)
+      if (!mbar_wait_warp(red_empty, rph ^ 1u, abort_flag, cwait)) break;
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        const int r = 128 * g + row;
+        if (r < slices * R) {
+          const float sc = __int_as_float((127 - LB * (r / R)) << 23);
+#pragma unroll
+          for (int c = 0; c < kStackCols / 2; ++c)
+            if (2 * c < nj) {
+              float h0, h1, l0, l1;
+              f2_unpack(acc_h[g][c], h0, h1);
+              f2_unpack(acc_l[g][c], l0, l1);
+              float2* o = red + (size_t)r * R + j0 + 2 * c;
+              o[0] = make_float2(h0 * sc, l0 * sc);
+              o[1] = make_float2(h1 * sc, l1 * sc);
+            }
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(red_full);
+      if (!mbar_wait_warp(red_full, rph, abort_flag, cwait)) break;
+      rph ^= 1u;
+      {
+        const char* wsb = (const char*)bs.ws;
+        const int e = ((const int*)(wsb + P->ea_off))[0] + P->ea_add + ((const int*)(wsb + P->eb_off))[0] +
+                      P->eb_add - 2 * LB;
+        double* C = (P->kind == PK_PAB ? bs.pab : bs.pij) + P->c_off;
+        const float sg = (float)P->alpha;
+        for (int x = ew * 32 + lane; x < R * R; x += 32 * kStackEpi) {
+          const int i = x / R, j = x - i * R;
+          const int m = ti.tm * R + i, n = ti.tn * R + j;
+          if (m > n || n >= P->N) continue;   // each unordered pair once
+          df s = {0.f, 0.f};
+          for (int p = slices - 1; p >= 0; --p) {
+            const float2 w = red[(size_t)(p * R + i) * R + j];
+            s = df_add(s, {w.x, w.y});
+          }
+          const double val = df_scaled(sg * s.h, sg * s.l, e);
+          atomicAdd(C + (long long)m * P->ldc + n, val);
+          if (m < n) atomicAdd(C + (long long)n * P->ldc + m, val);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(red_empty);
     }
   }
 
@@ -1036,6 +1407,10 @@ cudaError_t split_gemm_prepare() {
   RIMP2_PREP(48, 64, false, 16)
   RIMP2_PREP(64, 64, true, 16) RIMP2_PREP(48, 64, true, 16) RIMP2_PREP(32, 64, true, 16)
 #undef RIMP2_PREP
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_split_stack<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_split_stack<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   return e;
 }
 
@@ -1068,6 +1443,36 @@ cudaError_t launch_split_gemm(const SplitProb* d_probs, const long long* d_begin
 cudaError_t split_gemm_set_consumer_wait(long long ns) {
   const unsigned long long v = ns < 0 ? kWaitLimitNs : (unsigned long long)ns;
   return cudaMemcpyToSymbol(g_sg_consumer_wait_ns, &v, sizeof(v));
+}
+
+// Rows a slice of the stacked kernel for an extent n (nocc or nvir) of `slices` digit planes,
+// a multiple of 4, or 0 where it does not fit (more than 40 or 256 / slices rows).
+int split_stack_rows(int slices, int n) {
+  const int R = (n + 3) / 4 * 4;
+  return R > 0 && R <= 2 * kStackCols && slices * R <= 256 ? R : 0;
+}
+
+cudaError_t launch_split_stack(const SplitProb* d_probs, const long long* d_begins, int nprobs,
+                               long long total_tiles, Bases bs, unsigned* counter, int slices,
+                               int max_rows, bool fp8, int grid, cudaStream_t s) {
+  if (total_tiles <= 0) return cudaSuccess;
+  const size_t half = ((size_t)slices * max_rows * 64 + 1023) / 1024 * 1024;
+  const size_t red = (size_t)slices * max_rows * max_rows * sizeof(float2);
+  // 16 KB of slack: an MMA reads 128 rows of A and up to 12 rows past B whatever the tile holds
+  const size_t fixed = 1024 + 512 + red;
+  const size_t slack = 16384 > red ? 16384 - red : 0;
+  int stages = (int)((227 * 1024 - fixed - slack) / (2 * half));
+  stages = stages > 8 ? 8 : stages;
+  if (stages < 1) return cudaErrorInvalidValue;
+  const size_t smem = fixed + slack + (size_t)stages * 2 * half;
+  const unsigned g = (unsigned)(total_tiles < grid ? total_tiles : grid);
+  if (fp8)
+    k_split_stack<true><<<g, (2 + kStackEpi) * 32, smem, s>>>(d_probs, d_begins, nprobs, total_tiles, bs,
+                                                             counter, slices, stages, (uint32_t)half);
+  else
+    k_split_stack<false><<<g, (2 + kStackEpi) * 32, smem, s>>>(d_probs, d_begins, nprobs, total_tiles, bs,
+                                                              counter, slices, stages, (uint32_t)half);
+  return cudaGetLastError();
 }
 
 int split_gemm_grid() {

@@ -96,6 +96,13 @@ SplitLaunch split_launch_config(int slices, int bk = 32, int n_tile = 0, bool fp
 cudaError_t launch_split_gemm(const SplitProb* d_probs, const long long* d_begins, int nprobs,
                               long long total_tiles, Bases bs, unsigned* counter,
                               const SplitLaunch& cfg, int grid, cudaStream_t s);
+// The slice-stacked kernel for P_ij and P_ab of small fragments (TM_4D operands with boxes of
+// n_tile = split_stack_rows(slices, extent) rows; tiles_m tiles a side, upper triangle, the K
+// piece outermost in the tile order)
+int split_stack_rows(int slices, int n);
+cudaError_t launch_split_stack(const SplitProb* d_probs, const long long* d_begins, int nprobs,
+                               long long total_tiles, Bases bs, unsigned* counter, int slices,
+                               int max_rows, bool fp8, int grid, cudaStream_t s);
 int split_gemm_grid();
 // Consumer-side wait limit of the contraction kernel on the current device (ns < 0: the
 // normal 2 s); synchronous.  Used by a test hook only.

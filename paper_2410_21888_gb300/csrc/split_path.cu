@@ -15,6 +15,7 @@
 //   8. zero P, split GEMMs for P_ab and P_ij, then for Gamma (Appendix Gamma, D^MP2_ab,
 //      D^MP2_ij); Gamma contracts the leading s_g digit planes of Tt
 #include <climits>
+#include <cmath>
 #include <cstring>
 #include <algorithm>
 
@@ -859,6 +860,7 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
   const SplitLaunch& cg = sgl == st ? sp.cfg_t : sp.cfg_g;
   const int NTv = sp.cfg_v.n_tile_max, NTt = sp.cfg_t.n_tile_max, NTg = cg.n_tile_max;
   const int BKv = sp.cfg_v.bk, BKt = sp.cfg_t.bk, BKg = cg.bk;
+  const int BKs = sp.fp8 ? 64 : 32;   // K per stage of the slice-stacked kernel
   // split-K target of P_ab / P_ij in multiples of the grid: finer pieces keep the tiles of
   // one occupied-index range closer together in time (their operand rows stay in L2);
   // measured at nocc=100 nvir=500 naux=1500: the P launch 33.3 ms at 2x, 32.2 at 8x, 31.6
@@ -936,6 +938,32 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
       w.probs_v.push_back(P);
     }
     const uint64_t plane_b = (uint64_t)ov * ldd * E2;
+    // P_ij / P_ab of small extents: slice-stacked tiles, one a side, or two in BF16 (up to 80
+    // rows with 6 slices; three tiles of 40 x 40 rows then read less than a 128 x 64 tile or
+    // two; FP8 at nocc = 42: 1.73 ms either way, so it stays in the launch it shares with
+    // Gamma).  The contraction runs over k = (k1, k0) of 4-D views {k0, row, k1, slice}.
+    auto stacked = [&](int kind, int n, const uint64_t* d4, const uint64_t* s4, int k0, int k1) -> int {
+      const int most = sp.fp8 ? 1 : 2;
+      int nb = 1;
+      while (nb <= most && split_stack_rows(st, (n + nb - 1) / nb) == 0) ++nb;
+      if (nb > most) return 0;
+      SplitProb P{};
+      P.kind = kind; P.frag = idx;
+      P.M = P.N = n; P.n_tile = split_stack_rows(st, (n + nb - 1) / nb);
+      P.tiles_m = P.tiles_n = nb;
+      P.k0_blocks = (k0 + BKs - 1) / BKs; P.k1_count = k1;
+      P.a_mode = P.b_mode = TM_4D; P.div5 = 1;
+      P.ea_off = P.eb_off = s.scal + 4;
+      P.ea_add = kTtAdd; P.eb_add = kTAdd;
+      P.c_off = kind == PK_PAB ? f.pab_off : f.pij_off;
+      P.ldc = n; P.alpha = kind == PK_PAB ? 1.0 : -1.0; P.sym = 1; P.ks_outer = 1;
+      const uint32_t box[4] = {(uint32_t)BKs, (uint32_t)P.n_tile, 1, (uint32_t)st};
+      if (encode_tmap(&P.tmA, wsb + s.tts, 4, d4, s4, box, (int)E2) != RIMP2_OK ||
+          encode_tmap(&P.tmB, wsb + s.ts, 4, d4, s4, box, (int)E2) != RIMP2_OK)
+        return -1;
+      w.probs_s.push_back(P);
+      return 1;
+    };
     if (g) {  // Gamma[(i,a)][Q] = sum_(j,b) Tt[(i,a)][(j,b)] B[(j,b)][Q]
       SplitProb P{};
       P.kind = PK_GAMMA; P.frag = idx;
@@ -974,7 +1002,14 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
       // with the slice count of P, Gamma joins P's launch
       (sgl == st ? w.probs_c : w.probs_g).push_back(P);
     }
-    if (f.pab_off >= 0) {  // P_ab = sum_i sum_(j,c) Tt[(i,a)][(j,c)] T[(i,b)][(j,c)]
+    const uint64_t d4ab[4] = {(uint64_t)RL, (uint64_t)v, (uint64_t)o, (uint64_t)st};
+    const uint64_t s4ab[3] = {(uint64_t)ldd * E2, (uint64_t)v * ldd * E2, plane_b};
+    const int st_ab = f.pab_off >= 0 ? stacked(PK_PAB, v, d4ab, s4ab, RL, o) : 0;
+    const uint64_t d4ij[4] = {(uint64_t)vpad, (uint64_t)o, (uint64_t)ov, (uint64_t)st};
+    const uint64_t s4ij[3] = {(uint64_t)vpad * E2, (uint64_t)ldd * E2, plane_b};
+    const int st_ij = f.pij_off >= 0 ? stacked(PK_PIJ, o, d4ij, s4ij, vpad, ov) : 0;
+    if (st_ab < 0 || st_ij < 0) return RIMP2_ERR_UNSUPPORTED;
+    if (f.pab_off >= 0 && !st_ab) {  // P_ab = sum_i sum_(j,c) Tt[(i,a)][(j,c)] T[(i,b)][(j,c)]
       SplitProb P{};
       P.kind = PK_PAB; P.frag = idx;
       P.M = P.N = v; P.n_tile = NTt;
@@ -990,15 +1025,13 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
       // launch re-read its operands from DRAM (226 GB at nocc=100 nvir=500, 0.92 of HBM)
       P.ks_outer = 1;
       P.ntiles = (long long)P.tiles_m * P.tiles_n * P.ksplit;
-      const uint64_t d4[4] = {(uint64_t)RL, (uint64_t)v, (uint64_t)o, (uint64_t)st};
-      const uint64_t s4[3] = {(uint64_t)ldd * E2, (uint64_t)v * ldd * E2, plane_b};
       const uint32_t boxA[4] = {(uint32_t)BKt, SG_BM, 1, (uint32_t)st}, boxB[4] = {(uint32_t)BKt, (uint32_t)NTt, 1, (uint32_t)st};
-      if (encode_tmap(&P.tmA, wsb + s.tts, 4, d4, s4, boxA, (int)E2) != RIMP2_OK ||
-          encode_tmap(&P.tmB, wsb + s.ts, 4, d4, s4, boxB, (int)E2) != RIMP2_OK)
+      if (encode_tmap(&P.tmA, wsb + s.tts, 4, d4ab, s4ab, boxA, (int)E2) != RIMP2_OK ||
+          encode_tmap(&P.tmB, wsb + s.ts, 4, d4ab, s4ab, boxB, (int)E2) != RIMP2_OK)
         return RIMP2_ERR_UNSUPPORTED;
       w.probs_c.push_back(P);
     }
-    if (f.pij_off >= 0 && pij_direct) {  // P_ij = -sum_(k,a) sum_b Tt[(i,a)][(k,b)] T[(j,a)][(k,b)]
+    if (f.pij_off >= 0 && !st_ij && pij_direct) {  // P_ij = -sum_(k,a) sum_b Tt[(i,a)][(k,b)] T[(j,a)][(k,b)]
       SplitProb P{};
       P.kind = PK_PIJ; P.frag = idx;
       P.M = P.N = o; P.n_tile = NTt;
@@ -1018,7 +1051,7 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
           encode_tmap(&P.tmB, wsb + s.ts, 5, d5, s5, boxB, (int)E2) != RIMP2_OK)
         return RIMP2_ERR_UNSUPPORTED;
       w.probs_c.push_back(P);
-    } else if (f.pij_off >= 0) {
+    } else if (f.pij_off >= 0 && !st_ij) {
       // P_ij through the pair symmetry Tt_ik(a,b) = Tt_ki(b,a):
       // P_ij = -sum_(k,b) sum_a Tt[(k,b)][(i,a)] T[(k,b)][(j,a)]; the rows i of one
       // (k,b) row are vpad elements apart, so a 128-row TMA box reads one contiguous span
@@ -1034,11 +1067,9 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
       choose_split_k(P, sp.grid, split_mul);
       P.ks_outer = 1;   // as for P_ab: the tiles in flight share one (k,b) range
       P.ntiles = (long long)P.tiles_m * P.tiles_n * P.ksplit;
-      const uint64_t d4[4] = {(uint64_t)vpad, (uint64_t)o, (uint64_t)ov, (uint64_t)st};
-      const uint64_t s4[3] = {(uint64_t)vpad * E2, (uint64_t)ldd * E2, plane_b};
       const uint32_t boxA[4] = {(uint32_t)BKt, SG_BM, 1, (uint32_t)st}, boxB[4] = {(uint32_t)BKt, (uint32_t)NTt, 1, (uint32_t)st};
-      if (encode_tmap(&P.tmA, wsb + s.tts, 4, d4, s4, boxA, (int)E2) != RIMP2_OK ||
-          encode_tmap(&P.tmB, wsb + s.ts, 4, d4, s4, boxB, (int)E2) != RIMP2_OK)
+      if (encode_tmap(&P.tmA, wsb + s.tts, 4, d4ij, s4ij, boxA, (int)E2) != RIMP2_OK ||
+          encode_tmap(&P.tmB, wsb + s.ts, 4, d4ij, s4ij, boxB, (int)E2) != RIMP2_OK)
         return RIMP2_ERR_UNSUPPORTED;
       w.probs_c.push_back(P);
     }
@@ -1046,17 +1077,54 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
   // A split-K piece of P_ab / P_ij spans at least kMinPieceK elements of K: the per-problem
   // target (a multiple of the grid, for locality at large sizes) would otherwise cut the
   // P_ij of small fragments, K0 = nvir per outer index, into pieces whose drain, epilogue
-  // and atomics cost as much as their MMAs
-  for (auto& P : w.probs_c)
-    if (P.kind == PK_PAB || P.kind == PK_PIJ) {
-      const long long per = (long long)P.k0_blocks * BKt;   // K elements per outer index
-      const int chunk = (int)std::min<long long>(P.k1_count, (kMinPieceK + per - 1) / per);
-      if (P.k1_chunk < chunk) {
-        P.k1_chunk = chunk;
-        P.ksplit = std::max(1, (P.k1_count + chunk - 1) / chunk);
-        P.ntiles = (long long)P.tiles_m * P.tiles_n * P.ksplit;
+  // and atomics cost as much as their MMAs.  A launch whose pieces would not fill the grid
+  // twice takes shorter ones, down to one accumulation chunk.
+  {
+    double work = 0.0;
+    for (const auto& P : w.probs_c) work += (double)P.tiles_m * P.tiles_n * P.k1_count * P.k0_blocks * BKt;
+    const long long least = std::max<long long>(512, std::min<long long>(kMinPieceK, (long long)(work / (2.0 * sp.grid))));
+    for (auto& P : w.probs_c)
+      if (P.kind == PK_PAB || P.kind == PK_PIJ) {
+        const long long per = (long long)P.k0_blocks * BKt;   // K elements per outer index
+        const int chunk = (int)std::min<long long>(P.k1_count, (least + per - 1) / per);
+        if (P.k1_chunk < chunk) {
+          P.k1_chunk = chunk;
+          P.ksplit = std::max(1, (P.k1_count + chunk - 1) / chunk);
+          P.ntiles = (long long)P.tiles_m * P.tiles_n * P.ksplit;
+        }
       }
+  }
+  // Slice-stacked pieces: eight per SM over the launch, at least eight stages each
+  {
+    double stages = 0.0;
+    auto tri = [](const SplitProb& P) { return (long long)P.tiles_m * (P.tiles_m + 1) / 2; };
+    for (const auto& P : w.probs_s) stages += (double)tri(P) * P.k1_count * P.k0_blocks;
+    const double piece = std::max(8.0, stages / (8.0 * sp.grid));
+    w.stack_rows = 0;
+    for (auto& P : w.probs_s) {
+      P.k1_chunk = (int)std::min<double>(P.k1_count, std::max(1.0, std::ceil(piece / P.k0_blocks)));
+      P.ksplit = std::max(1, (P.k1_count + P.k1_chunk - 1) / P.k1_chunk);
+      P.ntiles = tri(P) * P.ksplit;
+      w.stack_rows = std::max(w.stack_rows, P.n_tile);
     }
+  }
+  // A Gamma launch of few tiles is cut along K as well (at least four stages a slab)
+  {
+    long long tiles = 0;
+    for (const auto& P : w.probs_g) tiles += P.ntiles;
+    const int want = tiles > 0 && sp.variant != 3 ? (int)std::min<long long>(8, sp.grid / tiles) : 1;
+    for (auto& P : w.probs_g) {
+      const int slabs = std::min(want, P.k0_blocks / 4);
+      if (P.k1_count != 1 || slabs < 2) continue;
+      const int per = (P.k0_blocks + slabs - 1) / slabs;
+      P.k1_count = P.ksplit = (P.k0_blocks + per - 1) / per;
+      P.k0_blocks = per;
+      P.a_mode = P.b_mode = TM_3DK; P.div5 = per * BKg; P.ks_outer = 1;
+      P.ntiles *= P.ksplit;
+      for (auto& d : fdev)
+        if (d.idx == P.frag) d.zero_gamma = 1;
+    }
+  }
   // Sixteen epilogue warps when every fragment's aux dimension is short: V's tiles then
   // have little K for their MMAs to hide the T = V/D epilogue behind, which more warps
   // share (MBE3 stated batch: dimer level 86.1 -> 79.3 ms); with naux ~1500 the extra
@@ -1089,6 +1157,7 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
   finish(w.probs_v, w.tiles_v);
   finish(w.probs_c, w.tiles_c);
   finish(w.probs_g, w.tiles_g);
+  finish(w.probs_s, w.tiles_s);
   // every problem's tiles and TMA boxes must match the kernel instance of its launch
   auto same_shape = [](const std::vector<SplitProb>& v, const SplitLaunch& c) {
     for (const auto& P : v)
@@ -1102,6 +1171,11 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
   for (const auto& P : w.probs_v) w.mma_v += prob_mma_flops(P, sv, BKv);
   for (const auto& P : w.probs_c) w.mma_c += prob_mma_flops(P, st, BKt);
   for (const auto& P : w.probs_g) w.mma_g += prob_mma_flops(P, sgl, BKg);
+  for (const auto& P : w.probs_s) {   // 128 rows x the accumulator columns of both row groups
+    const int R = P.n_tile, n0 = (st * R + 15) / 16 * 16;
+    const int n1 = st * R <= 128 ? 0 : ((st - 128 / R) * R + 15) / 16 * 16;
+    w.mma_c += 2.0 * SG_BM * (n0 + n1) * (double)P.k1_count * P.k0_blocks * BKs * (P.tiles_m * (P.tiles_m + 1) / 2);
+  }
   return RIMP2_OK;
 }
 
@@ -1111,9 +1185,11 @@ size_t split_layout_wave(SplitWave& w, size_t off) {
   w.off_pv = off; off = al256(off + w.probs_v.size() * sizeof(SplitProb));
   w.off_pc = off; off = al256(off + w.probs_c.size() * sizeof(SplitProb));
   w.off_pg = off; off = al256(off + w.probs_g.size() * sizeof(SplitProb));
+  w.off_ps = off; off = al256(off + w.probs_s.size() * sizeof(SplitProb));
   w.off_bv = off; off = al256(off + w.probs_v.size() * sizeof(long long));
   w.off_bc = off; off = al256(off + w.probs_c.size() * sizeof(long long));
   w.off_bg = off; off = al256(off + w.probs_g.size() * sizeof(long long));
+  w.off_bs = off; off = al256(off + w.probs_s.size() * sizeof(long long));
   return off;
 }
 
@@ -1122,6 +1198,7 @@ void split_fill_wave(const SplitWave& w, char* host) {
   if (!w.probs_v.empty()) memcpy(host + w.off_pv, w.probs_v.data(), w.probs_v.size() * sizeof(SplitProb));
   if (!w.probs_c.empty()) memcpy(host + w.off_pc, w.probs_c.data(), w.probs_c.size() * sizeof(SplitProb));
   if (!w.probs_g.empty()) memcpy(host + w.off_pg, w.probs_g.data(), w.probs_g.size() * sizeof(SplitProb));
+  if (!w.probs_s.empty()) memcpy(host + w.off_ps, w.probs_s.data(), w.probs_s.size() * sizeof(SplitProb));
   auto begins = [&](const std::vector<SplitProb>& v, size_t off) {
     for (size_t k = 0; k < v.size(); ++k) {
       const long long b = v[k].tile_begin;
@@ -1131,6 +1208,7 @@ void split_fill_wave(const SplitWave& w, char* host) {
   begins(w.probs_v, w.off_bv);
   begins(w.probs_c, w.off_bc);
   begins(w.probs_g, w.off_bg);
+  begins(w.probs_s, w.off_bs);
 }
 
 int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, const FragDev* dfd, int nf,
@@ -1192,6 +1270,12 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, const FragDev* d
                           ctr + 1, cfg, sp.grid, s);
     ++nl;
   }
+  if (e == cudaSuccess && w.tiles_s > 0) {
+    e = launch_split_stack((const SplitProb*)(dblk + w.off_ps), (const long long*)(dblk + w.off_bs),
+                           (int)w.probs_s.size(), w.tiles_s, bs, ctr + 3, sp.slices_t, w.stack_rows,
+                           sp.fp8, sp.grid, s);
+    ++nl;
+  }
   if (ev) cudaEventRecordWithFlags(ev[4], s, cudaEventRecordExternal);
   if (e == cudaSuccess && w.tiles_g > 0) {
     SplitLaunch cfg = sp.cfg_g;
@@ -1203,7 +1287,7 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, const FragDev* d
   }
   if (ev) cudaEventRecordWithFlags(ev[5], s, cudaEventRecordExternal);
   *launches = nl;
-  *tiles = w.tiles_v + w.tiles_c + w.tiles_g;
+  *tiles = w.tiles_v + w.tiles_c + w.tiles_g + w.tiles_s;
   return e == cudaSuccess ? RIMP2_OK : RIMP2_ERR_CUDA;
 }
 
