@@ -8,6 +8,7 @@
 
 #include <algorithm>
 
+#include "energy.cuh"
 #include "fp64_gemm.cuh"
 
 namespace rimp2 {
@@ -245,56 +246,11 @@ cudaError_t launch_amplitude_f64(const FragDev* d_frags, int nfrag, long long to
 
 // ------------------------------------------------------------------ energy reduction
 
-__device__ __forceinline__ void two_sum(double a, double b, double& s, double& e) {
-  s = a + b;
-  const double bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
-}
-
-// One CTA per fragment: E = sum_ij e_pair[i][j] with compensated (TwoSum) sums in a
-// fixed order; copies e_pair to the caller's buffer when requested.
 __global__ void __launch_bounds__(256)
 k_energy_reduce(const FragDev* __restrict__ frags, Bases bs) {
-  __shared__ double ss[256], cc[256];
-  const FragDev F = frags[blockIdx.x];
-  const long long n = (long long)F.o * F.o;
-  // compensated (TwoSum) sum of x[0..n): per-thread running sums, then a tree
-  auto csum = [&](const double* x, double* copy_to) -> double {
-    double s = 0.0, c = 0.0;
-    for (long long e = threadIdx.x; e < n; e += blockDim.x) {
-      const double y = x[e];
-      double t, err;
-      two_sum(s, y, t, err);
-      s = t;
-      c += err;
-      if (copy_to) copy_to[e] = y;
-    }
-    ss[threadIdx.x] = s;
-    cc[threadIdx.x] = c;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-      if ((int)threadIdx.x < w) {
-        double t, err;
-        two_sum(ss[threadIdx.x], ss[threadIdx.x + w], t, err);
-        ss[threadIdx.x] = t;
-        cc[threadIdx.x] += cc[threadIdx.x + w] + err;
-      }
-      __syncthreads();
-    }
-    const double r = ss[0] + cc[0];
-    __syncthreads();   // ss / cc are reused by the next sum
-    return r;
-  };
-  const double e = csum(bs.ws + F.ep_off, F.epair_off >= 0 ? bs.epair + F.epair_off : nullptr);
-  if (threadIdx.x == 0) bs.energy[F.idx] = e;
-  if ((bs.energy_os || bs.energy_scs) && F.epos_off >= 0) {
-    const double eos = csum(bs.ws + F.epos_off, nullptr);
-    if (threadIdx.x == 0) {
-      if (bs.energy_os) bs.energy_os[F.idx] = eos;
-      // spin-component scaling: c_os E_OS + c_ss E_SS with E_SS = E - E_OS
-      if (bs.energy_scs) bs.energy_scs[F.idx] = bs.scs_os * eos + bs.scs_ss * (e - eos);
-    }
-  }
+  const FragDev& F = frags[blockIdx.x];
+  fragment_energy(bs.ws + F.ep_off, F.epos_off >= 0 ? bs.ws + F.epos_off : nullptr,
+                  (long long)F.o * F.o, F.epair_off >= 0 ? bs.epair + F.epair_off : nullptr, F.idx, bs);
 }
 
 cudaError_t launch_energy_reduce(const FragDev* d_frags, int nfrag, Bases bs, cudaStream_t s) {
@@ -308,13 +264,11 @@ cudaError_t launch_energy_reduce(const FragDev* d_frags, int nfrag, Bases bs, cu
 __global__ void k_zero_p(const FragDev* __restrict__ frags, Bases bs) {
   const FragDev F = frags[blockIdx.y];
   const long long no = (long long)F.o * F.o, nv = (long long)F.v * F.v;
-  const long long ng = (F.zero_gamma && F.gamma_off >= 0) ? (long long)F.o * F.v * F.X : 0;
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < no + nv + ng;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < no + nv;
        e += stride) {
     if (e < no) { if (F.pij_off >= 0) bs.pij[F.pij_off + e] = 0.0; }
-    else if (e < no + nv) { if (F.pab_off >= 0) bs.pab[F.pab_off + (e - no)] = 0.0; }
-    else bs.gamma[F.gamma_off + (e - no - nv)] = 0.0;
+    else if (F.pab_off >= 0) bs.pab[F.pab_off + (e - no)] = 0.0;
   }
 }
 

@@ -234,7 +234,7 @@ int upload_descriptors(rimp2_plan* p, const rimp2_frag* frags, const double* B, 
       int rc = build_fp64_wave(p, frags, w);
       if (rc != RIMP2_OK) return rc;
     } else {
-      int rc = split_build_wave(p->split, frags, m, B, ws, w.fdev, w.split, w.total_pairs, w.max_b);
+      int rc = split_build_wave(p->split, frags, m, B, ws, w.split, w.total_pairs);
       if (rc != RIMP2_OK) return rc;
     }
     p->waves.push_back(std::move(w));
@@ -288,17 +288,19 @@ int enqueue(rimp2_plan* p, const rimp2_batch* b, void* ws, cudaStream_t s) {
   bs.energy_scs = b->energy_scs; bs.scs_os = p->opt.scs_os; bs.scs_ss = p->opt.scs_ss;
   int launches = 0;
   long long tiles = 0;
-  if (cudaMemsetAsync(p->d_counters, 0, p->waves.size() * 8 * sizeof(unsigned), s) != cudaSuccess)
+  // the split path's prologue kernel clears its wave's counters
+  if (p->precision == RIMP2_FP64 &&
+      cudaMemsetAsync(p->d_counters, 0, p->waves.size() * 8 * sizeof(unsigned), s) != cudaSuccess)
     return RIMP2_ERR_CUDA;
   for (size_t wi = 0; wi < p->waves.size(); ++wi) {
     WaveDesc& w = p->waves[wi];
     const FragDev* dfd = (const FragDev*)(p->dblk + w.off_fdev);
-    const int nf = (int)w.fdev.size();
+    const int nf = (int)w.frags.size();
     unsigned* ctr = p->d_counters + wi * 8;
     cudaError_t e = cudaSuccess;
     cudaEvent_t* ev = p->stage_ev.empty() ? nullptr : &p->stage_ev[wi * kEv];
     if (ev && cudaEventRecordWithFlags(ev[0], s, cudaEventRecordExternal) != cudaSuccess) return RIMP2_ERR_CUDA;
-    if (p->opt.check_inputs) {
+    if (p->opt.check_inputs && p->precision == RIMP2_FP64) {
       e = launch_check_inputs(dfd, nf, (w.max_b + 255) / 256, bs, s);
       ++launches;
       if (e != cudaSuccess) return RIMP2_ERR_CUDA;
@@ -325,8 +327,8 @@ int enqueue(rimp2_plan* p, const rimp2_batch* b, void* ws, cudaStream_t s) {
     } else {
       int nl = 0;
       long long nt = 0;
-      int rc = split_enqueue_wave(p->split, w.split, p->dblk, dfd, nf, w.total_pairs, bs, ctr, s,
-                                  &nl, &nt, ev);
+      int rc = split_enqueue_wave(p->split, w.split, p->dblk, nf, w.total_pairs, bs,
+                                  p->opt.check_inputs != 0, ctr, s, &nl, &nt, ev);
       launches += nl;
       tiles += nt;
       if (rc != RIMP2_OK) return rc;

@@ -427,6 +427,24 @@ __device__ __forceinline__ double df_scaled(float h, float l, int e) {
   return ok ? a + b : ldexp((double)h + (double)l, e);
 }
 
+// Transposes a 4 x 4 block held by four neighbouring lanes (a row each, x[c] its columns):
+// afterwards x[k] is row k of column lane & 3, so that four lanes hold 32 consecutive bytes of
+// an FP64 row.
+__device__ __forceinline__ void quad_transpose(float (&x)[4], int lane) {
+  const bool b = lane & 1, c = lane & 2;
+  float r0 = __shfl_xor_sync(0xffffffffu, b ? x[0] : x[1], 1);
+  float r1 = __shfl_xor_sync(0xffffffffu, b ? x[2] : x[3], 1);
+  if (b) { x[0] = r0; x[2] = r1; } else { x[1] = r0; x[3] = r1; }
+  r0 = __shfl_xor_sync(0xffffffffu, c ? x[0] : x[2], 2);
+  r1 = __shfl_xor_sync(0xffffffffu, c ? x[1] : x[3], 2);
+  if (c) { x[0] = r0; x[1] = r1; } else { x[2] = r0; x[3] = r1; }
+}
+
+__device__ __forceinline__ void prefetch_tmaps(const SplitProb* P) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(&P->tmA) : "memory");
+  asm volatile("prefetch.tensormap [%0];" ::"l"(&P->tmB) : "memory");
+}
+
 // ------------------------------------------------------------------ tile decode
 
 struct TileInfo {
@@ -559,6 +577,7 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
   int* stage_eb = (int*)(stage_dn + EPI * NC);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int first_prob = 0;
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) {
       mbar_init(full + s, 1);
@@ -576,6 +595,9 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    // the CTA's first entry is its own index: found, and its tensor maps fetched, meanwhile
+    first_prob = find_problem(probs, begins, nprobs, (long long)blockIdx.x);
+    prefetch_tmaps(probs + first_prob);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -604,11 +626,13 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
       uint32_t tph = 0;
       bool pending[8] = {false, false, false, false, false, false, false, false};
       uint32_t pend_ph[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      for (;;) {
-        const long long t = (long long)atomicAdd(counter, 1u);
+      for (bool first = true;; first = false) {
+        // entries 0 .. gridDim.x - 1 are dealt by index, the others through the counter
+        const long long t = first ? (long long)blockIdx.x
+                                  : (long long)gridDim.x + (long long)atomicAdd(counter, 1u);
         // the problem search is done here once per entry; the MMA and epilogue warps take
         // its result from shared memory
-        const int pi = t < total ? find_problem(probs, begins, nprobs, t) : 0;
+        const int pi = first ? first_prob : t < total ? find_problem(probs, begins, nprobs, t) : 0;
         TileInfo ti{};
         if (t < total) {
           ti = decode_tile(probs, pi, t, NT);
@@ -616,7 +640,8 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
             // a tile without work is not handed on; where it starts a run of them (the
             // columns of a V row group right of the diagonal), the queue moves past the run
             const long long run_end = skipped_run_end(ti, t, NT);
-            if (run_end > t + 1) atomicMax(counter, (unsigned)min(run_end, total));
+            if (run_end > t + 1 && min(run_end, total) > (long long)gridDim.x)
+              atomicMax(counter, (unsigned)(min(run_end, total) - (long long)gridDim.x));
             continue;
           }
         }
@@ -853,13 +878,11 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
       const SplitProb* P = ti.P;
       const int m = ti.tm * SG_BM + row;
       unsigned emax = 0;
-      if (m < P->M) {
+      if (P->kind == PK_V && m < P->M) {
         const int nbase = ti.tn * NT + c0;
         const char* wsb = (const char*)bs.ws;
-        const int* EA = (const int*)(wsb + P->ea_off);
-        const int* EB = (const int*)(wsb + P->eb_off);
-        const int ea = (P->kind == PK_V ? ea_pre : (P->ea_rows ? EA[m] : EA[0])) + P->ea_add;
-        if (P->kind == PK_V) {
+        const int ea = ea_pre + P->ea_add;
+        {
           float* Th = (float*)(wsb + P->c_off);
           float* Tl = (float*)(wsb + P->c2_off);
           const float2 dm = dm_pre;
@@ -944,28 +967,48 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
               }
             }
           }
-        } else {
-          double* C = (P->kind == PK_GAMMA || P->kind == PK_RAW) ? bs.gamma
-                      : P->kind == PK_PAB ? bs.pab : bs.pij;
-          C += P->c_off;
+        }
+      }
+      if (P->kind != PK_V) {
+        // Groups of four columns, transposed over four lanes: a store or addition of the warp
+        // then covers whole 32-byte sectors of eight rows instead of 8 bytes of 32 rows (the
+        // additions of a 128 x 80 tile took 10 us that way)
+        const char* wsb = (const char*)bs.ws;
+        const int* EA = (const int*)(wsb + P->ea_off);
+        const int* EB = (const int*)(wsb + P->eb_off);
+        double* C = (P->kind == PK_GAMMA || P->kind == PK_RAW) ? bs.gamma
+                    : P->kind == PK_PAB ? bs.pab : bs.pij;
+        C += P->c_off;
+        const float sg = (float)P->alpha;   // +1 or -1: applied to the two parts, exactly
+        const int mq = m - (lane & 3);
+        const bool plain = (P->kind == PK_GAMMA || P->kind == PK_RAW) && P->ksplit == 1;
+        const int ea0 = (P->ea_rows ? 0 : EA[0]) + P->ea_add + P->eb_add - 2 * LB;
 #pragma unroll
-          for (int c = 0; c < NC; ++c) {
-            const int n = nbase + c;
-            if (n >= P->N) continue;
-            const int e = ea + (P->eb_rows ? EB[n] : EB[0]) + P->eb_add - 2 * LB;
-            // alpha is +1 or -1: applied to the two parts, exactly
-            const float sg = (float)P->alpha;
-            const double val = df_scaled(sg * acc_h[c], sg * acc_l[c], e);
-            if ((P->kind == PK_GAMMA || P->kind == PK_RAW) && P->ksplit == 1) {
-              C[(long long)m * P->ldc + n] = val;
+        for (int g = 0; g < NC / 4; ++g) {
+          float h[4], l[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) { h[c] = acc_h[4 * g + c]; l[c] = acc_l[4 * g + c]; }
+          quad_transpose(h, lane);
+          quad_transpose(l, lane);
+          const int n = ti.tn * NT + c0 + 4 * g + (lane & 3);
+          if (n >= P->N) continue;
+          const int en = ea0 + (P->eb_rows ? EB[n] : EB[0]);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int mk = mq + k;
+            if (mk >= P->M) continue;
+            const double val = df_scaled(sg * h[k], sg * l[k], en + (P->ea_rows ? EA[mk] : 0));
+            double* p = C + (long long)mk * P->ldc + n;
+            if (plain) {
+              *p = val;
             } else if (P->sym) {
               // each unordered pair once: (m,n) and its mirror for m < n, the diagonal once;
               // m > n is covered by the mirror of a computed tile
-              if (m > n) continue;
-              atomicAdd(C + (long long)m * P->ldc + n, val);
-              if (m < n) atomicAdd(C + (long long)n * P->ldc + m, val);
+              if (mk > n) continue;
+              atomicAdd(p, val);
+              if (mk < n) atomicAdd(C + (long long)n * P->ldc + mk, val);
             } else {
-              atomicAdd(C + (long long)m * P->ldc + n, val);
+              atomicAdd(p, val);
             }
           }
         }
@@ -1050,6 +1093,7 @@ k_split_stack(const SplitProb* __restrict__ probs, const long long* __restrict__
   float2* red = (float2*)(smem + (size_t)stages * stage_bytes + 512);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int first_prob = 0;
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) {
       mbar_init(full + s, 1);
@@ -1067,6 +1111,9 @@ k_split_stack(const SplitProb* __restrict__ probs, const long long* __restrict__
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    // the CTA's first entry is its own index: found, and its tensor maps fetched, meanwhile
+    first_prob = find_problem(probs, begins, nprobs, (long long)blockIdx.x);
+    prefetch_tmaps(probs + first_prob);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -1094,9 +1141,10 @@ k_split_stack(const SplitProb* __restrict__ probs, const long long* __restrict__
       int tslot = 0;
       bool pending[8] = {false, false, false, false, false, false, false, false};
       uint32_t pend_ph[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      for (;;) {
-        const long long t = (long long)atomicAdd(counter, 1u);
-        const int pi = t < total ? find_problem(probs, begins, nprobs, t) : 0;
+      for (bool first = true;; first = false) {
+        const long long t = first ? (long long)blockIdx.x
+                                  : (long long)gridDim.x + (long long)atomicAdd(counter, 1u);
+        const int pi = first ? first_prob : t < total ? find_problem(probs, begins, nprobs, t) : 0;
         if (!mbar_wait(tile_empty + tslot, tph ^ 1u, abort_flag)) break;
         tile_idx[tslot] = t;
         tile_prob[tslot] = pi;

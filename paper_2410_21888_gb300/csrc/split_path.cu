@@ -1,19 +1,19 @@
 // Split-precision path of the RI-MP2 hot path (precision RIMP2_BF16_SPLIT).
 //
 // Per wave of fragments:
-//   1. k_split_reset   per-fragment exponent slots
-//   2. k_slice_b1      B -> balanced base-512 digits with one scale per row (i,a): the
-//                      operands of V (Eq. MP2_ints); also d_m = e_i - e_a per row
-//   3. k_bcol_max      max over (j,b) of |B^Q_jb| for every aux index Q
-//   4. k_slice_b2      B -> digits with one scale per aux index Q, transposed to
-//                      [Q][(j,b)]: the B operand of Gamma
-//   5. split GEMM      V on the tensor cores, epilogue T = V / D kept as a double-float
-//                      pair of planes, max |T| exponent
-//   6. k_amp_split     Tt = 2T - T^T, pair energies e_ij (FP64 per pair), digits of Tt and
-//                      T with one scale per fragment
-//   7. energy reduce   FP64 compensated cross-pair sum (shared with the FP64 path)
-//   8. zero P, split GEMMs for P_ab and P_ij, then for Gamma (Appendix Gamma, D^MP2_ab,
-//      D^MP2_ij); Gamma contracts the leading s_g digit planes of Tt
+//   1. k_split_prologue  counters and maxima slots, check of the orbital energies
+//   2. k_slice_b1        B -> balanced base-512 digits with one scale per row (i,a): the
+//                        operands of V (Eq. MP2_ints); d_m = e_i - e_a per row, check of B;
+//                        other CTAs of the launch: max over (j,b) of |B^Q_jb| per aux index Q
+//   3. k_slice_b2        B -> digits with one scale per aux index Q, transposed to
+//                        [Q][(j,b)]: the B operand of Gamma
+//   4. split GEMM        V on the tensor cores, epilogue T = V / D kept as a double-float
+//                        pair of planes, max |T| exponent
+//   5. k_amp_split       Tt = 2T - T^T, digits of Tt and T with one scale per fragment, pair
+//                        energies e_ij and the FP64 compensated cross-pair sums, zeroes P
+//   6. split GEMMs for P_ab and P_ij (128 x 64 tiles, or slice-stacked for small extents),
+//      then for Gamma (Appendix Gamma, D^MP2_ab, D^MP2_ij); Gamma contracts the leading s_g
+//      digit planes of Tt
 #include <climits>
 #include <cmath>
 #include <cstring>
@@ -22,6 +22,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
+#include "energy.cuh"
 #include "split_path.cuh"
 
 namespace rimp2 {
@@ -38,6 +39,8 @@ constexpr long long kMinPieceK = 4096;
 // nocc=100 nvir=500 naux=1500 (K = 51200): the Gamma/P launch takes 144.7 ms with slabs
 // of 2048, 140.5 with 4096, 138.0 with 8192, 136.5 with 16384 and 138.5 without slabs.
 constexpr long long kGammaSlabK = 16384;
+// rows of B per CTA of the column maxima (eight loads in flight a lane)
+constexpr int kColRows = 256;
 int rup(int x, int m) { return (x + m - 1) / m * m; }
 
 }  // namespace
@@ -255,16 +258,64 @@ __device__ __forceinline__ void pow2_factors(int e, float& s1, float& s2) {
 
 // ------------------------------------------------------------------ kernels
 
-// One CTA per fragment: the atomicMax targets (max |T| exponent, column maxima of |B|)
-__global__ void k_split_reset(const SplitFragDev* __restrict__ f, int n, Bases bs) {
+// One CTA per fragment: the slots later kernels count or take maxima in (max |T| exponent,
+// column maxima of |B|, amplitude CTA counters), the wave's work-queue counters, the check of
+// the orbital energies (finite, max(eps_occ) < min(eps_vir), so that every denominator is
+// negative; B is checked where it is sliced), and the energies and P_ab of a fragment without
+// occupied orbitals, which has no amplitude CTAs.
+__global__ void __launch_bounds__(256)
+k_split_prologue(const SplitFragDev* __restrict__ f, unsigned* ctr, int check, Bases bs) {
   const SplitFragDev& F = f[blockIdx.x];
   char* ws = (char*)bs.ws;
-  if (threadIdx.x == 0) ((unsigned*)(ws + F.scal))[1] = 0u;
-  for (int i = threadIdx.x; i < F.o; i += blockDim.x) ((unsigned*)(ws + F.ecnt))[i] = 0u;
+  if (blockIdx.x == 0 && threadIdx.x < 8) ctr[threadIdx.x] = 0u;
+  if (threadIdx.x == 0) {
+    ((unsigned*)(ws + F.scal))[1] = 0u;
+    if (F.o == 0) {
+      bs.energy[F.idx] = 0.0;
+      if (bs.energy_os) bs.energy_os[F.idx] = 0.0;
+      if (bs.energy_scs) bs.energy_scs[F.idx] = 0.0;
+    }
+  }
+  if (F.o == 0 && F.pab_off >= 0)
+    for (long long e = threadIdx.x; e < (long long)F.v * F.v; e += blockDim.x) bs.pab[F.pab_off + e] = 0.0;
+  for (int i = threadIdx.x; i <= F.o; i += blockDim.x) ((unsigned*)(ws + F.ecnt))[i] = 0u;
   if (F.sg_out > 0) {
     unsigned long long* cm = (unsigned long long*)(ws + F.ecolm);
     for (int q = threadIdx.x; q < F.X; q += blockDim.x) cm[q] = 0ull;
   }
+  if (!check) return;
+  // order-preserving keys of the energies (comparisons on the integer pipes; both zeros get
+  // the same one)
+  auto key = [](double x) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x), top = 1ull << 63;
+    return u & top ? (u == top ? top : ~u) : u | top;
+  };
+  auto is_nan = [](double x) { return abs_bits(x) > 0x7FF0000000000000ull; };
+  __shared__ unsigned long long smax[8], smin[8];
+  bool bad = false;
+  unsigned long long mx = 0ull, mn = ~0ull;
+  for (int e = threadIdx.x; e < F.o; e += blockDim.x) {
+    const double x = bs.eps[F.eo_off + e];
+    bad |= !finite_bits(x);
+    if (!is_nan(x)) mx = max(mx, key(x));
+  }
+  for (int e = threadIdx.x; e < F.v; e += blockDim.x) {
+    const double x = bs.eps[F.ev_off + e];
+    bad |= !finite_bits(x);
+    if (!is_nan(x)) mn = min(mn, key(x));
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, off));
+  }
+  if ((threadIdx.x & 31) == 0) { smax[threadIdx.x >> 5] = mx; smin[threadIdx.x >> 5] = mn; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) { mx = max(mx, smax[w]); mn = min(mn, smin[w]); }
+    if (F.o > 0 && F.v > 0 && !(mx < mn)) atomicOr(bs.status, ST_DENOM);
+  }
+  if (bad) atomicOr(bs.status, ST_NONFINITE);
 }
 
 // One warp per row (i,a) of B: row exponent, digits of the V operand, d_m and the diagonal
@@ -273,12 +324,10 @@ __global__ void k_split_reset(const SplitFragDev* __restrict__ f, int n, Bases b
 // the middle digit, an error of one sign that does not average out; the epilogue takes
 // this FP64 value instead.
 template <bool F8>
-__global__ void __launch_bounds__(256)
-k_slice_b1(const SplitFragDev* __restrict__ f, int nf, long long rows, int sv, Bases bs) {
+__device__ __forceinline__ void slice_row(const SplitFragDev* __restrict__ f, int nf, long long gr,
+                                          int sv, int check, const Bases& bs) {
   using DT = typename Digit<F8>::T;
-  const long long gr = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  if (gr >= rows) return;
   const SplitFragDev& F = f[find_sfd(f, nf, gr, 0)];
   const int r = (int)(gr - F.row_begin);
   const double* x = bs.B + F.b_off + (long long)r * F.X;
@@ -294,6 +343,8 @@ k_slice_b1(const SplitFragDev* __restrict__ f, int nf, long long rows, int sv, B
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     ss += __shfl_xor_sync(0xffffffffu, ss, off);
   }
+  // the largest |x| as bits is that of an infinity or a NaN where the row holds one
+  if (check && lane == 0 && mx >= 0x7FF0000000000000ull) atomicOr(bs.status, ST_NONFINITE);
   const int E = mx > 0 ? ilogb_bits(mx) + 2 + Digit<F8>::HEAD : -1000;
   char* ws = (char*)bs.ws;
   const long long plane = (long long)F.o * F.v * F.xpad;
@@ -330,19 +381,18 @@ k_slice_b1(const SplitFragDev* __restrict__ f, int nf, long long rows, int sv, B
 }
 
 // Column maxima of B for Gamma's B operand: max over rows (j,b) of |B^Q_jb| for every aux
-// index Q.  One CTA per 32 aux indices x 256 rows (lane: Q, warp: every 8th row), FP64
+// index Q.  One CTA per 32 aux indices x kColRows rows (lane: Q, warp: every 8th row), FP64
 // bits combined by atomicMax (non-negative doubles order like their bit patterns).
-__global__ void __launch_bounds__(256)
-k_bcol_max(const SplitFragDev* __restrict__ f, int nf, Bases bs) {
+__device__ __forceinline__ void column_maxima(const SplitFragDev* __restrict__ f, int nf, long long gb,
+                                              const Bases& bs) {
   __shared__ unsigned long long red[8][32];   // |B| maxima as bits
-  const long long gb = blockIdx.x;
   const SplitFragDev& F = f[find_sfd(f, nf, gb, 3)];
   const long long lb = gb - F.qblk_begin;
   const int nqb = (F.X + 31) / 32;
   const int qb = (int)(lb % nqb), rc = (int)(lb / nqb);
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int Q = qb * 32 + lane;
-  const int r0 = rc * 256, r1 = min(F.o * F.v, r0 + 256);
+  const int r0 = rc * kColRows, r1 = min(F.o * F.v, r0 + kColRows);
   unsigned long long mx = 0;
   if (Q < F.X) {
     const double* x = bs.B + F.b_off + Q;
@@ -354,6 +404,20 @@ k_bcol_max(const SplitFragDev* __restrict__ f, int nf, Bases bs) {
   if (g == 0) {
     for (int k = 1; k < 8; ++k) mx = max(mx, red[k][lane]);
     if (Q < F.X && mx > 0) atomicMax((unsigned long long*)((char*)bs.ws + F.ecolm) + Q, mx);
+  }
+}
+
+// Both passes over B in one launch: CTAs below row_blocks slice eight rows each, the others take
+// the column maxima
+template <bool F8>
+__global__ void __launch_bounds__(256)
+k_slice_b1(const SplitFragDev* __restrict__ f, int nf, long long rows, unsigned row_blocks, int sv,
+           int check, Bases bs) {
+  if (blockIdx.x < row_blocks) {
+    const long long gr = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (gr < rows) slice_row<F8>(f, nf, gr, sv, check, bs);
+  } else {
+    column_maxima(f, nf, (long long)(blockIdx.x - row_blocks), bs);
   }
 }
 
@@ -481,6 +545,15 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, Bases bs) {
   const int yq = 4 * (tid % (ROWS / 4)), yb = tid / (ROWS / 4);
 
   // the next step's direct and transposed elements; their offsets advance within a j block
+  // this CTA's share of the outputs that the contractions accumulate into
+  {
+    const long long ctas = (long long)strips * jranges * o, me = (long long)(blockIdx.x - F.pair_begin);
+    const long long no = F.pij_off >= 0 ? (long long)o * o : 0, nv = F.pab_off >= 0 ? (long long)v * v : 0;
+    const long long ng = F.zero_gamma ? (long long)o * v * F.X : 0;
+    for (long long e = me * 256 + tid; e < no; e += ctas * 256) bs.pij[F.pij_off + e] = 0.0;
+    for (long long e = me * 256 + tid; e < nv; e += ctas * 256) bs.pab[F.pab_off + e] = 0.0;
+    for (long long e = me * 256 + tid; e < ng; e += ctas * 256) __stcs(bs.gamma + F.gamma_off + e, 0.0);
+  }
   float4 dh, dl, xh, xl;
   long long id = 0, ix = 0;
   const long long xstep = (long long)C * ldt;
@@ -641,6 +714,15 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, Bases bs) {
       eq[(long long)jj * o + i] = eo;
     }
   }
+  // the last row's CTA sums the fragment's energies
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd((unsigned*)(ws + F.ecnt) + o, 1u) + 1u == (unsigned)o;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  fragment_energy(ep, ep + (long long)o * o, (long long)o * o,
+                  F.epair_off >= 0 ? bs.epair + F.epair_off : nullptr, F.idx, bs);
 }
 
 // ------------------------------------------------------------------ host
@@ -782,7 +864,7 @@ Layout frag_layout(const SplitPlan& sp, const rimp2_frag& f) {
   L.ecol = off; off += al256(X * 4);
   L.ep = off; off += al256(2 * o * o * 8);   // pair energies, opposite-spin pair energies
   L.epart = off; off += al256(o * o * 8 * ((v + 7) / 8) * 16);   // warps' shares, at most
-  L.ecnt = off; off += al256(o * 4);
+  L.ecnt = off; off += al256((o + 1) * 4);
   L.scal = off; off += 256;
   L.total = off;
   return L;
@@ -849,8 +931,7 @@ size_t split_frag_ws_bytes(const SplitPlan& sp, const rimp2_frag& f) {
 }
 
 int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<int>& members,
-                     const double* B, void* ws, std::vector<FragDev>& fdev, SplitWave& w,
-                     long long& total_pairs, long long& max_b) {
+                     const double* B, void* ws, SplitWave& w, long long& total_pairs) {
   (void)B;
   char* wsb = (char*)ws;
   size_t off = 0;
@@ -889,6 +970,7 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
     s.sg_out = g ? sgl : 0;
     s.st_out = std::max(s.st_t, s.sg_out);
     s.b_off = f.b_off; s.eo_off = f.eo_off; s.ev_off = f.ev_off;
+    s.gamma_off = f.gamma_off; s.pij_off = f.pij_off; s.pab_off = f.pab_off; s.epair_off = f.epair_off;
     s.bs1 = off + L.bs1; s.bs2 = off + L.bs2; s.erow = off + L.erow; s.drow = off + L.drow;
     s.vdrow = off + L.vdrow; s.dnh = off + L.dnh; s.dnl = off + L.dnl;
     s.thi = off + L.thi; s.tlo = off + L.tlo; s.tts = off + L.tts; s.ts = off + L.ts;
@@ -898,21 +980,10 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
     rows += ov;
     if (g) {
       b2t += (long long)((X + 31) / 32) * ((RL + 127) / 128);
-      qbl += (long long)((X + 31) / 32) * ((ov + 255) / 256);
+      qbl += (long long)((X + 31) / 32) * ((ov + kColRows - 1) / kColRows);
       w.want_gamma = true;
     }
     w.sfd.push_back(s);
-    // the shared FP64 kernels (checks, energy reduce, zeroing) use FragDev
-    FragDev d{};
-    d.o = o; d.v = v; d.X = X; d.idx = idx;
-    d.b_off = f.b_off; d.eo_off = f.eo_off; d.ev_off = f.ev_off;
-    d.t_off = d.tt_off = -1;
-    d.ep_off = (long long)(s.ep / 8);
-    d.epos_off = d.ep_off + (long long)o * o;
-    d.gamma_off = f.gamma_off; d.pij_off = f.pij_off; d.pab_off = f.pab_off;
-    d.epair_off = f.epair_off;
-    fdev.push_back(d);
-    max_b = std::max<long long>(max_b, (long long)ov * X);
     off += L.total;
     if (ov == 0) continue;
 
@@ -983,7 +1054,7 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
         slabs = (kb + per - 1) / per;
         P.k0_blocks = per; P.k1_count = slabs; P.ksplit = slabs;
         P.a_mode = P.b_mode = TM_3DK; P.div5 = per * BKg; P.ks_outer = 1;
-        fdev.back().zero_gamma = 1;
+        w.sfd.back().zero_gamma = 1;
       }
       // the leading s_g planes of Tt (one scale per fragment) and B with one scale per aux
       // index Q
@@ -1121,7 +1192,7 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
       P.k0_blocks = per;
       P.a_mode = P.b_mode = TM_3DK; P.div5 = per * BKg; P.ks_outer = 1;
       P.ntiles *= P.ksplit;
-      for (auto& d : fdev)
+      for (auto& d : w.sfd)
         if (d.idx == P.frag) d.zero_gamma = 1;
     }
   }
@@ -1211,25 +1282,21 @@ void split_fill_wave(const SplitWave& w, char* host) {
   begins(w.probs_s, w.off_bs);
 }
 
-int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, const FragDev* dfd, int nf,
-                       long long total_pairs, Bases bs, unsigned* ctr, cudaStream_t s,
-                       int* launches, long long* tiles, cudaEvent_t* ev) {
+int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long long total_pairs,
+                       Bases bs, int check, unsigned* ctr, cudaStream_t s, int* launches,
+                       long long* tiles, cudaEvent_t* ev) {
   const SplitFragDev* sfd = (const SplitFragDev*)(dblk + w.off_sfd);
   int nl = 0;
   cudaError_t e = cudaSuccess;
   if (nf > 0) {
-    k_split_reset<<<(unsigned)nf, 128, 0, s>>>(sfd, nf, bs);
+    k_split_prologue<<<(unsigned)nf, 256, 0, s>>>(sfd, ctr, check, bs);
     ++nl;
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && w.rows > 0) {
-    if (sp.fp8) k_slice_b1<true><<<(unsigned)((w.rows + 7) / 8), 256, 0, s>>>(sfd, nf, w.rows, sp.slices_v, bs);
-    else k_slice_b1<false><<<(unsigned)((w.rows + 7) / 8), 256, 0, s>>>(sfd, nf, w.rows, sp.slices_v, bs);
-    ++nl;
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess && w.qblks > 0) {
-    k_bcol_max<<<(unsigned)w.qblks, 256, 0, s>>>(sfd, nf, bs);
+    const unsigned rb = (unsigned)((w.rows + 7) / 8), blocks = rb + (unsigned)w.qblks;
+    if (sp.fp8) k_slice_b1<true><<<blocks, 256, 0, s>>>(sfd, nf, w.rows, rb, sp.slices_v, check, bs);
+    else k_slice_b1<false><<<blocks, 256, 0, s>>>(sfd, nf, w.rows, rb, sp.slices_v, check, bs);
     ++nl;
     e = cudaGetLastError();
   }
@@ -1259,8 +1326,6 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, const FragDev* d
     ++nl;
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) { e = launch_energy_reduce(dfd, nf, bs, s); ++nl; }
-  if (e == cudaSuccess) { e = launch_zero_p(dfd, nf, bs, s); ++nl; }
   if (ev) cudaEventRecordWithFlags(ev[3], s, cudaEventRecordExternal);
   if (e == cudaSuccess && w.tiles_c > 0) {
     SplitLaunch cfg = sp.cfg_t;

@@ -34,7 +34,9 @@ struct SplitFragDev {
   long long pair_begin;   // first amplitude CTA of the fragment
   int amp_jchunk, pad3;   // j blocks per amplitude CTA
   long long epart;  // float4 [o][o][..]: the amplitude warps' shares of e_ij and its os part
-  long long ecnt;   // uint32 [o]: amplitude CTAs done per i
+  long long ecnt;   // uint32 [o + 1]: amplitude CTAs done per i, then rows i done
+  long long gamma_off, pij_off, pab_off, epair_off;   // into the caller's pools, or -1
+  int zero_gamma, pad4;   // 1: Gamma is accumulated by atomics, the amplitude stage zeroes it
   long long row_begin, b2_tile_begin;
   long long qblk_begin;   // first block (32 Q x 256 rows) of the fragment in the column maxima pass
   int sg_out, pad2;       // slices of Gamma's operands (0: no Gamma)
@@ -84,12 +86,12 @@ int split_plan_init(SplitPlan& sp, int precision, const rimp2_options& opt);
 void split_plan_release(SplitPlan& sp);
 size_t split_frag_ws_bytes(const SplitPlan& sp, const rimp2_frag& f);
 int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<int>& members,
-                     const double* B, void* ws, std::vector<FragDev>& fdev, SplitWave& w,
-                     long long& total_pairs, long long& max_b);
+                     const double* B, void* ws, SplitWave& w, long long& total_pairs);
 size_t split_layout_wave(SplitWave& w, size_t off);
 void split_fill_wave(const SplitWave& w, char* host_block);
-int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, const FragDev* dfd, int nf,
-                       long long total_pairs, Bases bs, unsigned* ctr, cudaStream_t s,
-                       int* launches, long long* tiles, cudaEvent_t* ev);
+// check: 1 for the checks of B and the orbital energies
+int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long long total_pairs,
+                       Bases bs, int check, unsigned* ctr, cudaStream_t s, int* launches,
+                       long long* tiles, cudaEvent_t* ev);
 
 }  // namespace rimp2
