@@ -42,12 +42,24 @@ __device__ __forceinline__ int ilogb_bits(unsigned long long b) {
 // rounding and scaled by a power of two gives l.  Bit-identical to the two conversions
 // wherever h and any non-zero l are normal floats (|x| in [2^-74, 2^127)); other inputs,
 // far from anything this library sees, take the FP64 conversions.
+// (That path is a call: inlined, the compiler executes its four FP64 instructions for every
+// element and selects, which bounds the slicing kernels by the FP64 unit.)
+static __device__ __noinline__ float2 split_to_df_fp64(double x) {
+  const float h = (float)x;
+  return make_float2(h, (float)(x - (double)h));
+}
 __device__ __forceinline__ void split_to_df(double x, float& h, float& l) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
   const int e = (int)((u >> 52) & 0x7FFu);
-  if (e < 949 || e > 1149) {
-    h = (float)x;
-    l = (float)(x - (double)h);
+  if (__builtin_expect(e < 949 || e > 1149, 0)) {
+    if ((u << 1) == 0ull) {   // zeros are ordinary: padding, absent blocks
+      h = __uint_as_float((unsigned)(u >> 32));
+      l = 0.0f;
+      return;
+    }
+    const float2 d = split_to_df_fp64(x);
+    h = d.x;
+    l = d.y;
     return;
   }
   const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;

@@ -63,9 +63,12 @@ __device__ __forceinline__ dfl d_add(dfl a, dfl b) {
   s.l += a.l + b.l;
   return d_fast(s.h, s.l);
 }
+// (split on the integer pipes: a conversion occupies the SM's FP64 unit for 16 clocks a warp,
+// however few lanes need it)
 __device__ __forceinline__ dfl d_from(double x) {
-  const float h = (float)x;
-  return {h, (float)(x - (double)h)};
+  dfl d;
+  split_to_df(x, d.h, d.l);
+  return d;
 }
 
 __device__ __forceinline__ int find_sfd(const SplitFragDev* __restrict__ f, int n, long long t,
@@ -323,20 +326,52 @@ k_split_prologue(const SplitFragDev* __restrict__ f, unsigned* ctr, int check, B
 // digits: there the truncated triangle's first dropped even level holds the square of
 // the middle digit, an error of one sign that does not average out; the epilogue takes
 // this FP64 value instead.
-template <bool F8>
+// NCH > 0: the row has at most 128 NCH elements and stays in registers between the maximum
+// and the slicing, all its loads in flight at once (four consecutive elements a lane and
+// chunk); 0: longer rows are read twice (the second time from L1; registers for 512 or more
+// elements cost the occupancy that hides the FP64 sum of squares).  16 trimers (574 MB of B,
+// 8 slices): 461 us plus 82 for a separate check of B before, now 400.
+template <bool F8, int NCH>
 __device__ __forceinline__ void slice_row(const SplitFragDev* __restrict__ f, int nf, long long gr,
                                           int sv, int check, const Bases& bs) {
   using DT = typename Digit<F8>::T;
   const int lane = threadIdx.x & 31;
   const SplitFragDev& F = f[find_sfd(f, nf, gr, 0)];
-  const int r = (int)(gr - F.row_begin);
-  const double* x = bs.B + F.b_off + (long long)r * F.X;
+  const int r = (int)(gr - F.row_begin), X = F.X;
+  const double* x = bs.B + F.b_off + (long long)r * X;
+  const bool al = ((uintptr_t)x & 15) == 0;   // rows of odd length start on 8-byte boundaries
+  auto load4 = [&](int q0, double (&v)[4]) {
+    if (al && q0 + 4 <= X) {
+      const double2 a = *(const double2*)(x + q0), b = *(const double2*)(x + q0 + 2);
+      v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = q0 + k < X ? x[q0 + k] : 0.0;
+    }
+  };
   unsigned long long mx = 0;   // max |x| as bits
   double ss = 0.0;
-  for (int q = lane; q < F.X; q += 32) {
-    const double xq = x[q];
-    mx = max(mx, abs_bits(xq));
-    ss = fma(xq, xq, ss);
+  auto look = [&](const double (&v)[4]) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      mx = max(mx, abs_bits(v[k]));
+      ss = fma(v[k], v[k], ss);
+    }
+  };
+  double row[NCH > 0 ? NCH : 1][4];
+  if constexpr (NCH > 0) {
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) load4(4 * lane + 128 * c, row[c]);
+#pragma unroll
+    for (int c = 0; c < NCH; ++c)
+      if (128 * c < X) look(row[c]);
+  } else {
+#pragma unroll 4
+    for (int q0 = 4 * lane; q0 < X; q0 += 128) {
+      double v[4];
+      load4(q0, v);
+      look(v);
+    }
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
@@ -351,32 +386,43 @@ __device__ __forceinline__ void slice_row(const SplitFragDev* __restrict__ f, in
   DT* out = (DT*)(ws + F.bs1) + (long long)r * F.xpad;
   float s1, s2;
   pow2_factors(Digit<F8>::LB - E, s1, s2);
-  // four consecutive elements a lane, one packed store per plane (elements in [X, xpad)
-  // get zero digits; the V operand's tensor map ends at X)
-  for (int q0 = 4 * lane; q0 < F.X; q0 += 128) {
+  // one packed store per plane (elements in [X, xpad) get zero digits; the V operand's tensor
+  // map ends at X)
+  auto slice4 = [&](int q0, const double (&v)[4]) {
     dfl xs[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       float h, l;
-      split_to_df(q0 + k < F.X ? x[q0 + k] : 0.0, h, l);
+      split_to_df(v[k], h, l);
       xs[k] = {(h * s1) * s2, (l * s1) * s2};
     }
     put4<F8>(xs, sv, out + q0, plane);
+  };
+  if constexpr (NCH > 0) {
+#pragma unroll
+    for (int c = 0; c < NCH; ++c)
+      if (4 * lane + 128 * c < X) slice4(4 * lane + 128 * c, row[c]);
+  } else {
+    for (int q0 = 4 * lane; q0 < X; q0 += 128) {
+      double v[4];
+      load4(q0, v);
+      slice4(q0, v);
+    }
   }
+  const int i = r / F.v, a = r - i * F.v;
   if (lane == 0) {
     ((int*)(ws + F.erow))[r] = E;
-    const int i = r / F.v, a = r - i * F.v;
     const dfl d = d_from(bs.eps[F.eo_off + i] - bs.eps[F.ev_off + a]);
     ((float2*)(ws + F.drow))[r] = make_float2(d.h, d.l);
     // the same terms by padded j blocks for the amplitude kernel's 16-byte loads
-    float* dnh = (float*)(ws + F.dnh) + (long long)i * F.vpadt;
-    float* dnl = (float*)(ws + F.dnl) + (long long)i * F.vpadt;
-    dnh[a] = d.h;
-    dnl[a] = d.l;
-    if (a == F.v - 1)
-      for (int k = F.v; k < F.vpadt; ++k) dnh[k] = dnl[k] = 0.f;
+    ((float*)(ws + F.dnh))[(long long)i * F.vpadt + a] = d.h;
+    ((float*)(ws + F.dnl))[(long long)i * F.vpadt + a] = d.l;
     const dfl vd = d_from(ss);
     ((float2*)(ws + F.vdrow))[r] = make_float2(vd.h, vd.l);
+  }
+  if (a == F.v - 1 && F.v + lane < F.vpadt) {
+    ((float*)(ws + F.dnh))[(long long)i * F.vpadt + F.v + lane] = 0.f;
+    ((float*)(ws + F.dnl))[(long long)i * F.vpadt + F.v + lane] = 0.f;
   }
 }
 
@@ -409,13 +455,13 @@ __device__ __forceinline__ void column_maxima(const SplitFragDev* __restrict__ f
 
 // Both passes over B in one launch: CTAs below row_blocks slice eight rows each, the others take
 // the column maxima
-template <bool F8>
-__global__ void __launch_bounds__(256)
+template <bool F8, int NCH>
+__global__ void __launch_bounds__(256, 6)
 k_slice_b1(const SplitFragDev* __restrict__ f, int nf, long long rows, unsigned row_blocks, int sv,
            int check, Bases bs) {
   if (blockIdx.x < row_blocks) {
     const long long gr = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (gr < rows) slice_row<F8>(f, nf, gr, sv, check, bs);
+    if (gr < rows) slice_row<F8, NCH>(f, nf, gr, sv, check, bs);
   } else {
     column_maxima(f, nf, (long long)(blockIdx.x - row_blocks), bs);
   }
@@ -423,13 +469,16 @@ k_slice_b1(const SplitFragDev* __restrict__ f, int nf, long long rows, unsigned 
 
 // Gamma's B operand: Bs2[p][Q][c], c = j*vpad + b (zero for b >= nvir), one scale
 // 2^E_Q per aux index, E_Q = ilogb(max_(j,b) |B^Q_jb|) + 2 + HEAD (also stored for the GEMM
-// epilogue).  Tiles of 32 aux indices x 128 columns c transposed through shared memory;
-// each thread then writes four consecutive c of one Q, one packed store per plane.
+// epilogue).  Tiles of 32 aux indices x 128 columns c, loaded with every element in flight and
+// transposed through shared memory; each thread then writes four consecutive c of one Q, one
+// packed store per plane, the lanes of a row covering whole 128-byte lines.
 template <bool F8>
 __global__ void __launch_bounds__(256)
 k_slice_b2(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
   using DT = typename Digit<F8>::T;
-  __shared__ double tile[128][33];
+  constexpr int LPR = F8 ? 32 : 16;   // lanes of a row: 128 bytes of digits
+  constexpr int LDC = 130;            // 16-byte rows
+  __shared__ __align__(16) double tile[32][LDC];
   const long long gt = blockIdx.x;
   const SplitFragDev& F = f[find_sfd(f, nf, gt, 1)];
   const long long lt = gt - F.b2_tile_begin;
@@ -437,15 +486,20 @@ k_slice_b2(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
   const int ntc = (RL + 127) / 128;
   const int tq = (int)(lt / ntc), tc = (int)(lt % ntc);
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const double* B = bs.B + F.b_off;
-  for (int r = ty; r < 128; r += 8) {
-    const int c = tc * 128 + r, Q = tq * 32 + tx;
-    double val = 0.0;
-    if (c < RL && Q < F.X) {
-      const int j = c / F.vpad, b = c - j * F.vpad;
-      if (b < F.v) val = B[((long long)j * F.v + b) * F.X + Q];
+  {
+    const int Q = tq * 32 + tx;
+    const double* B = bs.B + F.b_off + Q;
+    int c = tc * 128 + ty, j = c / F.vpad, b = c - j * F.vpad;
+    double val[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      val[k] = c < RL && b < F.v && Q < F.X ? B[((long long)j * F.v + b) * F.X] : 0.0;
+      c += 8;
+      b += 8;
+      if (b >= F.vpad) { b -= F.vpad; ++j; }   // vpad is a multiple of 8
     }
-    tile[r][tx] = val;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) tile[tx][ty + 8 * k] = val[k];
   }
   __syncthreads();
   char* ws = (char*)bs.ws;
@@ -453,25 +507,30 @@ k_slice_b2(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
   int* ec = (int*)(ws + F.ecol);
   const long long plane = (long long)F.X * F.ldd;
   DT* out = (DT*)(ws + F.bs2);
-  const int qi = threadIdx.x >> 3, cg = threadIdx.x & 7;
-  const int Q = tq * 32 + qi;
-  if (Q >= F.X) return;
-  const int E = cm[Q] > 0 ? ilogb_bits(cm[Q]) + 2 + Digit<F8>::HEAD : -1000;
-  if (tc == 0 && cg == 0) ec[Q] = E;
-  float s1, s2;
-  pow2_factors(Digit<F8>::LB - E, s1, s2);
+  const int cl0 = 4 * (tx % LPR);
+#pragma unroll 1
+  for (int qi = ty * (32 / LPR) + tx / LPR; qi < 32; qi += 8 * (32 / LPR)) {
+    const int Q = tq * 32 + qi;
+    if (Q >= F.X) break;
+    const int E = cm[Q] > 0 ? ilogb_bits(cm[Q]) + 2 + Digit<F8>::HEAD : -1000;
+    if (tc == 0 && cl0 == 0) ec[Q] = E;
+    float s1, s2;
+    pow2_factors(Digit<F8>::LB - E, s1, s2);
 #pragma unroll
-  for (int k4 = 0; k4 < 4; ++k4) {
-    const int cl = k4 * 32 + cg * 4, c = tc * 128 + cl;   // RL is a multiple of 4
-    if (c >= RL) break;
-    dfl xs[4];
+    for (int cl = cl0; cl < 128; cl += 4 * LPR) {
+      const int c = tc * 128 + cl;   // RL is a multiple of 4
+      if (c >= RL) break;
+      const double2 u = *(const double2*)&tile[qi][cl], w = *(const double2*)&tile[qi][cl + 2];
+      const double v4[4] = {u.x, u.y, w.x, w.y};
+      dfl xs[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      float h, l;
-      split_to_df(tile[cl + k][qi], h, l);
-      xs[k] = {(h * s1) * s2, (l * s1) * s2};
+      for (int k = 0; k < 4; ++k) {
+        float h, l;
+        split_to_df(v4[k], h, l);
+        xs[k] = {(h * s1) * s2, (l * s1) * s2};
+      }
+      put4<F8>(xs, st, out + (long long)Q * F.ldd + c, plane);
     }
-    put4<F8>(xs, st, out + (long long)Q * F.ldd + c, plane);
   }
 }
 
@@ -1201,9 +1260,9 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
   // share (MBE3 stated batch: dimer level 86.1 -> 79.3 ms); with naux ~1500 the extra
   // warps cost V's MMA issuer a little (41.6 -> 42.2 ms at nocc=100 nvir=500).
   {
-    int max_x = 0;
-    for (const auto& s : w.sfd) max_x = std::max(max_x, s.X);
-    w.epi_warps = max_x <= 1024 ? 16 : 8;
+    w.max_x = 0;
+    for (const auto& s : w.sfd) w.max_x = std::max(w.max_x, s.X);
+    w.epi_warps = w.max_x <= 1024 ? 16 : 8;
   }
   // Amplitude stage: CTAs (i, j range, strip).  One range of all j where the strips alone make
   // eight rounds of three CTAs per SM (a shorter last round costs less of the whole); shorter
@@ -1295,8 +1354,9 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long lon
   }
   if (e == cudaSuccess && w.rows > 0) {
     const unsigned rb = (unsigned)((w.rows + 7) / 8), blocks = rb + (unsigned)w.qblks;
-    if (sp.fp8) k_slice_b1<true><<<blocks, 256, 0, s>>>(sfd, nf, w.rows, rb, sp.slices_v, check, bs);
-    else k_slice_b1<false><<<blocks, 256, 0, s>>>(sfd, nf, w.rows, rb, sp.slices_v, check, bs);
+    auto b1 = [&](auto kernel) { kernel<<<blocks, 256, 0, s>>>(sfd, nf, w.rows, rb, sp.slices_v, check, bs); };
+    if (w.max_x <= 256) sp.fp8 ? b1(k_slice_b1<true, 2>) : b1(k_slice_b1<false, 2>);
+    else sp.fp8 ? b1(k_slice_b1<true, 0>) : b1(k_slice_b1<false, 0>);
     ++nl;
     e = cudaGetLastError();
   }

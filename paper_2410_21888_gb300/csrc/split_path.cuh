@@ -74,6 +74,7 @@ struct SplitWave {
   std::vector<SplitProb> probs_s;   // P_ab / P_ij of small extents (slice-stacked kernel)
   long long tiles_v = 0, tiles_c = 0, tiles_g = 0, tiles_s = 0, rows = 0, b2_tiles = 0, qblks = 0;
   bool want_gamma = false;
+  int max_x = 0;       // largest naux of the wave
   int amp_lpr = 32;    // lanes per row of the amplitude kernel
   int epi_warps = 8;   // epilogue warps of the wave's contraction launches (see build)
   double mma_v = 0, mma_c = 0, mma_g = 0;   // tensor-core FLOPs issued per launch
