@@ -38,13 +38,18 @@ __device__ __forceinline__ void fragment_energy(const double* ep, const double* 
   }
   if (lane == 0) { sh[warp][0] = s; sh[warp][1] = c; sh[warp][2] = so; sh[warp][3] = co; }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  for (int w = 1; w < 8; ++w) {
-    comp_add(s, c, sh[w][0]);
-    comp_add(so, co, sh[w][2]);
-    c += sh[w][1];
-    co += sh[w][3];
+  if (warp != 0) return;
+  s = sh[lane & 7][0]; c = sh[lane & 7][1]; so = sh[lane & 7][2]; co = sh[lane & 7][3];
+#pragma unroll
+  for (int off = 4; off > 0; off >>= 1) {
+    const double a = __shfl_xor_sync(0xffffffffu, s, off), b = __shfl_xor_sync(0xffffffffu, c, off);
+    const double ao = __shfl_xor_sync(0xffffffffu, so, off), bo = __shfl_xor_sync(0xffffffffu, co, off);
+    comp_add(s, c, a);
+    comp_add(so, co, ao);
+    c += b;
+    co += bo;
   }
+  if (lane != 0) return;
   const double e = s + c;
   bs.energy[idx] = e;
   if (!epos) return;

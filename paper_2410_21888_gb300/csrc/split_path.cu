@@ -5,13 +5,13 @@
 //   2. k_slice_b1        B -> balanced base-512 digits with one scale per row (i,a): the
 //                        operands of V (Eq. MP2_ints); d_m = e_i - e_a per row, check of B;
 //                        other CTAs of the launch: max over (j,b) of |B^Q_jb| per aux index Q
-//   3. k_slice_b2        B -> digits with one scale per aux index Q, transposed to
-//                        [Q][(j,b)]: the B operand of Gamma
-//   4. split GEMM        V on the tensor cores, epilogue T = V / D kept as a double-float
+//   3. split GEMM        V on the tensor cores, epilogue T = V / D kept as a double-float
 //                        pair of planes, max |T| exponent
-//   5. k_amp_split       Tt = 2T - T^T, digits of Tt and T with one scale per fragment, pair
-//                        energies e_ij and the FP64 compensated cross-pair sums, zeroes P
-//   6. split GEMMs for P_ab and P_ij (128 x 64 tiles, or slice-stacked for small extents),
+//   4. k_amp_split       Tt = 2T - T^T, digits of Tt and T with one scale per fragment, pair
+//                        energies e_ij and the FP64 compensated cross-pair sums, zeroes P;
+//                        other CTAs of the launch: B -> digits with one scale per aux index
+//                        Q, transposed to [Q][(j,b)], the B operand of Gamma
+//   5. split GEMMs for P_ab and P_ij (128 x 64 tiles, or slice-stacked for small extents),
 //      then for Gamma (Appendix Gamma, D^MP2_ab, D^MP2_ij); Gamma contracts the leading s_g
 //      digit planes of Tt
 #include <climits>
@@ -469,37 +469,36 @@ k_slice_b1(const SplitFragDev* __restrict__ f, int nf, long long rows, unsigned 
 
 // Gamma's B operand: Bs2[p][Q][c], c = j*vpad + b (zero for b >= nvir), one scale
 // 2^E_Q per aux index, E_Q = ilogb(max_(j,b) |B^Q_jb|) + 2 + HEAD (also stored for the GEMM
-// epilogue).  Tiles of 32 aux indices x 128 columns c, loaded with every element in flight and
-// transposed through shared memory; each thread then writes four consecutive c of one Q, one
-// packed store per plane, the lanes of a row covering whole 128-byte lines.
+// epilogue).  Tiles of B2Q aux indices x B2C columns c (128 bytes of digits), loaded with
+// every element in flight and transposed through shared memory; each thread then writes four
+// consecutive c of one Q, one packed store per plane, the lanes of a row covering whole lines.
+template <bool F8> constexpr int B2Q = F8 ? 16 : 32;
+template <bool F8> constexpr int B2C = F8 ? 128 : 64;
+
 template <bool F8>
-__global__ void __launch_bounds__(256)
-k_slice_b2(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
+__device__ __forceinline__ void slice_b2(const SplitFragDev* __restrict__ f, int nf, long long gt, int st,
+                                         double (*tile)[B2C<F8> + 2], const Bases& bs) {
   using DT = typename Digit<F8>::T;
-  constexpr int LPR = F8 ? 32 : 16;   // lanes of a row: 128 bytes of digits
-  constexpr int LDC = 130;            // 16-byte rows
-  __shared__ __align__(16) double tile[32][LDC];
-  const long long gt = blockIdx.x;
+  constexpr int NQ = B2Q<F8>, NC = B2C<F8>, RS = 256 / NQ;   // RS: columns c per load pass
   const SplitFragDev& F = f[find_sfd(f, nf, gt, 1)];
   const long long lt = gt - F.b2_tile_begin;
   const int RL = F.o * F.vpad;
-  const int ntc = (RL + 127) / 128;
+  const int ntc = (RL + NC - 1) / NC;
   const int tq = (int)(lt / ntc), tc = (int)(lt % ntc);
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   {
-    const int Q = tq * 32 + tx;
+    const int tx = threadIdx.x % NQ, ty = threadIdx.x / NQ, Q = tq * NQ + tx;
     const double* B = bs.B + F.b_off + Q;
-    int c = tc * 128 + ty, j = c / F.vpad, b = c - j * F.vpad;
-    double val[16];
+    int c = tc * NC + ty, j = c / F.vpad, b = c - j * F.vpad;
+    double val[NC / RS];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
+    for (int k = 0; k < NC / RS; ++k) {
       val[k] = c < RL && b < F.v && Q < F.X ? B[((long long)j * F.v + b) * F.X] : 0.0;
-      c += 8;
-      b += 8;
-      if (b >= F.vpad) { b -= F.vpad; ++j; }   // vpad is a multiple of 8
+      c += RS;
+      b += RS;
+      while (b >= F.vpad) { b -= F.vpad; ++j; }
     }
 #pragma unroll
-    for (int k = 0; k < 16; ++k) tile[tx][ty + 8 * k] = val[k];
+    for (int k = 0; k < NC / RS; ++k) tile[tx][ty + RS * k] = val[k];
   }
   __syncthreads();
   char* ws = (char*)bs.ws;
@@ -507,30 +506,25 @@ k_slice_b2(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
   int* ec = (int*)(ws + F.ecol);
   const long long plane = (long long)F.X * F.ldd;
   DT* out = (DT*)(ws + F.bs2);
-  const int cl0 = 4 * (tx % LPR);
+  const int cl = 4 * (threadIdx.x % (NC / 4)), c = tc * NC + cl;   // RL is a multiple of 4
 #pragma unroll 1
-  for (int qi = ty * (32 / LPR) + tx / LPR; qi < 32; qi += 8 * (32 / LPR)) {
-    const int Q = tq * 32 + qi;
-    if (Q >= F.X) break;
+  for (int qi = threadIdx.x / (NC / 4); qi < NQ; qi += 1024 / NC) {
+    const int Q = tq * NQ + qi;
+    if (Q >= F.X || c >= RL) break;
     const int E = cm[Q] > 0 ? ilogb_bits(cm[Q]) + 2 + Digit<F8>::HEAD : -1000;
-    if (tc == 0 && cl0 == 0) ec[Q] = E;
+    if (c == 0) ec[Q] = E;
     float s1, s2;
     pow2_factors(Digit<F8>::LB - E, s1, s2);
+    const double2 u = *(const double2*)&tile[qi][cl], w = *(const double2*)&tile[qi][cl + 2];
+    const double v4[4] = {u.x, u.y, w.x, w.y};
+    dfl xs[4];
 #pragma unroll
-    for (int cl = cl0; cl < 128; cl += 4 * LPR) {
-      const int c = tc * 128 + cl;   // RL is a multiple of 4
-      if (c >= RL) break;
-      const double2 u = *(const double2*)&tile[qi][cl], w = *(const double2*)&tile[qi][cl + 2];
-      const double v4[4] = {u.x, u.y, w.x, w.y};
-      dfl xs[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        float h, l;
-        split_to_df(v4[k], h, l);
-        xs[k] = {(h * s1) * s2, (l * s1) * s2};
-      }
-      put4<F8>(xs, st, out + (long long)Q * F.ldd + c, plane);
+    for (int k = 0; k < 4; ++k) {
+      float h, l;
+      split_to_df(v4[k], h, l);
+      xs[k] = {(h * s1) * s2, (l * s1) * s2};
     }
+    put4<F8>(xs, st, out + (long long)Q * F.ldd + c, plane);
   }
 }
 
@@ -554,13 +548,21 @@ k_slice_b2(const SplitFragDev* __restrict__ f, int nf, int st, Bases bs) {
 // LPR: lanes per row, 32, or fewer where the rows are short (amp_lanes).
 template <bool F8, int LPR>
 __global__ void __launch_bounds__(256, 3)
-k_amp_split(const SplitFragDev* __restrict__ f, int nf, Bases bs) {
+k_amp_split(const SplitFragDev* __restrict__ f, int nf, unsigned amp_ctas, int sg, Bases bs) {
   using DT = typename Digit<F8>::T;
   constexpr int LB = Digit<F8>::LB;
   constexpr int GROUPS = 32 / LPR, ROWS = 8 * GROUPS, C = 4 * LPR;
   constexpr int LDY = C + 4;   // 16-byte rows; the transposing writes of a warp then hit all banks
-  __shared__ __align__(16) float Yh[2][ROWS * LDY], Yl[2][ROWS * LDY];
+  union Smem {
+    float y[2][2][ROWS * LDY];    // [hi / lo][buffer]
+    double tile[B2Q<F8>][B2C<F8> + 2];
+  };
+  __shared__ __align__(16) Smem sm;
   __shared__ int s_last;
+  if (blockIdx.x >= amp_ctas) {   // Gamma's B operand, needed only after this launch
+    slice_b2<F8>(f, nf, (long long)(blockIdx.x - amp_ctas), sg, sm.tile, bs);
+    return;
+  }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const SplitFragDev& F = f[find_sfd(f, nf, blockIdx.x, 2)];
   const int v = F.v, o = F.o, vpad = F.vpad, vpadt = F.vpadt;
@@ -642,8 +644,8 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, Bases bs) {
   int j = jb, b0 = 0;
   if (steps > 0) load(j, 0);
   for (int s = 0; s < steps; ++s) {
-    float* const Sh = Yh[s & 1];
-    float* const Sl = Yl[s & 1];
+    float* const Sh = sm.y[0][s & 1];
+    float* const Sl = sm.y[1][s & 1];
     Sh[(yq + 0) * LDY + yb] = xh.x; Sh[(yq + 1) * LDY + yb] = xh.y;
     Sh[(yq + 2) * LDY + yb] = xh.z; Sh[(yq + 3) * LDY + yb] = xh.w;
     Sl[(yq + 0) * LDY + yb] = xl.x; Sl[(yq + 1) * LDY + yb] = xl.y;
@@ -749,21 +751,24 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, Bases bs) {
   __threadfence();
   double* ep = (double*)(ws + F.ep);
   const int parts = v > 0 ? strips * 8 : 0;
-  for (int jj = i + warp; jj < o; jj += 8) {
-    const float4* p = (const float4*)(ws + F.epart) + ((long long)i * o + jj) * (strips * 8);
+  for (int j0 = i + 4 * warp; j0 < o; j0 += 32) {   // eight lanes a pair
+    const int jj = j0 + (lane >> 3);
     double e = 0.0, eo = 0.0;
+    if (jj < o) {
+      const float4* p = (const float4*)(ws + F.epart) + ((long long)i * o + jj) * (strips * 8);
 #pragma unroll 4
-    for (int k = lane; k < parts; k += 32) {
-      const float4 w = __ldcg(p + k);
-      e += (double)w.x + (double)w.y;
-      eo += (double)w.z + (double)w.w;
+      for (int k = lane & 7; k < parts; k += 8) {
+        const float4 w = __ldcg(p + k);
+        e += (double)w.x + (double)w.y;
+        eo += (double)w.z + (double)w.w;
+      }
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
+    for (int off = 4; off > 0; off >>= 1) {
       e += __shfl_xor_sync(0xffffffffu, e, off);
       eo += __shfl_xor_sync(0xffffffffu, eo, off);
     }
-    if (lane == 0) {
+    if (jj < o && (lane & 7) == 0) {
       e = ldexp(e, 1 - 2 * kt);   // the scales of T and Tt
       eo = ldexp(eo, -2 * kt);
       ep[(long long)i * o + jj] = e;
@@ -1038,7 +1043,8 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
     s.row_begin = rows; s.b2_tile_begin = b2t; s.qblk_begin = qbl;
     rows += ov;
     if (g) {
-      b2t += (long long)((X + 31) / 32) * ((RL + 127) / 128);
+      const int nq = sp.fp8 ? B2Q<true> : B2Q<false>, nc = sp.fp8 ? B2C<true> : B2C<false>;
+      b2t += (long long)((X + nq - 1) / nq) * ((RL + nc - 1) / nc);
       qbl += (long long)((X + 31) / 32) * ((ov + kColRows - 1) / kColRows);
       w.want_gamma = true;
     }
@@ -1360,12 +1366,6 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long lon
     ++nl;
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess && w.b2_tiles > 0) {
-    if (sp.fp8) k_slice_b2<true><<<(unsigned)w.b2_tiles, 256, 0, s>>>(sfd, nf, sp.slices_g, bs);
-    else k_slice_b2<false><<<(unsigned)w.b2_tiles, 256, 0, s>>>(sfd, nf, sp.slices_g, bs);
-    ++nl;
-    e = cudaGetLastError();
-  }
   if (ev) cudaEventRecordWithFlags(ev[1], s, cudaEventRecordExternal);
   if (e == cudaSuccess && w.tiles_v > 0) {
     SplitLaunch cfg = sp.cfg_v;
@@ -1377,7 +1377,10 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long lon
   }
   if (ev) cudaEventRecordWithFlags(ev[2], s, cudaEventRecordExternal);
   if (e == cudaSuccess && total_pairs > 0) {
-    auto amp = [&](auto kernel) { kernel<<<(unsigned)total_pairs, 256, 0, s>>>(sfd, nf, bs); };
+    const unsigned ctas = (unsigned)total_pairs;
+    auto amp = [&](auto kernel) {
+      kernel<<<ctas + (unsigned)w.b2_tiles, 256, 0, s>>>(sfd, nf, ctas, sp.slices_g, bs);
+    };
     switch (w.amp_lpr) {
       case 8: sp.fp8 ? amp(k_amp_split<true, 8>) : amp(k_amp_split<false, 8>); break;
       case 16: sp.fp8 ? amp(k_amp_split<true, 16>) : amp(k_amp_split<false, 16>); break;
