@@ -67,6 +67,8 @@ int plan_f64_tiles(std::vector<GemmProb>& v, int grid, int per_sm, long long& to
   };
   for (auto& P : v) {
     const bool split = P.kind == PK_PAB || P.kind == PK_PIJ || (P.kind == PK_GEN && P.accumulate);
+    // Gamma may be cut in two (P.accumulate: the caller zeroes it): 0 + x + y is the same in
+    // either order, so the result stays reproducible
     const double K = (double)std::max(1LL, P.k_total);
     auto ext = [&](int bt, int n) { return (double)std::min<long long>(bt, up16(n)); };
     int bt = F64_T;
@@ -89,6 +91,10 @@ int plan_f64_tiles(std::vector<GemmProb>& v, int grid, int per_sm, long long& to
     } else {
       while (bt > 16 && ext(bt, P.M) * ext(bt, P.N) * K > unit) bt /= 2;
       P.k_chunk = std::max<long long>(up16(P.k_total), 16);
+      if (P.kind == PK_GAMMA) {
+        P.accumulate = ext(bt, P.M) * ext(bt, P.N) * K > 4.0 * unit && P.k_total >= 128;
+        if (P.accumulate) P.k_chunk = up16((P.k_total + 1) / 2);
+      }
     }
     P.bt = bt;
     P.ksplit = (int)std::max<long long>(1, (P.k_total + P.k_chunk - 1) / P.k_chunk);
@@ -133,23 +139,32 @@ cudaError_t launch_gemm_f64(const GemmProb* d_probs, int nprobs, long long total
 
 // ------------------------------------------------------------------ amplitudes
 
-// One CTA per pair block (i <= j) of one fragment.  Reads T_ij and writes
-// Tt_ij = 2 T_ij - T_ij^T for the (i,j) block and, if i != j, Tt_ji = Tt_ij^T for the
-// (j,i) block.  Pair energy e_ij = sum_ab Tt_ij(a,b) V_ij(a,b) with V = T * D, and its
-// opposite-spin part sum_ab T_ij(a,b) V_ij(a,b).
+// One CTA per pair block (i <= j) of one fragment and share of its 32 x 32 tile pairs.  Reads
+// T_ij and writes Tt_ij = 2 T_ij - T_ij^T for the (i,j) block and, if i != j, Tt_ji = Tt_ij^T
+// for the (j,i) block.  Pair energy e_ij = sum_ab Tt_ij(a,b) V_ij(a,b) with V = T * D, and its
+// opposite-spin part sum_ab T_ij(a,b) V_ij(a,b).  FP64 operations bound it (a warp's takes the
+// SM's pipe for 16 clocks): seven an element, and those of the sums, which are therefore long
+// in a lane and short across lanes.  A wave of few pairs cuts them over several CTAs
+// (amp_split; 55 pairs of nocc=10 nvir=40 on 55 SMs took 15 us).  Cut pairs of a narrow v are
+// taken element by element: no idle lanes at tile edges, and the strided accesses of
+// T_ij(b,a) and Tt_ji(b,a) stay in the lines of one block of at most 32 KB.  Where the
+// fragment has a counter (cnt_off), its last CTA adds the shares in a fixed order and sums the
+// fragment's energies.
 __global__ void __launch_bounds__(256)
 k_amplitude_f64(const FragDev* __restrict__ frags, int nfrag, Bases bs) {
   __shared__ double X[32][33];
   __shared__ double Y[32][33];
-  __shared__ double red[8], red_os[8];
+  __shared__ double red[2][256], sum[2];
+  __shared__ int s_last;
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
-  const long long gp = blockIdx.x;
-  const int f = find_frag(frags, nfrag, gp, [](const FragDev& F) { return F.pair_begin; });
+  const int f = find_frag(frags, nfrag, (long long)blockIdx.x, [](const FragDev& F) { return F.cta_begin; });
   const FragDev F = frags[f];
+  const long long lc = blockIdx.x - F.cta_begin, gp = lc / F.amp_split;
+  const int share = (int)(lc - gp * F.amp_split);
   int i, j;
-  tri_index(gp - F.pair_begin, i, j);
+  tri_index(gp, i, j);
   const int v = F.v, o = F.o;
-  const long long ov = (long long)o * v;
+  const long long ov = (long long)o * v, npair = (long long)o * (o + 1) / 2;
   const double* __restrict__ T = bs.ws + F.t_off;
   double* __restrict__ Tt = bs.ws + (F.tt_off >= 0 ? F.tt_off : 0);   // unused if < 0
   const double* eo = bs.eps + F.eo_off;
@@ -158,9 +173,26 @@ k_amplitude_f64(const FragDev* __restrict__ frags, int nfrag, Bases bs) {
   const long long rowI = (long long)i * v, rowJ = (long long)j * v;
   double e_part = 0.0, e_os = 0.0;
   const int nt = (v + 31) / 32;
-  const long long npairs = (long long)nt * (nt + 1) / 2;
+  const long long ntp = (long long)nt * (nt + 1) / 2;
+  const bool flat = amp_flat(F.amp_split, v);
+  const long long q0 = ntp * share / F.amp_split, q1 = flat ? q0 : ntp * (share + 1) / F.amp_split;
 
-  for (long long q = 0; q < npairs; ++q) {
+  if (flat) {
+    const int vv = v * v, end = vv * (share + 1) / F.amp_split;
+    for (int e = vv * share / F.amp_split + tid; e < end; e += 256) {
+      const int a = e / v, b = e - a * v;
+      const double t = T[(rowI + a) * ov + rowJ + b];
+      const double tt = 2.0 * t - T[(rowI + b) * ov + rowJ + a];
+      if (F.tt_off >= 0) {
+        Tt[(rowI + a) * ov + rowJ + b] = tt;
+        if (i != j) Tt[(rowJ + b) * ov + rowI + a] = tt;
+      }
+      const double V = t * (eij - ev[a] - ev[b]);
+      e_part += tt * V;
+      e_os += t * V;
+    }
+  }
+  for (long long q = q0; q < q1; ++q) {
     int ta, tb;
     tri_index(q, ta, tb);
     // X = T_ij[ta-rows][tb-cols], Y = T_ij[tb-rows][ta-cols]
@@ -215,32 +247,64 @@ k_amplitude_f64(const FragDev* __restrict__ frags, int nfrag, Bases bs) {
     }
     __syncthreads();
   }
-  // block reduction of the pair energy
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    e_part += __shfl_down_sync(0xffffffffu, e_part, off);
-    e_os += __shfl_down_sync(0xffffffffu, e_os, off);
-  }
-  if (tx == 0) { red[ty] = e_part; red_os[ty] = e_os; }
+  // the CTA's share of the pair energy: eight values a lane, then across the lanes
+  red[0][tid] = e_part;
+  red[1][tid] = e_os;
   __syncthreads();
-  if (tid == 0) {
-    double e = 0.0, eos = 0.0;
-    for (int w = 0; w < 8; ++w) { e += red[w]; eos += red_os[w]; }
-    double* ep = bs.ws + F.ep_off;
-    ep[(long long)i * o + j] = e;
-    ep[(long long)j * o + i] = e;
-    if (F.epos_off >= 0) {
-      double* eq = bs.ws + F.epos_off;
-      eq[(long long)i * o + j] = eos;
-      eq[(long long)j * o + i] = eos;
-    }
+  if (ty < 2) {
+    double x = 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) x += red[ty][tx + 32 * w];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    if (tx == 0) sum[ty] = x;
   }
+  __syncthreads();
+  double* ep = bs.ws + F.ep_off;
+  double* eq = F.epos_off >= 0 ? bs.ws + F.epos_off : nullptr;
+  auto put = [&](int a, int b, double e, double eos) {
+    ep[(long long)a * o + b] = e;
+    ep[(long long)b * o + a] = e;
+    if (eq) {
+      eq[(long long)a * o + b] = eos;
+      eq[(long long)b * o + a] = eos;
+    }
+  };
+  if (tid == 0) {
+    if (F.amp_split == 1) put(i, j, sum[0], sum[1]);
+    else ((double2*)(bs.ws + F.part_off))[gp * F.amp_split + share] = make_double2(sum[0], sum[1]);
+  }
+  if (F.cnt_off < 0) return;
+  __threadfence();
+  __syncthreads();
+  if (tid == 0)
+    s_last = atomicAdd((unsigned*)(bs.ws + F.cnt_off), 1u) + 1u == (unsigned)(npair * F.amp_split);
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (F.amp_split > 1) {
+    for (long long p = tid; p < npair; p += 256) {
+      const double2* w = (const double2*)(bs.ws + F.part_off) + p * F.amp_split;
+      double e = 0.0, eos = 0.0;
+      for (int k = 0; k < F.amp_split; ++k) {
+        const double2 x = __ldcg(w + k);
+        e += x.x;
+        eos += x.y;
+      }
+      int a, b;
+      tri_index(p, a, b);
+      put(a, b, e, eos);
+    }
+    __threadfence_block();
+    __syncthreads();
+  }
+  fragment_energy(ep, eq, (long long)o * o, F.epair_off >= 0 ? bs.epair + F.epair_off : nullptr, F.idx, bs);
 }
 
-cudaError_t launch_amplitude_f64(const FragDev* d_frags, int nfrag, long long total_pairs,
-                                 Bases bs, cudaStream_t s) {
-  if (total_pairs <= 0) return cudaSuccess;
-  k_amplitude_f64<<<(unsigned)total_pairs, 256, 0, s>>>(d_frags, nfrag, bs);
+cudaError_t launch_amplitude_f64(const FragDev* d_frags, int nfrag, long long total_ctas, Bases bs,
+                                 cudaStream_t s) {
+  if (total_ctas <= 0) return cudaSuccess;
+  k_amplitude_f64<<<(unsigned)total_ctas, 256, 0, s>>>(d_frags, nfrag, bs);
   return cudaGetLastError();
 }
 
@@ -259,36 +323,38 @@ cudaError_t launch_energy_reduce(const FragDev* d_frags, int nfrag, Bases bs, cu
   return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------ zero P outputs
+// ------------------------------------------------------------------ prologue and input checks
 
-__global__ void k_zero_p(const FragDev* __restrict__ frags, Bases bs) {
+// What a call's first launch prepares: the wave's queue counters (ctr, eight; may be null),
+// the fragment's amplitude counter, zero P (and Gamma where it is accumulated), the energies of
+// a fragment without pairs.  check: denominators must be negative for every (i,j,a,b), i.e.
+// max(eps_occ) < min(eps_vir); B and eps must be finite.  Violations set bits of the status
+// word.  (Seven launches a call of nocc=10 nvir=40 had three of these few microseconds each.)
+__global__ void __launch_bounds__(256)
+k_prologue(const FragDev* __restrict__ frags, unsigned* ctr, int check, Bases bs) {
   const FragDev F = frags[blockIdx.y];
-  const long long no = (long long)F.o * F.o, nv = (long long)F.v * F.v;
+  const long long first = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < no + nv;
-       e += stride) {
-    if (e < no) { if (F.pij_off >= 0) bs.pij[F.pij_off + e] = 0.0; }
-    else if (F.pab_off >= 0) bs.pab[F.pab_off + (e - no)] = 0.0;
+  if (ctr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 8) ctr[threadIdx.x] = 0u;
+  if (F.pij_off >= 0)
+    for (long long e = first; e < (long long)F.o * F.o; e += stride) bs.pij[F.pij_off + e] = 0.0;
+  if (F.pab_off >= 0)
+    for (long long e = first; e < (long long)F.v * F.v; e += stride) bs.pab[F.pab_off + e] = 0.0;
+  if (F.zero_gamma)
+    for (long long e = first; e < (long long)F.o * F.v * F.X; e += stride) bs.gamma[F.gamma_off + e] = 0.0;
+  if (F.cnt_off >= 0 && first == 0) {
+    *(unsigned*)(bs.ws + F.cnt_off) = 0u;
+    if (F.o == 0) {
+      bs.energy[F.idx] = 0.0;
+      if (bs.energy_os) bs.energy_os[F.idx] = 0.0;
+      if (bs.energy_scs) bs.energy_scs[F.idx] = 0.0;
+    }
   }
-}
-
-cudaError_t launch_zero_p(const FragDev* d_frags, int nfrag, Bases bs, cudaStream_t s) {
-  if (nfrag <= 0) return cudaSuccess;
-  k_zero_p<<<dim3(256, nfrag), 256, 0, s>>>(d_frags, bs);
-  return cudaGetLastError();
-}
-
-// ------------------------------------------------------------------ input checks
-
-// Denominators must be negative for every (i,j,a,b): max(eps_occ) < min(eps_vir).
-// B and eps must be finite.  Violations set bits of the status word.
-__global__ void k_check_inputs(const FragDev* __restrict__ frags, Bases bs) {
-  const FragDev F = frags[blockIdx.y];
+  if (!check) return;
   bool bad_nf = false;
   const long long nb = (long long)F.o * F.v * F.X;
   const double* B = bs.B + F.b_off;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nb; e += stride)
+  for (long long e = first; e < nb; e += stride)
     bad_nf |= !finite_bits(B[e]);
   if (blockIdx.x == 0) {
     __shared__ double smax[256], smin[256];
@@ -319,11 +385,11 @@ __global__ void k_check_inputs(const FragDev* __restrict__ frags, Bases bs) {
   if (bad_nf) atomicOr(bs.status, ST_NONFINITE);
 }
 
-cudaError_t launch_check_inputs(const FragDev* d_frags, int nfrag, long long max_bx, Bases bs,
-                                cudaStream_t s) {
+cudaError_t launch_prologue(const FragDev* d_frags, int nfrag, long long max_bx, unsigned* ctr, int check,
+                            Bases bs, cudaStream_t s) {
   if (nfrag <= 0) return cudaSuccess;
   const unsigned bx = (unsigned)(max_bx < 1 ? 1 : (max_bx > 256 ? 256 : max_bx));
-  k_check_inputs<<<dim3(bx, nfrag), 256, 0, s>>>(d_frags, bs);
+  k_prologue<<<dim3(bx, nfrag), 256, 0, s>>>(d_frags, ctr, check, bs);
   return cudaGetLastError();
 }
 

@@ -104,7 +104,9 @@ extern "C" int rimp2_energy_fp64_noalloc(int32_t nocc, int32_t nvir, int32_t nau
   fd.ep_off = (long long)(t_bytes / sizeof(double));
   fd.gamma_off = fd.pij_off = fd.pab_off = -1;
   fd.epair_off = epair ? 0 : -1;
-  fd.pair_begin = 0;
+  fd.cta_begin = 0;
+  fd.amp_split = 1;
+  fd.part_off = fd.cnt_off = -1;
   fd.epos_off = -1;
   GemmProb P{};
   long long tiles = 0;
@@ -127,7 +129,7 @@ extern "C" int rimp2_energy_fp64_noalloc(int32_t nocc, int32_t nvir, int32_t nau
   bs.status = (unsigned*)scratch;
   const FragDev* d_fd = (const FragDev*)(scratch + kFragOff);
   if (e == cudaSuccess)
-    e = launch_check_inputs(d_fd, 1, ((long long)ov * naux + 255) / 256, bs, s);
+    e = launch_prologue(d_fd, 1, ((long long)ov * naux + 255) / 256, nullptr, 1, bs, s);
   if (e == cudaSuccess)
     e = launch_gemm_f64((const GemmProb*)(scratch + kProbOff), 1, tiles, bs,
                         (unsigned*)(scratch + kCounterOff), grid, s);

@@ -129,12 +129,21 @@ namespace {
 
 bool wants_tt(const rimp2_frag& f) { return f.gamma_off >= 0 || f.pij_off >= 0 || f.pab_off >= 0; }
 
+// Amplitude CTAs a pair may be cut over, at most; CTAs of a wave whose
+// pairs are cut, at most
+constexpr int kMaxAmpSplit = 16, kMaxAmpParts = 1024;
+size_t amp_part_elems(const rimp2_frag& f) {
+  return 2 * std::min<size_t>((size_t)f.nocc * (f.nocc + 1) / 2 * kMaxAmpSplit, kMaxAmpParts);
+}
+
 // Workspace of one fragment on the FP64 path; build_fp64_wave lays out exactly this:
-// T, Tt (when an output needs it), pair energies and their opposite-spin part.
+// T, Tt (when an output needs it), pair energies and their opposite-spin part, the amplitude
+// CTAs' shares of them and their counter.
 size_t frag_ws_elems_fp64(const rimp2_frag& f) {
   const size_t ov = (size_t)f.nocc * f.nvir;
   return align_up(ov * ov, kAlignElems) * (wants_tt(f) ? 2 : 1) +
-         align_up(2 * (size_t)f.nocc * f.nocc, kAlignElems);
+         align_up(2 * (size_t)f.nocc * f.nocc, kAlignElems) +
+         align_up(amp_part_elems(f) + 1, kAlignElems);
 }
 
 size_t frag_ws_elems(const rimp2_plan* p, const rimp2_frag& f) {
@@ -169,7 +178,9 @@ int build_fp64_wave(rimp2_plan* p, const rimp2_frag* frags, WaveDesc& w) {
     ws += align_up(2 * (size_t)f.nocc * f.nocc, kAlignElems);
     d.gamma_off = f.gamma_off; d.pij_off = f.pij_off; d.pab_off = f.pab_off;
     d.epair_off = f.epair_off;
-    d.pair_begin = pairs;
+    d.part_off = (long long)ws;
+    d.cnt_off = d.part_off + (long long)amp_part_elems(f);
+    ws += align_up(amp_part_elems(f) + 1, kAlignElems);
     pairs += (long long)f.nocc * (f.nocc + 1) / 2;
     w.fdev.push_back(d);
     w.max_b = std::max<long long>(w.max_b, (long long)ov * f.naux);
@@ -216,9 +227,23 @@ int build_fp64_wave(rimp2_plan* p, const rimp2_frag* frags, WaveDesc& w) {
       w.probs_c.push_back(P);
     }
   }
-  w.total_pairs = pairs;
+  // amplitude CTAs per pair: up to four a SM where the pairs are few, with at least one pair
+  // of tiles (or two elements a thread) each
+  w.total_pairs = 0;
+  for (auto& d : w.fdev) {
+    const long long nt = (d.v + 31) / 32, ntp = nt * (nt + 1) / 2;
+    const long long want = std::min(p->gemm_grid, kMaxAmpParts) / std::max(pairs, 1LL);
+    const long long cut = amp_flat(2, d.v) ? ((long long)d.v * d.v + 511) / 512 : ntp;
+    d.amp_split = (int)std::max(1LL, std::min(std::min<long long>(want, kMaxAmpSplit), cut));
+    d.cta_begin = w.total_pairs;
+    w.total_pairs += (long long)d.o * (d.o + 1) / 2 * d.amp_split;
+  }
   w.grid_v = plan_f64_tiles(w.probs_v, p->gemm_grid, F64_ITEMS_PER_SM, w.tiles_v);
   w.grid_c = plan_f64_tiles(w.probs_c, p->gemm_grid, p->variant == 0 ? F64_ITEMS_PER_SM : (F64_ITEMS_PER_SM / 4) << (p->variant == 1 ? 1 : 3), w.tiles_c);
+  for (const auto& P : w.probs_c)
+    if (P.kind == PK_GAMMA && P.accumulate)
+      for (auto& d : w.fdev)
+        if (d.idx == P.frag) d.zero_gamma = 1;
   // the layout must fit the workspace the plan sized with frag_ws_elems_fp64
   if (ws * sizeof(double) + 256 > p->ws_bytes) return RIMP2_ERR_WORKSPACE;
   return RIMP2_OK;
@@ -288,10 +313,6 @@ int enqueue(rimp2_plan* p, const rimp2_batch* b, void* ws, cudaStream_t s) {
   bs.energy_scs = b->energy_scs; bs.scs_os = p->opt.scs_os; bs.scs_ss = p->opt.scs_ss;
   int launches = 0;
   long long tiles = 0;
-  // the split path's prologue kernel clears its wave's counters
-  if (p->precision == RIMP2_FP64 &&
-      cudaMemsetAsync(p->d_counters, 0, p->waves.size() * 8 * sizeof(unsigned), s) != cudaSuccess)
-    return RIMP2_ERR_CUDA;
   for (size_t wi = 0; wi < p->waves.size(); ++wi) {
     WaveDesc& w = p->waves[wi];
     const FragDev* dfd = (const FragDev*)(p->dblk + w.off_fdev);
@@ -300,20 +321,17 @@ int enqueue(rimp2_plan* p, const rimp2_batch* b, void* ws, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     cudaEvent_t* ev = p->stage_ev.empty() ? nullptr : &p->stage_ev[wi * kEv];
     if (ev && cudaEventRecordWithFlags(ev[0], s, cudaEventRecordExternal) != cudaSuccess) return RIMP2_ERR_CUDA;
-    if (p->opt.check_inputs && p->precision == RIMP2_FP64) {
-      e = launch_check_inputs(dfd, nf, (w.max_b + 255) / 256, bs, s);
-      ++launches;
-      if (e != cudaSuccess) return RIMP2_ERR_CUDA;
-    }
     if (p->precision == RIMP2_FP64) {
+      // (both paths' first kernel clears the wave's queue counters)
+      e = launch_prologue(dfd, nf, (w.max_b + 255) / 256, ctr, p->opt.check_inputs != 0, bs, s);
+      launches += nf > 0;
+      if (e != cudaSuccess) return RIMP2_ERR_CUDA;
       if (ev) cudaEventRecordWithFlags(ev[1], s, cudaEventRecordExternal);
       e = launch_gemm_f64((const GemmProb*)(p->dblk + w.off_pv), (int)w.probs_v.size(), w.tiles_v,
                           bs, ctr + 0, w.grid_v, s);
       launches += w.tiles_v > 0;
       if (ev) cudaEventRecordWithFlags(ev[2], s, cudaEventRecordExternal);
       if (e == cudaSuccess) { e = launch_amplitude_f64(dfd, nf, w.total_pairs, bs, s); launches += w.total_pairs > 0; }
-      if (e == cudaSuccess) { e = launch_energy_reduce(dfd, nf, bs, s); ++launches; }
-      if (e == cudaSuccess) { e = launch_zero_p(dfd, nf, bs, s); ++launches; }
       if (ev) cudaEventRecordWithFlags(ev[3], s, cudaEventRecordExternal);
       if (e == cudaSuccess) {
         e = launch_gemm_f64((const GemmProb*)(p->dblk + w.off_pc), (int)w.probs_c.size(), w.tiles_c,

@@ -122,7 +122,7 @@ struct GemmProb {
   const double* pa;          // PK_GEN: A, Bop and C base pointers (offsets unused)
   const double* pb;
   double* pc;
-  int accumulate, pad;       // PK_GEN: 1 adds into C (atomics); 0 stores (needs ksplit 1)
+  int accumulate, pad;       // PK_GEN, PK_GAMMA: 1 adds into C (atomics); 0 stores (ksplit 1)
 };
 
 // Per-fragment info used by the elementwise / reduction kernels.
@@ -132,12 +132,19 @@ struct FragDev {
   long long t_off, tt_off, ep_off;   // workspace offsets (elements)
   long long epos_off;         // opposite-spin pair energies [o][o] (elements), or -1
   long long gamma_off, pij_off, pab_off, epair_off;  // -1: not requested
-  long long pair_begin;       // prefix of o(o+1)/2 pair blocks in the wave
+  long long cta_begin;        // first amplitude CTA of the fragment
+  long long part_off;         // double2 [pairs][amp_split]: the CTAs' shares of the pair energies
+  long long cnt_off;          // amplitude CTAs done, or -1: no fused energy sums
+  int amp_split, zero_gamma;  // amplitude CTAs per pair; 1: Gamma is accumulated, zero it first
 };
 
+// Amplitude CTAs of a cut pair take elements instead of 32 x 32 tile pairs
+__host__ __device__ inline bool amp_flat(int split, int v) { return split > 1 && v <= 64; }
+
 // ---- launchers (fp64_kernels.cu) ----
-cudaError_t launch_check_inputs(const FragDev* d_frags, int nfrag, long long max_bx,
-                                Bases bs, cudaStream_t s);
+// ctr: eight queue counters to clear, or null; check: 1 for the input checks
+cudaError_t launch_prologue(const FragDev* d_frags, int nfrag, long long max_bx, unsigned* ctr, int check,
+                            Bases bs, cudaStream_t s);
 cudaError_t launch_gemm_f64(const GemmProb* d_probs, int nprobs, long long total_tiles,
                             Bases bs, unsigned* counter, int grid, cudaStream_t s);
 int gemm_f64_occupancy_grid();
@@ -147,9 +154,8 @@ constexpr int F64_ITEMS_PER_SM = 16;
 // Sets the tiles, K pieces and queue positions of one launch's problems; grid: CTAs that
 // fit the GPU.  Returns the CTAs to launch.
 int plan_f64_tiles(std::vector<GemmProb>& probs, int grid, int per_sm, long long& total);
-cudaError_t launch_amplitude_f64(const FragDev* d_frags, int nfrag, long long total_pairs,
-                                 Bases bs, cudaStream_t s);
+cudaError_t launch_amplitude_f64(const FragDev* d_frags, int nfrag, long long total_ctas, Bases bs,
+                                 cudaStream_t s);
 cudaError_t launch_energy_reduce(const FragDev* d_frags, int nfrag, Bases bs, cudaStream_t s);
-cudaError_t launch_zero_p(const FragDev* d_frags, int nfrag, Bases bs, cudaStream_t s);
 
 }  // namespace rimp2
