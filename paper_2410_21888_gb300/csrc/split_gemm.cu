@@ -542,7 +542,8 @@ __device__ __forceinline__ void tma_operand(uint32_t dst, const CUtensorMap* tm,
 template <int NT, int ROWB, bool F8, int EPI>
 __global__ void __launch_bounds__((2 + EPI) * 32, 1)
 k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ begins, int nprobs,
-             long long total, Bases bs, unsigned* __restrict__ counter, int slices, int stages) {
+             long long total, Bases bs, unsigned* __restrict__ counter, int slices, int stages,
+             int beside) {
   constexpr int NC = NT / (EPI / 4);         // columns per epilogue thread
   // two register buffers in the drain where the registers allow it (168 a thread with
   // 8 epilogue warps, 96 with 16)
@@ -609,6 +610,7 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_trigger();   // TMEM is held: a CTA of the next kernel can only wait for it, not take it
   const uint32_t tmem_base = *tmem_base_slot;
   const uint64_t cwait = g_sg_consumer_wait_ns;   // consumer-side wait limit
   // Two sets of level accumulators when both fit the 512 TMEM columns: the MMAs of the
@@ -1029,6 +1031,7 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u)
                  : "memory");
   }
+  if (beside) pdl_wait();
 }
 
 // ------------------------------------------------------------------ slice-stacked kernel
@@ -1069,7 +1072,7 @@ template <bool F8>
 __global__ void __launch_bounds__((2 + kStackEpi) * 32, 1)
 k_split_stack(const SplitProb* __restrict__ probs, const long long* __restrict__ begins, int nprobs,
               long long total, Bases bs, unsigned* __restrict__ counter, int slices, int stages,
-              uint32_t half_bytes) {
+              uint32_t half_bytes, int beside) {
   constexpr int ROWB = 64, BKE = F8 ? 64 : 32;
   constexpr int CHUNK_STAGES = (F8 ? SG_CHUNK_K_FP8 : SG_CHUNK_K_BF16) / BKE;
   constexpr int LB = F8 ? SG_LB_FP8 : SG_LB_BF16;
@@ -1125,6 +1128,7 @@ k_split_stack(const SplitProb* __restrict__ probs, const long long* __restrict__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_trigger();   // TMEM is held: a CTA of the next kernel can only wait for it, not take it
   const uint32_t tmem_base = *tmem_base_slot;
   const uint64_t cwait = g_sg_consumer_wait_ns;
   // Row groups of a tile with R rows a slice: group 0 is rows 0..127 against all slices q,
@@ -1384,6 +1388,7 @@ k_split_stack(const SplitProb* __restrict__ probs, const long long* __restrict__
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u)
                  : "memory");
   }
+  if (beside) pdl_wait();
 }
 
 // ------------------------------------------------------------------ host side
@@ -1426,16 +1431,14 @@ template <int NT, int ROWB, bool F8>
 static cudaError_t launch_nt(const SplitProb* d_probs, const long long* d_begins, int nprobs,
                              long long total, Bases bs, unsigned* counter, const SplitLaunch& cfg,
                              int grid, cudaStream_t s) {
+  const int beside = cfg.beside;
   if constexpr (ROWB == 64) {
-    if (cfg.epi_warps == 16) {
-      k_split_gemm<NT, ROWB, F8, 16><<<grid, (2 + 16) * 32, cfg.smem, s>>>(
-          d_probs, d_begins, nprobs, total, bs, counter, cfg.slices, cfg.stages);
-      return cudaGetLastError();
-    }
+    if (cfg.epi_warps == 16)
+      return launch_pdl(k_split_gemm<NT, ROWB, F8, 16>, grid, (2 + 16) * 32, cfg.smem, s, cfg.beside, d_probs,
+                        d_begins, nprobs, total, bs, counter, cfg.slices, cfg.stages, beside);
   }
-  k_split_gemm<NT, ROWB, F8, 8><<<grid, (2 + 8) * 32, cfg.smem, s>>>(
-      d_probs, d_begins, nprobs, total, bs, counter, cfg.slices, cfg.stages);
-  return cudaGetLastError();
+  return launch_pdl(k_split_gemm<NT, ROWB, F8, 8>, grid, (2 + 8) * 32, cfg.smem, s, cfg.beside, d_probs, d_begins,
+                    nprobs, total, bs, counter, cfg.slices, cfg.stages, beside);
 }
 
 // Opt in to the large dynamic shared memory once per device, outside any capture.
@@ -1502,7 +1505,7 @@ int split_stack_rows(int slices, int n) {
 
 cudaError_t launch_split_stack(const SplitProb* d_probs, const long long* d_begins, int nprobs,
                                long long total_tiles, Bases bs, unsigned* counter, int slices,
-                               int max_rows, bool fp8, int grid, cudaStream_t s) {
+                               int max_rows, bool fp8, int grid, bool beside, cudaStream_t s) {
   if (total_tiles <= 0) return cudaSuccess;
   const size_t half = ((size_t)slices * max_rows * 64 + 1023) / 1024 * 1024;
   const size_t red = (size_t)slices * max_rows * max_rows * sizeof(float2);
@@ -1514,13 +1517,11 @@ cudaError_t launch_split_stack(const SplitProb* d_probs, const long long* d_begi
   if (stages < 1) return cudaErrorInvalidValue;
   const size_t smem = fixed + slack + (size_t)stages * 2 * half;
   const unsigned g = (unsigned)(total_tiles < grid ? total_tiles : grid);
-  if (fp8)
-    k_split_stack<true><<<g, (2 + kStackEpi) * 32, smem, s>>>(d_probs, d_begins, nprobs, total_tiles, bs,
-                                                             counter, slices, stages, (uint32_t)half);
-  else
-    k_split_stack<false><<<g, (2 + kStackEpi) * 32, smem, s>>>(d_probs, d_begins, nprobs, total_tiles, bs,
-                                                              counter, slices, stages, (uint32_t)half);
-  return cudaGetLastError();
+  auto go = [&](auto kernel) {
+    return launch_pdl(kernel, g, (2 + kStackEpi) * 32, smem, s, beside, d_probs, d_begins, nprobs, total_tiles,
+                      bs, counter, slices, stages, (uint32_t)half, (int)beside);
+  };
+  return fp8 ? go(k_split_stack<true>) : go(k_split_stack<false>);
 }
 
 int split_gemm_grid() {

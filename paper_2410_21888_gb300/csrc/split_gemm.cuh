@@ -87,6 +87,9 @@ struct SplitLaunch {
   int stages;     // pipeline depth
   size_t smem;    // dynamic shared memory bytes
   int epi_warps;  // epilogue warps: 8, or 16 (more warps for a tile's drain and epilogue)
+  // the launch before in the stream is another contraction of the same call, on which this
+  // one doesn't depend: this one's CTAs fill the SMs that it leaves (see pdl_trigger)
+  bool beside;
 };
 
 // n_tile: columns per level accumulator (0: widest that fits 512 TMEM columns; else 64,
@@ -102,7 +105,7 @@ cudaError_t launch_split_gemm(const SplitProb* d_probs, const long long* d_begin
 int split_stack_rows(int slices, int n);
 cudaError_t launch_split_stack(const SplitProb* d_probs, const long long* d_begins, int nprobs,
                                long long total_tiles, Bases bs, unsigned* counter, int slices,
-                               int max_rows, bool fp8, int grid, cudaStream_t s);
+                               int max_rows, bool fp8, int grid, bool beside, cudaStream_t s);
 int split_gemm_grid();
 // Consumer-side wait limit of the contraction kernel on the current device (ns < 0: the
 // normal 2 s); synchronous.  Used by a test hook only.

@@ -1390,6 +1390,9 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long lon
     e = cudaGetLastError();
   }
   if (ev) cudaEventRecordWithFlags(ev[3], s, cudaEventRecordExternal);
+  // The P launches and Gamma's read what the amplitude launch wrote and nothing of each other:
+  // the next one's CTAs take the SMs that the one before leaves (at nocc=10 nvir=40 all 134 CTAs
+  // of both run at once).  Events between the launches keep them apart.
   if (e == cudaSuccess && w.tiles_c > 0) {
     SplitLaunch cfg = sp.cfg_t;
     cfg.epi_warps = w.epi_warps;
@@ -1401,13 +1404,14 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long lon
   if (e == cudaSuccess && w.tiles_s > 0) {
     e = launch_split_stack((const SplitProb*)(dblk + w.off_ps), (const long long*)(dblk + w.off_bs),
                            (int)w.probs_s.size(), w.tiles_s, bs, ctr + 3, sp.slices_t, w.stack_rows,
-                           sp.fp8, sp.grid, s);
+                           sp.fp8, sp.grid, !ev && w.tiles_c > 0, s);
     ++nl;
   }
   if (ev) cudaEventRecordWithFlags(ev[4], s, cudaEventRecordExternal);
   if (e == cudaSuccess && w.tiles_g > 0) {
     SplitLaunch cfg = sp.cfg_g;
     cfg.epi_warps = w.epi_warps;
+    cfg.beside = !ev && (w.tiles_c > 0 || w.tiles_s > 0);
     e = launch_split_gemm((const SplitProb*)(dblk + w.off_pg), (const long long*)(dblk + w.off_bg),
                           (int)w.probs_g.size(), w.tiles_g, bs,
                           ctr + 2, cfg, sp.grid, s);
