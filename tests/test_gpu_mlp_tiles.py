@@ -1,7 +1,7 @@
-"""Tile edges of the screen's network kernels (16 samples a tile in the gradient, 64 in the
-prediction, one CTA per tile up to the grid, then a loop) and parameter vectors without
-16-byte alignment, against the NumPy FP64 oracle.  Tolerances as in test_gpu_mlp.py: FP32
-accumulation over chains of 64 terms and three layers stays below 2e-4 in norm (gradient)
+"""Tile edges of the screen's network kernels (16 samples a tile and CTA in the gradient, 8
+samples a tile and warp in the prediction, up to the grid, then a loop) and parameter vectors
+without 16-byte alignment, against the NumPy FP64 oracle.  Tolerances as in test_gpu_mlp.py:
+FP32 accumulation over chains of 64 terms and three layers stays below 2e-4 in norm (gradient)
 and 1e-4 of the largest prediction."""
 import numpy as np
 import pytest
