@@ -467,30 +467,43 @@ __device__ __forceinline__ int find_problem(const SplitProb* __restrict__ probs,
   return lo;
 }
 
+// a / b, 0 <= a, b: in 32 bits where both fit, which they practically always do (a 64-bit
+// division is some hundred dependent instructions, and a tile's decoding had four: 40 MBE3
+// dimers' Gamma 4.02 -> 3.95 ms, 100 trimers' V 12.50 -> 12.32 ms, nocc=42 FP8 P and Gamma
+// 1.68 -> 1.64 ms)
+__device__ __forceinline__ long long div_pos(long long a, long long b) {
+  return ((a | b) >> 32) == 0 ? (long long)((unsigned)a / (unsigned)b) : a / b;
+}
+
 __device__ __forceinline__ TileInfo decode_tile(const SplitProb* __restrict__ probs, int pi,
                                                 long long t, int nt) {
   TileInfo ti;
   ti.P = probs + pi;
   const SplitProb* P = ti.P;
   const long long lt = t - P->tile_begin;
-  const long long per = (long long)P->tiles_m * P->tiles_n;
-  int ks;
-  long long tt;
-  if (P->ks_outer) { ks = (int)(lt / per); tt = lt - (long long)ks * per; }
-  else { ks = (int)(lt % P->ksplit); tt = lt / P->ksplit; }
+  int ks = 0;
+  long long tt = lt;
+  if (P->ks_outer) {
+    const long long per = (long long)P->tiles_m * P->tiles_n;
+    ks = (int)div_pos(lt, per);
+    tt = lt - (long long)ks * per;
+  } else if (P->ksplit > 1) {
+    tt = div_pos(lt, P->ksplit);
+    ks = (int)(lt - tt * P->ksplit);
+  }
   if (P->group_m > 1) {
     // groups of group_m rows, walked column by column: the group's A rows stay in L2
     // while each column block of B is used by group_m tiles that run side by side
     const long long gsz = (long long)P->group_m * P->tiles_n;
-    const int g = (int)(tt / gsz);
+    const int g = (int)div_pos(tt, gsz);
     const int first = g * P->group_m;
     const int gm = min(P->group_m, P->tiles_m - first);
     const int r = (int)(tt - g * gsz);
-    ti.tm = first + r % gm;
     ti.tn = r / gm;
+    ti.tm = first + r - ti.tn * gm;
   } else {
-    ti.tm = (int)(tt / P->tiles_n);
-    ti.tn = (int)(tt % P->tiles_n);
+    ti.tm = (int)div_pos(tt, P->tiles_n);
+    ti.tn = (int)(tt - (long long)ti.tm * P->tiles_n);
   }
   ti.k1b = ks * ti.P->k1_chunk;
   ti.k1e = min(ti.P->k1_count, ti.k1b + ti.P->k1_chunk);
@@ -628,25 +641,32 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
       uint32_t tph = 0;
       bool pending[8] = {false, false, false, false, false, false, false, false};
       uint32_t pend_ph[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      for (bool first = true;; first = false) {
-        // entries 0 .. gridDim.x - 1 are dealt by index, the others through the counter
-        const long long t = first ? (long long)blockIdx.x
-                                  : (long long)gridDim.x + (long long)atomicAdd(counter, 1u);
-        // the problem search is done here once per entry; the MMA and epilogue warps take
-        // its result from shared memory
-        const int pi = first ? first_prob : t < total ? find_problem(probs, begins, nprobs, t) : 0;
-        TileInfo ti{};
-        if (t < total) {
+      // The problem search is done here once per entry; the MMA and epilogue warps take its
+      // result from shared memory.  Entries 0 .. gridDim.x - 1 are dealt by index, the others
+      // through the counter, when the loads of the one before are issued.  (Claiming them some
+      // stages earlier, to hide the counter's round trip, lost more by the order in which the
+      // SMs then share operands in L2: V of 40 MBE3 dimers 3.57 -> 3.73 ms.)
+      long long t = (long long)blockIdx.x;
+      int pi = first_prob;
+      TileInfo ti{};
+      auto next_entry = [&]() {
+        t = (long long)gridDim.x + (long long)atomicAdd(counter, 1u);
+        if (t < total) pi = find_problem(probs, begins, nprobs, t);
+      };
+      auto decode = [&]() {
+        while (t < total) {
           ti = decode_tile(probs, pi, t, NT);
-          if (ti.skip) {
-            // a tile without work is not handed on; where it starts a run of them (the
-            // columns of a V row group right of the diagonal), the queue moves past the run
-            const long long run_end = skipped_run_end(ti, t, NT);
-            if (run_end > t + 1 && min(run_end, total) > (long long)gridDim.x)
-              atomicMax(counter, (unsigned)(min(run_end, total) - (long long)gridDim.x));
-            continue;
-          }
+          if (!ti.skip) return;
+          // a tile without work is not handed on; where it starts a run of them (the
+          // columns of a V row group right of the diagonal), the queue moves past the run
+          const long long run_end = skipped_run_end(ti, t, NT);
+          if (run_end > t + 1 && min(run_end, total) > (long long)gridDim.x)
+            atomicMax(counter, (unsigned)(min(run_end, total) - (long long)gridDim.x));
+          next_entry();
         }
+      };
+      decode();
+      for (;;) {
         if (!mbar_wait(tile_empty + tslot, tph ^ 1u, abort_flag)) break;
         tile_idx[tslot] = t;
         tile_prob[tslot] = pi;
@@ -655,25 +675,27 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
         if (tslot == 0) tph ^= 1u;
         if (t >= total) break;
         const SplitProb* P = ti.P;
-        const int rowA = ti.tm * SG_BM, rowB = ti.tn * NT;
+        const int rowA = ti.tm * SG_BM, rowB = ti.tn * NT, nK = ti.nK, k0b = P->k0_blocks;
+        int k1 = ti.k1b, kb = 0;
         bool ok = true;
-        for (int kk = 0; kk < ti.nK; ++kk) {
+        for (int kk = 0; kk < nK; ++kk) {
           if (!mbar_wait(empty + st, ph ^ 1u, abort_flag)) { ok = false; break; }
           pending[st] = false;
           mbar_arrive_expect_tx(full + st, stage_bytes);
           pending[st] = true;
           pend_ph[st] = ph;
-          const int k1 = ti.k1b + kk / P->k0_blocks;
-          const int x = (kk % P->k0_blocks) * BKE;
           const uint32_t base = smem_u32(smem + (size_t)st * stage_bytes);
           // one box per operand covers all slices (the outermost tensor dimension): slice
           // p of A lands at p * A_TILE, slice q of B at slices * A_TILE + q * B_TILE
-          tma_operand(base, &P->tmA, full + st, P->a_mode, x, rowA, k1, P->div5, 0);
-          tma_operand(base + slices * A_TILE, &P->tmB, full + st, P->b_mode, x, rowB, k1, P->div5,
+          tma_operand(base, &P->tmA, full + st, P->a_mode, kb * BKE, rowA, k1, P->div5, 0);
+          tma_operand(base + slices * A_TILE, &P->tmB, full + st, P->b_mode, kb * BKE, rowB, k1, P->div5,
                       0);
+          if (++kb == k0b) { kb = 0; ++k1; }
           if (++st == (uint32_t)stages) { st = 0; ph ^= 1u; }
         }
         if (!ok) break;
+        next_entry();
+        decode();
       }
       if (*abort_flag) {
         // let our own copies in flight land before the CTA leaves (bounded)
@@ -1058,7 +1080,7 @@ __device__ __forceinline__ StackTile stack_tile(const SplitProb* __restrict__ pr
   ti.P = probs + pi;
   const int tri = ti.P->tiles_m * (ti.P->tiles_m + 1) / 2;
   const long long lt = t - ti.P->tile_begin;
-  const int ks = (int)(lt / tri);
+  const int ks = (int)div_pos(lt, tri);
   int r = (int)(lt - (long long)ks * tri), c = 0;
   while (r > c) { ++c; r -= c; }   // column by column: r <= c
   ti.tm = r;
@@ -1145,10 +1167,14 @@ k_split_stack(const SplitProb* __restrict__ probs, const long long* __restrict__
       int tslot = 0;
       bool pending[8] = {false, false, false, false, false, false, false, false};
       uint32_t pend_ph[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      for (bool first = true;; first = false) {
-        const long long t = first ? (long long)blockIdx.x
-                                  : (long long)gridDim.x + (long long)atomicAdd(counter, 1u);
-        const int pi = first ? first_prob : t < total ? find_problem(probs, begins, nprobs, t) : 0;
+      // entries as in k_split_gemm
+      long long t = (long long)blockIdx.x;
+      int pi = first_prob;
+      auto next_entry = [&]() {
+        t = (long long)gridDim.x + (long long)atomicAdd(counter, 1u);
+        if (t < total) pi = find_problem(probs, begins, nprobs, t);
+      };
+      for (;;) {
         if (!mbar_wait(tile_empty + tslot, tph ^ 1u, abort_flag)) break;
         tile_idx[tslot] = t;
         tile_prob[tslot] = pi;
@@ -1158,8 +1184,9 @@ k_split_stack(const SplitProb* __restrict__ probs, const long long* __restrict__
         if (t >= total) break;
         const StackTile ti = stack_tile(probs, pi, t);
         const SplitProb* P = ti.P;
-        const int R = P->n_tile;
+        const int R = P->n_tile, k0b = P->k0_blocks;
         const uint32_t bytes = 2u * (uint32_t)(slices * R * ROWB);
+        int k1 = ti.k1b, kb = 0;
         bool ok = true;
         for (int kk = 0; kk < ti.nK; ++kk) {
           if (!mbar_wait(empty + st, ph ^ 1u, abort_flag)) { ok = false; break; }
@@ -1167,14 +1194,14 @@ k_split_stack(const SplitProb* __restrict__ probs, const long long* __restrict__
           mbar_arrive_expect_tx(full + st, bytes);
           pending[st] = true;
           pend_ph[st] = ph;
-          const int k1 = ti.k1b + kk / P->k0_blocks;
-          const int x = (kk % P->k0_blocks) * BKE;
           const uint32_t base = smem_u32(smem + (size_t)st * stage_bytes);
-          tma_operand(base, &P->tmA, full + st, P->a_mode, x, ti.tm * R, k1, P->div5, 0);
-          tma_operand(base + half_bytes, &P->tmB, full + st, P->b_mode, x, ti.tn * R, k1, P->div5, 0);
+          tma_operand(base, &P->tmA, full + st, P->a_mode, kb * BKE, ti.tm * R, k1, P->div5, 0);
+          tma_operand(base + half_bytes, &P->tmB, full + st, P->b_mode, kb * BKE, ti.tn * R, k1, P->div5, 0);
+          if (++kb == k0b) { kb = 0; ++k1; }
           if (++st == (uint32_t)stages) { st = 0; ph ^= 1u; }
         }
         if (!ok) break;
+        next_entry();
       }
       if (*abort_flag) {
         for (int s = 0; s < stages; ++s)
