@@ -494,6 +494,7 @@ int rimp2_plan_create(const rimp2_frag* frags, int32_t nfrag, int32_t precision,
   if (precision != RIMP2_FP64) {
     rc = split_plan_init(p->split, precision, o);
     if (rc != RIMP2_OK) { delete p; return rc; }
+    split_shape_v(p->split, o, frags, nfrag);
   }
   // waves: batch order, a new wave when the workspace budget would be exceeded
   size_t cur = 0, worst = 0;

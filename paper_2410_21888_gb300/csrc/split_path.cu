@@ -844,12 +844,9 @@ int split_plan_init(SplitPlan& sp, int precision, const rimp2_options& opt) {
   sp.slices_t = opt.slices_t;
   sp.slices_g = opt.slices_g;
   sp.fp8 = precision == RIMP2_FP8_SPLIT;
-  // Default tile widths per launch (BF16; an n_tile option overrides them): V takes 48
-  // columns when two accumulator sets then fit TMEM, so that its heavy epilogue (T = V/D,
-  // two stores per element) overlaps the next chunk's MMAs; Gamma, with K = nocc x nvir,
-  // takes 80, whose wider B tiles cut its operand traffic; P_ab / P_ij keep 64.  Measured
-  // by the autotuner at nocc=100 nvir=500 naux=1500 (5 / 6 / 5 slices): V 44.8 ms against
-  // 45.8 at 64 columns, Gamma 74 against 80 ms.
+  // First tile widths per launch (BF16; an n_tile option overrides them): Gamma, with K =
+  // nocc x nvir, takes 80 columns, whose wider B tiles cut its operand traffic (nocc=100
+  // nvir=500 naux=1500: 74 ms against 80 at 64); P_ab / P_ij keep 64; V: split_shape_v.
   int nv = opt.n_tile, ng = opt.n_tile;
   if (!sp.fp8 && opt.n_tile == 0) {
     nv = 2 * sp.slices_v * 48 <= 512 ? 48 : 0;
@@ -863,6 +860,38 @@ int split_plan_init(SplitPlan& sp, int precision, const rimp2_options& opt) {
   if (split_gemm_prepare() != cudaSuccess) { cudaGetLastError(); return RIMP2_ERR_CUDA; }
   sp.ready = true;
   return RIMP2_OK;
+}
+
+// V's tile width before any tuning.  Its operands come from L2, (128 + n_tile) rows for
+// 128 x n_tile results, and bound a launch of many tiles; wider tiles need less of them, but
+// leave SMs idle where the tiles are few, spend longer in an epilogue where K is short, and
+// with up to 5 slices only 48 columns leave TMEM for a second accumulator set, which a K of
+// more than two chunks (512 each, drained by 8 warps from 1024 on) needs.  Measured, BF16 with
+// 5 slices at 48 / 64 / 80 columns: nocc=10 nvir=40 naux=150 31 / 33 / 43 us, nocc=20 nvir=80
+// naux=300 46 / 49 / 57 us, nocc=29 nvir=117 naux=437 111 / 110 / 125 us, 40 MBE3 dimers (naux
+// about 420) 3.58 / 3.21 / 3.22 ms, nocc=42 nvir=168 naux=630 453 / 442 / 428 us, nocc=50
+// nvir=250 naux=750 1.46 / 1.38 / 1.30 ms, nocc=40 nvir=160 naux=1200 627 / 713 / 776 us,
+// nocc=100 nvir=500 naux=1500 40.3 / 45.0 / 48.8 ms.  8 slices at 48 / 64: nocc=20 55 / 66 us,
+// nocc=29 174 / 162, nocc=42 854 / 768 us; FP8 with 8 slices: nocc=20 47 / 57 us, nocc=29 119 /
+// 121, nocc=42 480 / 442 us.
+void split_shape_v(SplitPlan& sp, const rimp2_options& opt, const rimp2_frag* frags, int nfrag) {
+  if (opt.n_tile != 0) return;
+  double tiles = 0.0, blocks = 0.0;   // tiles of 128 x 48 with results; times naux
+  for (int f = 0; f < nfrag; ++f) {
+    const double ov = (double)frags[f].nocc * frags[f].nvir, t = ov * (ov + SG_BM) / (2.0 * SG_BM * 48);
+    tiles += t;
+    blocks += t * frags[f].naux;
+  }
+  const bool two = !sp.fp8 && 2 * sp.slices_v * 48 <= 512;
+  const int want = tiles < 4.0 * sp.grid || (two && blocks > 1024.0 * tiles) ? 48
+                   : two && blocks >= 576.0 * tiles                       ? 80
+                                                                          : 64;
+  for (int nt : {want, 64, 48})
+    for (size_t i = 0; i < sp.cand_v.size(); ++i)
+      if (sp.cand_v[i].n_tile_max == nt && sp.cand_v[i].bk == sp.cand_v[0].bk) {
+        split_set_shapes(sp, (int)i, 0, 0);
+        return;
+      }
 }
 
 void split_plan_release(SplitPlan&) {}

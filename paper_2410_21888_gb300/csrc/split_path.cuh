@@ -50,8 +50,8 @@ struct SplitPlan {
   bool ready = false;
   bool fp8 = false;  // RIMP2_FP8_SPLIT: e4m3 digits
   int variant = 0;   // contraction-stage variant (autotuner), see split_variant_desc
-  // tile shapes (n_tile, K per stage) the autotuner trials per launch, the configured
-  // default first, and the index of each launch's shape in use
+  // tile shapes (n_tile, K per stage) the autotuner trials per launch and the index of each
+  // launch's shape in use (tuning records keep indices: the order of the lists stays)
   std::vector<SplitLaunch> cand_v, cand_t, cand_g;
   int shape_v = 0, shape_t = 0, shape_g = 0;
 };
@@ -59,6 +59,8 @@ struct SplitPlan {
 // Selects the tile shapes of the V, P_ab / P_ij and Gamma launches (indices into the
 // candidate lists, clamped to their ends).
 void split_set_shapes(SplitPlan& sp, int iv, int it, int ig);
+// The V launch's shape for a plan of these fragments
+void split_shape_v(SplitPlan& sp, const rimp2_options& opt, const rimp2_frag* frags, int nfrag);
 
 // Variants of the Gamma/P contraction stage the autotuner times:
 //   0: P_ij rows read through the local (k,b)-major view, split-K target 8 x grid
