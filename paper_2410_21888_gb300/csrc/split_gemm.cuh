@@ -36,9 +36,8 @@ constexpr int SG_LB_FP8 = 5, SG_CHUNK_K_FP8 = 8192, SG_HEAD_FP8 = 0;
 // K per pipeline stage: 32 (64-byte rows, 64B swizzle) or 16 (32-byte rows, 32B swizzle);
 // the smaller stage fits twice as many stages in shared memory
 constexpr int SG_MAX_SLICES = 16;   // FP8; BF16 stops at 8
-// warp 0 TMA, warp 1 MMA, then the epilogue warps: 8 or 16 per launch (SplitLaunch::
-// epi_warps), each of the four TMEM lane quadrants served by 2 or 4 warps that split the
-// tile's columns between them
+// warp 0 TMA, warp 1 MMA, then the epilogue warps: 16 (8 with 16-wide K stages), each of the
+// four TMEM lane quadrants served by 4 (2) warps that split the tile's columns between them
 
 // TMA coordinate modes of one operand
 enum : int {
@@ -86,7 +85,6 @@ struct SplitLaunch {
   int n_tile_max; // widest n_tile of the launch (smem layout)
   int stages;     // pipeline depth
   size_t smem;    // dynamic shared memory bytes
-  int epi_warps;  // epilogue warps: 8, or 16 (more warps for a tile's drain and epilogue)
   // the launch before in the stream is another contraction of the same call, on which this
   // one doesn't depend: this one's CTAs fill the SMs that it leaves (see pdl_trigger)
   bool beside;

@@ -864,16 +864,14 @@ int split_plan_init(SplitPlan& sp, int precision, const rimp2_options& opt) {
 
 // V's tile width before any tuning.  Its operands come from L2, (128 + n_tile) rows for
 // 128 x n_tile results, and bound a launch of many tiles; wider tiles need less of them, but
-// leave SMs idle where the tiles are few, spend longer in an epilogue where K is short, and
-// with up to 5 slices only 48 columns leave TMEM for a second accumulator set, which a K of
-// more than two chunks (512 each, drained by 8 warps from 1024 on) needs.  Measured, BF16 with
-// 5 slices at 48 / 64 / 80 columns: nocc=10 nvir=40 naux=150 31 / 33 / 43 us, nocc=20 nvir=80
-// naux=300 46 / 49 / 57 us, nocc=29 nvir=117 naux=437 111 / 110 / 125 us, 40 MBE3 dimers (naux
-// about 420) 3.58 / 3.21 / 3.22 ms, nocc=42 nvir=168 naux=630 453 / 442 / 428 us, nocc=50
-// nvir=250 naux=750 1.46 / 1.38 / 1.30 ms, nocc=40 nvir=160 naux=1200 627 / 713 / 776 us,
-// nocc=100 nvir=500 naux=1500 40.3 / 45.0 / 48.8 ms.  8 slices at 48 / 64: nocc=20 55 / 66 us,
-// nocc=29 174 / 162, nocc=42 854 / 768 us; FP8 with 8 slices: nocc=20 47 / 57 us, nocc=29 119 /
-// 121, nocc=42 480 / 442 us.
+// leave SMs idle where the tiles are few and, with 5 slices, spend longer in the epilogue of a
+// short K (48 columns leave TMEM for a second accumulator set, which hides it).  Measured, BF16
+// with 5 slices at 48 / 64 / 80 columns: nocc=10 nvir=40 naux=150 31 / 33 / 43 us, nocc=20
+// nvir=80 naux=300 46 / 49 / 57 us, nocc=29 nvir=117 naux=437 111 / 110 / 125 us, 40 MBE3 dimers
+// (naux about 420) 3.58 / 3.21 / 3.22 ms, nocc=42 nvir=168 naux=630 453 / 442 / 428 us, nocc=50
+// nvir=250 naux=750 1.46 / 1.38 / 1.30 ms, nocc=100 nvir=500 naux=1500 38.9 / 37.2 / 34.3 ms
+// (96 columns: 35.6).  8 slices at 48 / 64: nocc=20 55 / 66 us, nocc=29 174 / 162, nocc=42 854 /
+// 768 us; FP8 with 8 slices: nocc=20 47 / 57 us, nocc=29 119 / 121, nocc=42 480 / 442 us.
 void split_shape_v(SplitPlan& sp, const rimp2_options& opt, const rimp2_frag* frags, int nfrag) {
   if (opt.n_tile != 0) return;
   double tiles = 0.0, blocks = 0.0;   // tiles of 128 x 48 with results; times naux
@@ -883,9 +881,7 @@ void split_shape_v(SplitPlan& sp, const rimp2_options& opt, const rimp2_frag* fr
     blocks += t * frags[f].naux;
   }
   const bool two = !sp.fp8 && 2 * sp.slices_v * 48 <= 512;
-  const int want = tiles < 4.0 * sp.grid || (two && blocks > 1024.0 * tiles) ? 48
-                   : two && blocks >= 576.0 * tiles                       ? 80
-                                                                          : 64;
+  const int want = tiles < 4.0 * sp.grid ? 48 : two && blocks >= 576.0 * tiles ? 80 : 64;
   for (int nt : {want, 64, 48})
     for (size_t i = 0; i < sp.cand_v.size(); ++i)
       if (sp.cand_v[i].n_tile_max == nt && sp.cand_v[i].bk == sp.cand_v[0].bk) {
@@ -1290,15 +1286,8 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
         if (d.idx == P.frag) d.zero_gamma = 1;
     }
   }
-  // Sixteen epilogue warps when every fragment's aux dimension is short: V's tiles then
-  // have little K for their MMAs to hide the T = V/D epilogue behind, which more warps
-  // share (MBE3 stated batch: dimer level 86.1 -> 79.3 ms); with naux ~1500 the extra
-  // warps cost V's MMA issuer a little (41.6 -> 42.2 ms at nocc=100 nvir=500).
-  {
-    w.max_x = 0;
-    for (const auto& s : w.sfd) w.max_x = std::max(w.max_x, s.X);
-    w.epi_warps = w.max_x <= 1024 ? 16 : 8;
-  }
+  w.max_x = 0;
+  for (const auto& f : w.sfd) w.max_x = std::max(w.max_x, f.X);
   // Amplitude stage: CTAs (i, j range, strip).  One range of all j where the strips alone make
   // eight rounds of three CTAs per SM (a shorter last round costs less of the whole); shorter
   // ranges, down to one j, for smaller waves
@@ -1397,11 +1386,9 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long lon
   }
   if (ev) cudaEventRecordWithFlags(ev[1], s, cudaEventRecordExternal);
   if (e == cudaSuccess && w.tiles_v > 0) {
-    SplitLaunch cfg = sp.cfg_v;
-    cfg.epi_warps = w.epi_warps;
     e = launch_split_gemm((const SplitProb*)(dblk + w.off_pv), (const long long*)(dblk + w.off_bv),
                           (int)w.probs_v.size(), w.tiles_v, bs,
-                          ctr + 0, cfg, sp.grid, s);
+                          ctr + 0, sp.cfg_v, sp.grid, s);
     ++nl;
   }
   if (ev) cudaEventRecordWithFlags(ev[2], s, cudaEventRecordExternal);
@@ -1423,11 +1410,9 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long lon
   // the next one's CTAs take the SMs that the one before leaves (at nocc=10 nvir=40 all 134 CTAs
   // of both run at once).  Events between the launches keep them apart.
   if (e == cudaSuccess && w.tiles_c > 0) {
-    SplitLaunch cfg = sp.cfg_t;
-    cfg.epi_warps = w.epi_warps;
     e = launch_split_gemm((const SplitProb*)(dblk + w.off_pc), (const long long*)(dblk + w.off_bc),
                           (int)w.probs_c.size(), w.tiles_c, bs,
-                          ctr + 1, cfg, sp.grid, s);
+                          ctr + 1, sp.cfg_t, sp.grid, s);
     ++nl;
   }
   if (e == cudaSuccess && w.tiles_s > 0) {
@@ -1439,7 +1424,6 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long lon
   if (ev) cudaEventRecordWithFlags(ev[4], s, cudaEventRecordExternal);
   if (e == cudaSuccess && w.tiles_g > 0) {
     SplitLaunch cfg = sp.cfg_g;
-    cfg.epi_warps = w.epi_warps;
     cfg.beside = !ev && (w.tiles_c > 0 || w.tiles_s > 0);
     e = launch_split_gemm((const SplitProb*)(dblk + w.off_pg), (const long long*)(dblk + w.off_bg),
                           (int)w.probs_g.size(), w.tiles_g, bs,

@@ -78,7 +78,6 @@ struct SplitWave {
   bool want_gamma = false;
   int max_x = 0;       // largest naux of the wave
   int amp_lpr = 32;    // lanes per row of the amplitude kernel
-  int epi_warps = 8;   // epilogue warps of the wave's contraction launches (see build)
   double mma_v = 0, mma_c = 0, mma_g = 0;   // tensor-core FLOPs issued per launch
   int stack_rows = 0;  // most rows a slice among probs_s
   size_t off_sfd = 0, off_pv = 0, off_pc = 0, off_pg = 0, off_ps = 0, off_bs = 0;  // byte offsets in the device block

@@ -21,7 +21,7 @@ def _run(dims, n, precision, **kw):
 @pytest.mark.parametrize("dims,n,precision,slices,width", [
     ((6, 21, 50), 1, "bf16", 0, 48), ((10, 90, 70), 3, "bf16", 0, 48),     # few tiles
     ((10, 90, 70), 14, "bf16", 0, 64), ((10, 90, 576), 14, "bf16", 0, 80),
-    ((10, 90, 575), 14, "bf16", 0, 64), ((10, 90, 1025), 14, "bf16", 0, 48),
+    ((10, 90, 575), 14, "bf16", 0, 64), ((10, 90, 1025), 14, "bf16", 0, 80),
     ((10, 90, 1025), 14, "bf16", 8, 64), ((6, 21, 50), 1, "bf16", 8, 48),
     ((6, 21, 50), 1, "fp8", 0, 48), ((10, 90, 600), 14, "fp8", 0, 64)])
 def test_width(dims, n, precision, slices, width):
