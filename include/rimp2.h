@@ -118,8 +118,8 @@ typedef struct rimp2_options {
                           launch - V, P_ab / P_ij, Gamma - takes its own i-th candidate of
                           n_tile x stage_k that fits TMEM), then the other variants of the
                           Gamma/P contraction stage (operand view of P_ij, split-K factor,
-                          Gamma slabs) with each launch's fastest shape; FP64: the split-K
-                          factor.  Results are identical up to rounding order. */
+                          Gamma slabs) with each launch's fastest shape; FP64: the work
+                          items per SM.  Results are identical up to rounding order. */
   int32_t profile_stages; /* 1: record CUDA events between the stages of each call so that
                              rimp2_get_stats reports stage_ms (default 0) */
   size_t max_workspace_bytes; /* 0: one wave for the whole batch; else waves sized so
@@ -160,9 +160,11 @@ typedef struct rimp2_stats {
   int32_t tune_done;       /* 1 once the autotune trials finished (or were cached) */
   double tune_ms[4];       /* autotune: contraction-stage ms measured for each variant */
   double stage_ms[4];      /* with profile_stages: device ms of the last call, summed over
-                              waves: [0] input checks and operand slicing, [1] V GEMM with the
-                              T = V/D epilogue, [2] amplitudes, pair/total energies, zeroing,
-                              [3] Gamma / P_ab / P_ij contractions */
+                              waves: [0] input checks, zeroing (FP64) and slicing of V's operand,
+                              [1] V GEMM with the T = V/D epilogue, [2] amplitudes, pair/total
+                              energies, split modes also zeroing and slicing of Gamma's operand
+                              B, [3] Gamma / P_ab / P_ij contractions (which overlap, and so
+                              take a little less, in a plan without profile_stages) */
   int32_t slices[3];       /* split modes: digit slices in use for V, P_ab / P_ij, Gamma */
   int32_t pad;
   double launch_ms[2];     /* with profile_stages: stage [3] split by launch: [0] the P_ab /

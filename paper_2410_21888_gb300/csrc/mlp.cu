@@ -7,7 +7,7 @@
 // of a sample and reading weights and activations as 16-byte rows; the latency of a tile's
 // layer chain bounds a minibatch.  (One warp per sample with the weights as W[unit][k] rows,
 // 32-way bank conflicts and five shuffles per weight row, took 1362 us for the gradient of a
-// 512-sample minibatch, the tiles 15 us; a whole training step fell from 1370 to 28 us.)
+// 512-sample minibatch, the tiles 15 us; a whole training step fell from 1370 to 21 us.)
 // Prediction and features: see k_mlp_predict and log10_pos.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

@@ -469,7 +469,7 @@ __device__ __forceinline__ int find_problem(const SplitProb* __restrict__ probs,
 
 // a / b, 0 <= a, b: in 32 bits where both fit, which they practically always do (a 64-bit
 // division is some hundred dependent instructions, and a tile's decoding had four: 40 MBE3
-// dimers' Gamma 4.02 -> 3.95 ms, 100 trimers' V 12.50 -> 12.32 ms, nocc=42 FP8 P and Gamma
+// dimers' Gamma 4.02 -> 3.95 ms, 16 trimers' V 12.50 -> 12.32 ms, nocc=42 FP8 P and Gamma
 // 1.68 -> 1.64 ms)
 __device__ __forceinline__ long long div_pos(long long a, long long b) {
   return ((a | b) >> 32) == 0 ? (long long)((unsigned)a / (unsigned)b) : a / b;
