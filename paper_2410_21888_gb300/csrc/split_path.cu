@@ -528,6 +528,49 @@ __device__ __forceinline__ void slice_b2(const SplitFragDev* __restrict__ f, int
   }
 }
 
+// Exponent of T's scale from the largest |T|'s
+template <bool F8>
+__device__ __forceinline__ int t_scale(unsigned emax) {
+  return Digit<F8>::LB - ((int)emax - 124 + Digit<F8>::HEAD);
+}
+
+// Pair energies e_ij, j >= i, and their opposite-spin parts: the amplitude warps' shares of row
+// i summed in a fixed order (FP64) by warp w of nw; strips: row strips of the fragment, kt: the
+// exponent of T's scale
+__device__ __forceinline__ void row_energies(const SplitFragDev& F, char* ws, int i, int w, int nw, int strips,
+                                             int kt) {
+  const int o = F.o, lane = threadIdx.x & 31;
+  double* ep = (double*)(ws + F.ep);
+  const int parts = F.v > 0 ? strips * 8 : 0;
+  for (int j0 = i + 4 * w; j0 < o; j0 += 4 * nw) {   // eight lanes a pair
+    const int jj = j0 + (lane >> 3);
+    double e = 0.0, eo = 0.0;
+    if (jj < o) {
+      const float4* p = (const float4*)(ws + F.epart) + ((long long)i * o + jj) * (strips * 8);
+#pragma unroll 4
+      for (int k = lane & 7; k < parts; k += 8) {
+        const float4 x = __ldcg(p + k);
+        e += (double)x.x + (double)x.y;
+        eo += (double)x.z + (double)x.w;
+      }
+    }
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) {
+      e += __shfl_xor_sync(0xffffffffu, e, off);
+      eo += __shfl_xor_sync(0xffffffffu, eo, off);
+    }
+    if (jj < o && (lane & 7) == 0) {
+      e = ldexp(e, 1 - 2 * kt);   // the scales of T and Tt
+      eo = ldexp(eo, -2 * kt);
+      ep[(long long)i * o + jj] = e;
+      ep[(long long)jj * o + i] = e;
+      double* eq = ep + (long long)o * o;   // opposite-spin pair energies
+      eq[(long long)i * o + jj] = eo;
+      eq[(long long)jj * o + i] = eo;
+    }
+  }
+}
+
 // Amplitude stage: Tt = 2T - T^T, digits of T and Tt (one scale per fragment each), pair
 // energies e_ij = sum_ab Tt_ij(a,b) V_ij(a,b) (V = T D) and their opposite-spin part
 // sum_ab T_ij(a,b) V_ij(a,b) for i <= j.
@@ -548,7 +591,7 @@ __device__ __forceinline__ void slice_b2(const SplitFragDev* __restrict__ f, int
 // LPR: lanes per row, 32, or fewer where the rows are short (amp_lanes).
 template <bool F8, int LPR>
 __global__ void __launch_bounds__(256, 3)
-k_amp_split(const SplitFragDev* __restrict__ f, int nf, unsigned amp_ctas, int sg, Bases bs) {
+k_amp_split(const SplitFragDev* __restrict__ f, int nf, unsigned amp_ctas, int sg, int sums, Bases bs) {
   using DT = typename Digit<F8>::T;
   constexpr int LB = Digit<F8>::LB;
   constexpr int GROUPS = 32 / LPR, ROWS = 8 * GROUPS, C = 4 * LPR;
@@ -590,7 +633,7 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, unsigned amp_ctas, int s
   // 2^(kt - 1) of Tt keep both within 2^(E - 2 - HEAD) and 2^(E - 1 - HEAD).  T_ij(b,a) is
   // scaled by the latter, so that Tt = 2T - T^T is a plain difference of scaled values, and the
   // energies are formed from the scaled T and Tt (all exact powers of two).
-  const int kt = LB - ((int)emax - 124 + Digit<F8>::HEAD);
+  const int kt = t_scale<F8>(emax);
   const bool one = kt <= 126 && kt >= -125;   // 2^kt is a normal float (unless |T| < 2^-121)
   float sa, sb;
   pow2_factors(kt, sa, sb);
@@ -741,7 +784,8 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, unsigned amp_ctas, int s
       e_h = e_l = o_h = o_l = 0ull;
     }
   }
-  // the last CTA of row i sums the warps' shares of e_ij, j >= i, in a fixed order (FP64)
+  if (!sums) return;   // k_split_energy's
+  // the last CTA of row i sums the warps' shares of e_ij, j >= i
   __threadfence();
   __syncthreads();
   if (tid == 0)
@@ -749,35 +793,7 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, unsigned amp_ctas, int s
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  double* ep = (double*)(ws + F.ep);
-  const int parts = v > 0 ? strips * 8 : 0;
-  for (int j0 = i + 4 * warp; j0 < o; j0 += 32) {   // eight lanes a pair
-    const int jj = j0 + (lane >> 3);
-    double e = 0.0, eo = 0.0;
-    if (jj < o) {
-      const float4* p = (const float4*)(ws + F.epart) + ((long long)i * o + jj) * (strips * 8);
-#pragma unroll 4
-      for (int k = lane & 7; k < parts; k += 8) {
-        const float4 w = __ldcg(p + k);
-        e += (double)w.x + (double)w.y;
-        eo += (double)w.z + (double)w.w;
-      }
-    }
-#pragma unroll
-    for (int off = 4; off > 0; off >>= 1) {
-      e += __shfl_xor_sync(0xffffffffu, e, off);
-      eo += __shfl_xor_sync(0xffffffffu, eo, off);
-    }
-    if (jj < o && (lane & 7) == 0) {
-      e = ldexp(e, 1 - 2 * kt);   // the scales of T and Tt
-      eo = ldexp(eo, -2 * kt);
-      ep[(long long)i * o + jj] = e;
-      ep[(long long)jj * o + i] = e;
-      double* eq = ep + (long long)o * o;   // opposite-spin pair energies
-      eq[(long long)i * o + jj] = eo;
-      eq[(long long)jj * o + i] = eo;
-    }
-  }
+  row_energies(F, ws, i, warp, 8, strips, kt);
   // the last row's CTA sums the fragment's energies
   __threadfence();
   __syncthreads();
@@ -785,7 +801,33 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, unsigned amp_ctas, int s
   __syncthreads();
   if (!s_last) return;
   __threadfence();
+  const double* ep = (const double*)(ws + F.ep);
   fragment_energy(ep, ep + (long long)o * o, (long long)o * o,
+                  F.epair_off >= 0 ? bs.epair + F.epair_off : nullptr, F.idx, bs);
+}
+
+// The energies of small fragments, a CTA each, beside the contractions that follow (they start
+// as soon as this kernel's CTAs have).  Counted down by the amplitude CTAs, row by row and then
+// for the fragment, the sums are a chain of fences and FP64 latencies that P and Gamma would
+// wait for.  A call (BF16) at nocc=4 65 -> 59 us, nocc=10 nvir=40 naux=150 88 -> 78, nocc=24
+// nvir=96 naux=360 343 -> 328; from nocc=32 on nothing is left of it, and one CTA is too few for
+// many pairs of a short call (nocc=100 nvir=20 naux=200 342 -> 581 us): up to kSepOcc.
+constexpr int kSepOcc = 24;
+
+template <bool F8>
+__global__ void __launch_bounds__(256)
+k_split_energy(const SplitFragDev* __restrict__ f, int lpr, Bases bs) {
+  pdl_trigger();
+  const SplitFragDev& F = f[blockIdx.x];
+  if (F.o == 0) return;   // the prologue's
+  char* ws = (char*)bs.ws;
+  const int warp = threadIdx.x >> 5, rows = 8 * 32 / lpr, strips = max(1, (F.v + rows - 1) / rows);
+  const int kt = t_scale<F8>(*(const unsigned*)(ws + F.scal + 4));
+  for (int i = warp; i < F.o; i += 8) row_energies(F, ws, i, 0, 1, strips, kt);
+  __threadfence_block();
+  __syncthreads();
+  const double* ep = (const double*)(ws + F.ep);
+  fragment_energy(ep, ep + (long long)F.o * F.o, (long long)F.o * F.o,
                   F.epair_off >= 0 ? bs.epair + F.epair_off : nullptr, F.idx, bs);
 }
 
@@ -1308,6 +1350,8 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
   w.rows = rows;
   w.b2_tiles = b2t;
   w.qblks = qbl;
+  w.sep_energy = !w.probs_c.empty() || !w.probs_s.empty() || !w.probs_g.empty();
+  for (const auto& d : w.sfd) w.sep_energy = w.sep_energy && d.o <= kSepOcc;
   finish(w.probs_v, w.tiles_v);
   finish(w.probs_c, w.tiles_c);
   finish(w.probs_g, w.tiles_g);
@@ -1395,7 +1439,7 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long lon
   if (e == cudaSuccess && total_pairs > 0) {
     const unsigned ctas = (unsigned)total_pairs;
     auto amp = [&](auto kernel) {
-      kernel<<<ctas + (unsigned)w.b2_tiles, 256, 0, s>>>(sfd, nf, ctas, sp.slices_g, bs);
+      kernel<<<ctas + (unsigned)w.b2_tiles, 256, 0, s>>>(sfd, nf, ctas, sp.slices_g, !w.sep_energy, bs);
     };
     switch (w.amp_lpr) {
       case 8: sp.fp8 ? amp(k_amp_split<true, 8>) : amp(k_amp_split<false, 8>); break;
@@ -1404,27 +1448,38 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long lon
     }
     ++nl;
     e = cudaGetLastError();
+    if (e == cudaSuccess && w.sep_energy) {
+      if (sp.fp8) k_split_energy<true><<<(unsigned)nf, 256, 0, s>>>(sfd, w.amp_lpr, bs);
+      else k_split_energy<false><<<(unsigned)nf, 256, 0, s>>>(sfd, w.amp_lpr, bs);
+      ++nl;
+      e = cudaGetLastError();
+    }
   }
   if (ev) cudaEventRecordWithFlags(ev[3], s, cudaEventRecordExternal);
   // The P launches and Gamma's read what the amplitude launch wrote and nothing of each other:
   // the next one's CTAs take the SMs that the one before leaves (at nocc=10 nvir=40 all 134 CTAs
   // of both run at once).  Events between the launches keep them apart.
+  bool beside = !ev && w.sep_energy;
   if (e == cudaSuccess && w.tiles_c > 0) {
+    SplitLaunch cfg = sp.cfg_t;
+    cfg.beside = beside;
     e = launch_split_gemm((const SplitProb*)(dblk + w.off_pc), (const long long*)(dblk + w.off_bc),
                           (int)w.probs_c.size(), w.tiles_c, bs,
-                          ctr + 1, sp.cfg_t, sp.grid, s);
+                          ctr + 1, cfg, sp.grid, s);
+    beside = !ev;
     ++nl;
   }
   if (e == cudaSuccess && w.tiles_s > 0) {
     e = launch_split_stack((const SplitProb*)(dblk + w.off_ps), (const long long*)(dblk + w.off_bs),
                            (int)w.probs_s.size(), w.tiles_s, bs, ctr + 3, sp.slices_t, w.stack_rows,
-                           sp.fp8, sp.grid, !ev && w.tiles_c > 0, s);
+                           sp.fp8, sp.grid, beside, s);
+    beside = !ev;
     ++nl;
   }
   if (ev) cudaEventRecordWithFlags(ev[4], s, cudaEventRecordExternal);
   if (e == cudaSuccess && w.tiles_g > 0) {
     SplitLaunch cfg = sp.cfg_g;
-    cfg.beside = !ev && (w.tiles_c > 0 || w.tiles_s > 0);
+    cfg.beside = beside;
     e = launch_split_gemm((const SplitProb*)(dblk + w.off_pg), (const long long*)(dblk + w.off_bg),
                           (int)w.probs_g.size(), w.tiles_g, bs,
                           ctr + 2, cfg, sp.grid, s);

@@ -73,6 +73,7 @@ constexpr int kSplitVariants = 4;
 struct SplitWave {
   std::vector<SplitFragDev> sfd;
   std::vector<SplitProb> probs_v, probs_c, probs_g;   // V; P_ab / P_ij; Gamma
+  bool sep_energy = false;   // energies by k_split_energy instead of the last amplitude CTAs
   std::vector<SplitProb> probs_s;   // P_ab / P_ij of small extents (slice-stacked kernel)
   long long tiles_v = 0, tiles_c = 0, tiles_g = 0, tiles_s = 0, rows = 0, b2_tiles = 0, qblks = 0;
   bool want_gamma = false;
