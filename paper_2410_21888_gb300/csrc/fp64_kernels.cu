@@ -28,7 +28,7 @@ __device__ __forceinline__ int find_frag(const FragDev* __restrict__ frags, int 
 
 __global__ void __launch_bounds__(256, F64_CTAS)
 k_gemm_f64(const GemmProb* __restrict__ probs, int nprobs, long long total, Bases bs,
-           unsigned* __restrict__ counter) {
+           unsigned* __restrict__ counter, int beside) {
   __shared__ F64Smem sm;
   __shared__ F64Entry e;
   for (;;) {
@@ -38,6 +38,7 @@ k_gemm_f64(const GemmProb* __restrict__ probs, int nprobs, long long total, Base
     f64_item(e.P, bs, e.tm, e.tn, e.ks, sm);
     __syncthreads();  // the shared tile and descriptor are rewritten for the next item
   }
+  if (beside) pdl_wait();
 }
 
 // Tile width, K pieces and queue position of every problem of one launch (sorted longest
@@ -130,14 +131,49 @@ int gemm_f64_occupancy_grid() {
 }
 
 cudaError_t launch_gemm_f64(const GemmProb* d_probs, int nprobs, long long total_tiles,
-                            Bases bs, unsigned* counter, int grid, cudaStream_t s) {
+                            Bases bs, unsigned* counter, int grid, cudaStream_t s, bool beside) {
   if (total_tiles <= 0) return cudaSuccess;
   const long long g = total_tiles < grid ? total_tiles : grid;
-  k_gemm_f64<<<(unsigned)g, 256, 0, s>>>(d_probs, nprobs, total_tiles, bs, counter);
-  return cudaGetLastError();
+  return launch_pdl(k_gemm_f64, (unsigned)g, 256, 0, s, beside, d_probs, nprobs, total_tiles, bs, counter,
+                    (int)beside);
 }
 
 // ------------------------------------------------------------------ amplitudes
+
+__device__ __forceinline__ void put_pair(const FragDev& F, const Bases& bs, int a, int b, double e, double eos) {
+  double* ep = bs.ws + F.ep_off;
+  ep[(long long)a * F.o + b] = e;
+  ep[(long long)b * F.o + a] = e;
+  if (F.epos_off >= 0) {
+    double* eq = bs.ws + F.epos_off;
+    eq[(long long)a * F.o + b] = eos;
+    eq[(long long)b * F.o + a] = eos;
+  }
+}
+
+// The energies of a fragment, by one CTA of 256 threads, when its amplitude CTAs have ended:
+// their shares of each pair energy (cut pairs) are added in a fixed order
+__device__ __forceinline__ void sum_energies(const FragDev& F, const Bases& bs) {
+  if (F.amp_split > 1) {
+    const long long npair = (long long)F.o * (F.o + 1) / 2;
+    for (long long p = threadIdx.x; p < npair; p += 256) {
+      const double2* w = (const double2*)(bs.ws + F.part_off) + p * F.amp_split;
+      double e = 0.0, eos = 0.0;
+      for (int k = 0; k < F.amp_split; ++k) {
+        const double2 x = __ldcg(w + k);
+        e += x.x;
+        eos += x.y;
+      }
+      int a, b;
+      tri_index(p, a, b);
+      put_pair(F, bs, a, b, e, eos);
+    }
+    __threadfence_block();
+    __syncthreads();
+  }
+  fragment_energy(bs.ws + F.ep_off, F.epos_off >= 0 ? bs.ws + F.epos_off : nullptr, (long long)F.o * F.o,
+                  F.epair_off >= 0 ? bs.epair + F.epair_off : nullptr, F.idx, bs);
+}
 
 // One CTA per pair block (i <= j) of one fragment and share of its 32 x 32 tile pairs.  Reads
 // T_ij and writes Tt_ij = 2 T_ij - T_ij^T for the (i,j) block and, if i != j, Tt_ji = Tt_ij^T
@@ -147,15 +183,14 @@ cudaError_t launch_gemm_f64(const GemmProb* d_probs, int nprobs, long long total
 // in a lane and short across lanes.  A wave of few pairs cuts them over several CTAs
 // (amp_split; 55 pairs of nocc=10 nvir=40 on 55 SMs took 15 us).  Cut pairs of a narrow v are
 // taken element by element: no idle lanes at tile edges, and the strided accesses of
-// T_ij(b,a) and Tt_ji(b,a) stay in the lines of one block of at most 32 KB.  Where the
-// fragment has a counter (cnt_off), its last CTA adds the shares in a fixed order and sums the
-// fragment's energies.
+// T_ij(b,a) and Tt_ji(b,a) stay in the lines of one block of at most 32 KB.  The energies are
+// k_energy_reduce's: sums by the last CTA to finish cost every CTA a fence and the
+// contractions their length (nocc=10 nvir=40 143 -> 137 us, nocc=100 nvir=20 2842 -> 2786).
 __global__ void __launch_bounds__(256)
 k_amplitude_f64(const FragDev* __restrict__ frags, int nfrag, Bases bs) {
   __shared__ double X[32][33];
   __shared__ double Y[32][33];
   __shared__ double red[2][256], sum[2];
-  __shared__ int s_last;
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
   const int f = find_frag(frags, nfrag, (long long)blockIdx.x, [](const FragDev& F) { return F.cta_begin; });
   const FragDev F = frags[f];
@@ -164,7 +199,7 @@ k_amplitude_f64(const FragDev* __restrict__ frags, int nfrag, Bases bs) {
   int i, j;
   tri_index(gp, i, j);
   const int v = F.v, o = F.o;
-  const long long ov = (long long)o * v, npair = (long long)o * (o + 1) / 2;
+  const long long ov = (long long)o * v;
   const double* __restrict__ T = bs.ws + F.t_off;
   double* __restrict__ Tt = bs.ws + (F.tt_off >= 0 ? F.tt_off : 0);   // unused if < 0
   const double* eo = bs.eps + F.eo_off;
@@ -260,45 +295,10 @@ k_amplitude_f64(const FragDev* __restrict__ frags, int nfrag, Bases bs) {
     if (tx == 0) sum[ty] = x;
   }
   __syncthreads();
-  double* ep = bs.ws + F.ep_off;
-  double* eq = F.epos_off >= 0 ? bs.ws + F.epos_off : nullptr;
-  auto put = [&](int a, int b, double e, double eos) {
-    ep[(long long)a * o + b] = e;
-    ep[(long long)b * o + a] = e;
-    if (eq) {
-      eq[(long long)a * o + b] = eos;
-      eq[(long long)b * o + a] = eos;
-    }
-  };
   if (tid == 0) {
-    if (F.amp_split == 1) put(i, j, sum[0], sum[1]);
+    if (F.amp_split == 1) put_pair(F, bs, i, j, sum[0], sum[1]);
     else ((double2*)(bs.ws + F.part_off))[gp * F.amp_split + share] = make_double2(sum[0], sum[1]);
   }
-  if (F.cnt_off < 0) return;
-  __threadfence();
-  __syncthreads();
-  if (tid == 0)
-    s_last = atomicAdd((unsigned*)(bs.ws + F.cnt_off), 1u) + 1u == (unsigned)(npair * F.amp_split);
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  if (F.amp_split > 1) {
-    for (long long p = tid; p < npair; p += 256) {
-      const double2* w = (const double2*)(bs.ws + F.part_off) + p * F.amp_split;
-      double e = 0.0, eos = 0.0;
-      for (int k = 0; k < F.amp_split; ++k) {
-        const double2 x = __ldcg(w + k);
-        e += x.x;
-        eos += x.y;
-      }
-      int a, b;
-      tri_index(p, a, b);
-      put(a, b, e, eos);
-    }
-    __threadfence_block();
-    __syncthreads();
-  }
-  fragment_energy(ep, eq, (long long)o * o, F.epair_off >= 0 ? bs.epair + F.epair_off : nullptr, F.idx, bs);
 }
 
 cudaError_t launch_amplitude_f64(const FragDev* d_frags, int nfrag, long long total_ctas, Bases bs,
@@ -310,11 +310,11 @@ cudaError_t launch_amplitude_f64(const FragDev* d_frags, int nfrag, long long to
 
 // ------------------------------------------------------------------ energy reduction
 
+// The energies, a CTA a fragment; the contractions that follow start beside it.
 __global__ void __launch_bounds__(256)
 k_energy_reduce(const FragDev* __restrict__ frags, Bases bs) {
-  const FragDev& F = frags[blockIdx.x];
-  fragment_energy(bs.ws + F.ep_off, F.epos_off >= 0 ? bs.ws + F.epos_off : nullptr,
-                  (long long)F.o * F.o, F.epair_off >= 0 ? bs.epair + F.epair_off : nullptr, F.idx, bs);
+  pdl_trigger();
+  sum_energies(frags[blockIdx.x], bs);
 }
 
 cudaError_t launch_energy_reduce(const FragDev* d_frags, int nfrag, Bases bs, cudaStream_t s) {
@@ -325,9 +325,8 @@ cudaError_t launch_energy_reduce(const FragDev* d_frags, int nfrag, Bases bs, cu
 
 // ------------------------------------------------------------------ prologue and input checks
 
-// What a call's first launch prepares: the wave's queue counters (ctr, eight; may be null),
-// the fragment's amplitude counter, zero P (and Gamma where it is accumulated), the energies of
-// a fragment without pairs.  check: denominators must be negative for every (i,j,a,b), i.e.
+// What a call's first launch prepares: the wave's queue counters (ctr, eight; may be null), zero
+// P (and Gamma where it is accumulated).  check: denominators must be negative for every (i,j,a,b), i.e.
 // max(eps_occ) < min(eps_vir); B and eps must be finite.  Violations set bits of the status
 // word.  (Seven launches a call of nocc=10 nvir=40 had three of these few microseconds each.)
 __global__ void __launch_bounds__(256)
@@ -342,14 +341,6 @@ k_prologue(const FragDev* __restrict__ frags, unsigned* ctr, int check, Bases bs
     for (long long e = first; e < (long long)F.v * F.v; e += stride) bs.pab[F.pab_off + e] = 0.0;
   if (F.zero_gamma)
     for (long long e = first; e < (long long)F.o * F.v * F.X; e += stride) bs.gamma[F.gamma_off + e] = 0.0;
-  if (F.cnt_off >= 0 && first == 0) {
-    *(unsigned*)(bs.ws + F.cnt_off) = 0u;
-    if (F.o == 0) {
-      bs.energy[F.idx] = 0.0;
-      if (bs.energy_os) bs.energy_os[F.idx] = 0.0;
-      if (bs.energy_scs) bs.energy_scs[F.idx] = 0.0;
-    }
-  }
   if (!check) return;
   bool bad_nf = false;
   const long long nb = (long long)F.o * F.v * F.X;

@@ -106,7 +106,7 @@ extern "C" int rimp2_energy_fp64_noalloc(int32_t nocc, int32_t nvir, int32_t nau
   fd.epair_off = epair ? 0 : -1;
   fd.cta_begin = 0;
   fd.amp_split = 1;
-  fd.part_off = fd.cnt_off = -1;
+  fd.part_off = -1;
   fd.epos_off = -1;
   GemmProb P{};
   long long tiles = 0;

@@ -138,12 +138,12 @@ size_t amp_part_elems(const rimp2_frag& f) {
 
 // Workspace of one fragment on the FP64 path; build_fp64_wave lays out exactly this:
 // T, Tt (when an output needs it), pair energies and their opposite-spin part, the amplitude
-// CTAs' shares of them and their counter.
+// CTAs' shares of them.
 size_t frag_ws_elems_fp64(const rimp2_frag& f) {
   const size_t ov = (size_t)f.nocc * f.nvir;
   return align_up(ov * ov, kAlignElems) * (wants_tt(f) ? 2 : 1) +
          align_up(2 * (size_t)f.nocc * f.nocc, kAlignElems) +
-         align_up(amp_part_elems(f) + 1, kAlignElems);
+         align_up(amp_part_elems(f), kAlignElems);
 }
 
 size_t frag_ws_elems(const rimp2_plan* p, const rimp2_frag& f) {
@@ -179,8 +179,7 @@ int build_fp64_wave(rimp2_plan* p, const rimp2_frag* frags, WaveDesc& w) {
     d.gamma_off = f.gamma_off; d.pij_off = f.pij_off; d.pab_off = f.pab_off;
     d.epair_off = f.epair_off;
     d.part_off = (long long)ws;
-    d.cnt_off = d.part_off + (long long)amp_part_elems(f);
-    ws += align_up(amp_part_elems(f) + 1, kAlignElems);
+    ws += align_up(amp_part_elems(f), kAlignElems);
     pairs += (long long)f.nocc * (f.nocc + 1) / 2;
     w.fdev.push_back(d);
     w.max_b = std::max<long long>(w.max_b, (long long)ov * f.naux);
@@ -332,10 +331,11 @@ int enqueue(rimp2_plan* p, const rimp2_batch* b, void* ws, cudaStream_t s) {
       launches += w.tiles_v > 0;
       if (ev) cudaEventRecordWithFlags(ev[2], s, cudaEventRecordExternal);
       if (e == cudaSuccess) { e = launch_amplitude_f64(dfd, nf, w.total_pairs, bs, s); launches += w.total_pairs > 0; }
+      if (e == cudaSuccess) { e = launch_energy_reduce(dfd, nf, bs, s); launches += nf > 0; }
       if (ev) cudaEventRecordWithFlags(ev[3], s, cudaEventRecordExternal);
       if (e == cudaSuccess) {
         e = launch_gemm_f64((const GemmProb*)(p->dblk + w.off_pc), (int)w.probs_c.size(), w.tiles_c,
-                            bs, ctr + 1, w.grid_c, s);
+                            bs, ctr + 1, w.grid_c, s, !ev && nf > 0);
         launches += w.tiles_c > 0;
       }
       tiles += w.tiles_v + w.tiles_c;

@@ -134,7 +134,6 @@ struct FragDev {
   long long gamma_off, pij_off, pab_off, epair_off;  // -1: not requested
   long long cta_begin;        // first amplitude CTA of the fragment
   long long part_off;         // double2 [pairs][amp_split]: the CTAs' shares of the pair energies
-  long long cnt_off;          // amplitude CTAs done, or -1: no fused energy sums
   int amp_split, zero_gamma;  // amplitude CTAs per pair; 1: Gamma is accumulated, zero it first
 };
 
@@ -173,8 +172,9 @@ cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size
 // ctr: eight queue counters to clear, or null; check: 1 for the input checks
 cudaError_t launch_prologue(const FragDev* d_frags, int nfrag, long long max_bx, unsigned* ctr, int check,
                             Bases bs, cudaStream_t s);
+// beside: the launch before in the stream calls pdl_trigger and the GEMM doesn't depend on it
 cudaError_t launch_gemm_f64(const GemmProb* d_probs, int nprobs, long long total_tiles,
-                            Bases bs, unsigned* counter, int grid, cudaStream_t s);
+                            Bases bs, unsigned* counter, int grid, cudaStream_t s, bool beside = false);
 int gemm_f64_occupancy_grid();
 // Work items per SM a launch is cut into (more: better balance, shorter items): nocc=29
 // nvir=117 naux=437 takes 10.35 ms for Gamma and P with 16, 11.1 with 8, 10.5 with 32.

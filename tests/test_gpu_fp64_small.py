@@ -1,5 +1,5 @@
 """Few pairs on the FP64 path: pairs cut over several amplitude CTAs, Gamma in two K pieces that
-are added into a zeroed output, energies summed by the last amplitude CTA.  Sizes around the
+are added into a zeroed output, energies summed beside the contractions.  Sizes around the
 shortest K that is cut (nocc nvir = 128), one and several 32-wide tiles, one pair and more pairs
 than CTAs.  A second run on new inputs must start from clean outputs and counters, and agree with
 the first call of a fresh plan to the bit (two Gamma pieces add in either order to the same sum).
