@@ -119,9 +119,12 @@ typedef struct rimp2_options {
                           n_tile x stage_k that fits TMEM), then the other variants of the
                           Gamma/P contraction stage (operand view of P_ij, split-K factor,
                           Gamma slabs) with each launch's fastest shape; FP64: the work
-                          items per SM.  Results are identical up to rounding order. */
+                          items per SM.  Results are identical up to rounding order.
+                          Events between the stages keep launches apart that otherwise
+                          overlap, so only the trials record them (and profile_stages) */
   int32_t profile_stages; /* 1: record CUDA events between the stages of each call so that
-                             rimp2_get_stats reports stage_ms (default 0) */
+                             rimp2_get_stats reports stage_ms (0 otherwise, but for the
+                             calls that run an autotune trial) (default 0) */
   size_t max_workspace_bytes; /* 0: one wave for the whole batch; else waves sized so
                                  the workspace stays below this many bytes */
   int32_t stage_k;     /* split modes: K elements per pipeline stage of the tensor-core
