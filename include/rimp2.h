@@ -131,10 +131,9 @@ typedef struct rimp2_options {
                           GEMM, 16 or 32 (0 = default 32) */
   int32_t n_tile;      /* BF16 split: columns per level accumulator of every launch, 48,
                           64, 80 or 96, at most the widest that fits TMEM for the slice
-                          count.  0 = per launch: V 48 when two sets of slices x 48
-                          accumulator columns fit the 512 TMEM columns (the MMAs of one
-                          512-long K chunk then run while the previous one is drained),
-                          a separate Gamma launch 80, P_ab / P_ij 64 */
+                          count.  0 = per launch: V 48 columns for few tiles, 64 or (long
+                          K) 80 for many, chosen for each wave, a separate Gamma launch
+                          80, P_ab / P_ij 64 */
   const char* autotune_cache; /* NULL, or a text file "<key> <variant>" per line: a plan
                                  whose key (precision, slices, shapes) is listed starts with
                                  that variant and skips the trials; new results are
@@ -178,7 +177,8 @@ typedef struct rimp2_stats {
                               included, skipped symmetric tiles excluded): [0] V, [1] the
                               P_ab / P_ij launch, [2] the separate Gamma launch, [3] unused */
   int32_t n_tile[3];       /* split modes: tile shape in use (accumulator columns, K per
-                              pipeline stage) of the V, P_ab / P_ij and Gamma launches */
+                              pipeline stage) of the V (several waves: the widest), P_ab /
+                              P_ij and Gamma launches */
   int32_t stage_k[3];
   int32_t tune_trials;     /* autotune: calls that run a trial (tile shapes, then variants) */
   int32_t pad2;

@@ -437,7 +437,13 @@ double span_ms(rimp2_plan* p, int a, int b) {
 
 void publish_shapes(rimp2_plan* p) {
   if (p->precision == RIMP2_FP64) return;
-  const SplitLaunch* c[3] = {&p->split.cfg_v, &p->split.cfg_t, &p->split.cfg_g};
+  // V: the widest of the waves'
+  const SplitLaunch* v = &p->split.cand_v[split_shape_v(p->split, p->frags.data(), p->wave_members[0])];
+  for (const auto& m : p->wave_members) {
+    const SplitLaunch& x = p->split.cand_v[split_shape_v(p->split, p->frags.data(), m)];
+    if (x.n_tile_max > v->n_tile_max) v = &x;
+  }
+  const SplitLaunch* c[3] = {v, &p->split.cfg_t, &p->split.cfg_g};
   for (int i = 0; i < 3; ++i) {
     p->stats.n_tile[i] = c[i]->n_tile_max;
     p->stats.stage_k[i] = c[i]->bk;
@@ -499,7 +505,6 @@ int rimp2_plan_create(const rimp2_frag* frags, int32_t nfrag, int32_t precision,
   if (precision != RIMP2_FP64) {
     rc = split_plan_init(p->split, precision, o);
     if (rc != RIMP2_OK) { delete p; return rc; }
-    split_shape_v(p->split, o, frags, nfrag);
   }
   // waves: batch order, a new wave when the workspace budget would be exceeded
   size_t cur = 0, worst = 0;

@@ -875,9 +875,9 @@ void split_set_shapes(SplitPlan& sp, int iv, int it, int ig) {
   sp.shape_t = pick(sp.cand_t, it);
   // Gamma with P's slice count runs in P's launch: it must take that launch's shape
   sp.shape_g = sp.slices_g == sp.slices_t ? sp.shape_t : pick(sp.cand_g, ig);
-  sp.cfg_v = sp.cand_v[sp.shape_v];
   sp.cfg_t = sp.cand_t[sp.shape_t];
   sp.cfg_g = sp.cand_g[sp.shape_g];
+  sp.v_by_wave = false;
 }
 
 int split_plan_init(SplitPlan& sp, int precision, const rimp2_options& opt) {
@@ -898,26 +898,29 @@ int split_plan_init(SplitPlan& sp, int precision, const rimp2_options& opt) {
   sp.cand_t = shape_candidates(sp.slices_t, sp.fp8, opt.n_tile, opt.stage_k, opt.n_tile);
   sp.cand_g = shape_candidates(sp.slices_g, sp.fp8, ng, opt.stage_k, opt.n_tile);
   split_set_shapes(sp, 0, 0, 0);
+  sp.v_by_wave = opt.n_tile == 0;
   sp.grid = split_gemm_grid();
   if (split_gemm_prepare() != cudaSuccess) { cudaGetLastError(); return RIMP2_ERR_CUDA; }
   sp.ready = true;
   return RIMP2_OK;
 }
 
-// V's tile width before any tuning.  Its operands come from L2, (128 + n_tile) rows for
-// 128 x n_tile results, and bound a launch of many tiles; wider tiles need less of them, but
-// leave SMs idle where the tiles are few and, with 5 slices, spend longer in the epilogue of a
-// short K (48 columns leave TMEM for a second accumulator set, which hides it).  Measured, BF16
-// with 5 slices at 48 / 64 / 80 columns: nocc=10 nvir=40 naux=150 31 / 33 / 43 us, nocc=20
-// nvir=80 naux=300 46 / 49 / 57 us, nocc=29 nvir=117 naux=437 111 / 110 / 125 us, 40 MBE3 dimers
-// (naux about 420) 3.58 / 3.21 / 3.22 ms, nocc=42 nvir=168 naux=630 453 / 442 / 428 us, nocc=50
-// nvir=250 naux=750 1.46 / 1.38 / 1.30 ms, nocc=100 nvir=500 naux=1500 38.9 / 37.2 / 34.3 ms
-// (96 columns: 35.6).  8 slices at 48 / 64: nocc=20 55 / 66 us, nocc=29 174 / 162, nocc=42 854 /
-// 768 us; FP8 with 8 slices: nocc=20 47 / 57 us, nocc=29 119 / 121, nocc=42 480 / 442 us.
-void split_shape_v(SplitPlan& sp, const rimp2_options& opt, const rimp2_frag* frags, int nfrag) {
-  if (opt.n_tile != 0) return;
+// V's tile width before any tuning, by the work of one launch (of each wave: 64 monomers, nocc
+// 8..20, in 64 waves 4.04 ms with the whole batch's 64 columns, 3.99 with a wave's 48). Its
+// operands come from L2, (128 + n_tile) rows for 128 x n_tile results, and bound a launch of
+// many tiles; wider tiles need less of them, but leave SMs idle where the tiles are few and,
+// with 5 slices, spend longer in the epilogue of a short K (48 columns leave TMEM for a second
+// accumulator set, which hides it). Measured, BF16 with 5 slices at 48 / 64 / 80 columns:
+// nocc=10 nvir=40 naux=150 31 / 33 / 43 us, nocc=20 nvir=80 naux=300 46 / 49 / 57 us, nocc=29
+// nvir=117 naux=437 111 / 110 / 125 us, 40 MBE3 dimers (naux about 420) 3.58 / 3.21 / 3.22 ms,
+// nocc=42 nvir=168 naux=630 453 / 442 / 428 us, nocc=50 nvir=250 naux=750 1.46 / 1.38 / 1.30
+// ms, nocc=100 nvir=500 naux=1500 38.9 / 37.2 / 34.3 ms (96 columns: 35.6). 8 slices at 48 /
+// 64: nocc=20 55 / 66 us, nocc=29 174 / 162, nocc=42 854 / 768 us; FP8 with 8 slices: nocc=20
+// 47 / 57 us, nocc=29 119 / 121, nocc=42 480 / 442 us.
+int split_shape_v(const SplitPlan& sp, const rimp2_frag* frags, const std::vector<int>& members) {
+  if (!sp.v_by_wave) return sp.shape_v;
   double tiles = 0.0, blocks = 0.0;   // tiles of 128 x 48 with results; times naux
-  for (int f = 0; f < nfrag; ++f) {
+  for (int f : members) {
     const double ov = (double)frags[f].nocc * frags[f].nvir, t = ov * (ov + SG_BM) / (2.0 * SG_BM * 48);
     tiles += t;
     blocks += t * frags[f].naux;
@@ -926,10 +929,8 @@ void split_shape_v(SplitPlan& sp, const rimp2_options& opt, const rimp2_frag* fr
   const int want = tiles < 4.0 * sp.grid ? 48 : two && blocks >= 576.0 * tiles ? 80 : 64;
   for (int nt : {want, 64, 48})
     for (size_t i = 0; i < sp.cand_v.size(); ++i)
-      if (sp.cand_v[i].n_tile_max == nt && sp.cand_v[i].bk == sp.cand_v[0].bk) {
-        split_set_shapes(sp, (int)i, 0, 0);
-        return;
-      }
+      if (sp.cand_v[i].n_tile_max == nt && sp.cand_v[i].bk == sp.cand_v[0].bk) return (int)i;
+  return sp.shape_v;
 }
 
 void split_plan_release(SplitPlan&) {}
@@ -1070,8 +1071,9 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
   const int sv = sp.slices_v, st = sp.slices_t, sgl = sp.slices_g;
   // Gamma with P's slice count joins P's launch and so takes its tile shape
   const SplitLaunch& cg = sgl == st ? sp.cfg_t : sp.cfg_g;
-  const int NTv = sp.cfg_v.n_tile_max, NTt = sp.cfg_t.n_tile_max, NTg = cg.n_tile_max;
-  const int BKv = sp.cfg_v.bk, BKt = sp.cfg_t.bk, BKg = cg.bk;
+  w.cfg_v = sp.cand_v[split_shape_v(sp, frags, members)];
+  const int NTv = w.cfg_v.n_tile_max, NTt = sp.cfg_t.n_tile_max, NTg = cg.n_tile_max;
+  const int BKv = w.cfg_v.bk, BKt = sp.cfg_t.bk, BKg = cg.bk;
   const int BKs = sp.fp8 ? 64 : 32;   // K per stage of the slice-stacked kernel
   // split-K target of P_ab / P_ij in multiples of the grid: finer pieces keep the tiles of
   // one occupied-index range closer together in time (their operand rows stay in L2);
@@ -1362,7 +1364,7 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
       if (P.n_tile != c.n_tile_max) return false;
     return true;
   };
-  if (!same_shape(w.probs_v, sp.cfg_v) || !same_shape(w.probs_c, sp.cfg_t) ||
+  if (!same_shape(w.probs_v, w.cfg_v) || !same_shape(w.probs_c, sp.cfg_t) ||
       !same_shape(w.probs_g, sp.cfg_g))
     return RIMP2_ERR_UNSUPPORTED;
   w.mma_v = w.mma_c = w.mma_g = 0.0;
@@ -1432,7 +1434,7 @@ int split_enqueue_wave(SplitPlan& sp, SplitWave& w, char* dblk, int nf, long lon
   if (e == cudaSuccess && w.tiles_v > 0) {
     e = launch_split_gemm((const SplitProb*)(dblk + w.off_pv), (const long long*)(dblk + w.off_bv),
                           (int)w.probs_v.size(), w.tiles_v, bs,
-                          ctr + 0, sp.cfg_v, sp.grid, s);
+                          ctr + 0, w.cfg_v, sp.grid, s);
     ++nl;
   }
   if (ev) cudaEventRecordWithFlags(ev[2], s, cudaEventRecordExternal);

@@ -45,7 +45,7 @@ struct SplitFragDev {
 struct SplitPlan {
   int precision = 0;
   int slices_v = 0, slices_t = 0, slices_g = 0;
-  SplitLaunch cfg_v{}, cfg_t{}, cfg_g{};   // V; P_ab / P_ij; Gamma
+  SplitLaunch cfg_t{}, cfg_g{};   // P_ab / P_ij; Gamma (V: SplitWave::cfg_v)
   int grid = 0;
   bool ready = false;
   bool fp8 = false;  // RIMP2_FP8_SPLIT: e4m3 digits
@@ -54,13 +54,14 @@ struct SplitPlan {
   // launch's shape in use (tuning records keep indices: the order of the lists stays)
   std::vector<SplitLaunch> cand_v, cand_t, cand_g;
   int shape_v = 0, shape_t = 0, shape_g = 0;
+  bool v_by_wave = false;   // V's shape follows each wave's work (neither pinned nor tuned)
 };
 
 // Selects the tile shapes of the V, P_ab / P_ij and Gamma launches (indices into the
-// candidate lists, clamped to their ends).
+// candidate lists, clamped to their ends), V's for every wave.
 void split_set_shapes(SplitPlan& sp, int iv, int it, int ig);
-// The V launch's shape for a plan of these fragments
-void split_shape_v(SplitPlan& sp, const rimp2_options& opt, const rimp2_frag* frags, int nfrag);
+// The V launch's shape (index into cand_v) for a wave of these fragments
+int split_shape_v(const SplitPlan& sp, const rimp2_frag* frags, const std::vector<int>& members);
 
 // Variants of the Gamma/P contraction stage the autotuner times:
 //   0: P_ij rows read through the local (k,b)-major view, split-K target 8 x grid
@@ -72,6 +73,7 @@ constexpr int kSplitVariants = 4;
 
 struct SplitWave {
   std::vector<SplitFragDev> sfd;
+  SplitLaunch cfg_v{};       // V
   std::vector<SplitProb> probs_v, probs_c, probs_g;   // V; P_ab / P_ij; Gamma
   bool sep_energy = false;   // energies by k_split_energy instead of the last amplitude CTAs
   std::vector<SplitProb> probs_s;   // P_ab / P_ij of small extents (slice-stacked kernel)
