@@ -1313,11 +1313,13 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
       w.stack_rows = std::max(w.stack_rows, P.n_tile);
     }
   }
-  // A Gamma launch of few tiles is cut along K as well (at least four stages a slab)
+  // A Gamma launch of few tiles is cut along K as well, in two (at least four stages a slab):
+  // 0 + x + y is the same in either order, so Gamma's bits do not depend on which slab ends
+  // first, which three slabs would not give
   {
     long long tiles = 0;
     for (const auto& P : w.probs_g) tiles += P.ntiles;
-    const int want = tiles > 0 && sp.variant != 3 ? (int)std::min<long long>(8, sp.grid / tiles) : 1;
+    const int want = tiles > 0 && sp.variant != 3 ? (int)std::min<long long>(2, sp.grid / tiles) : 1;
     for (auto& P : w.probs_g) {
       const int slabs = std::min(want, P.k0_blocks / 4);
       if (P.k1_count != 1 || slabs < 2) continue;
