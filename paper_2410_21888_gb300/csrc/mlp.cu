@@ -7,16 +7,20 @@
 // of a sample and reading weights and activations as 16-byte rows; the latency of a tile's
 // layer chain bounds a minibatch.  (One warp per sample with the weights as W[unit][k] rows,
 // 32-way bank conflicts and five shuffles per weight row, took 1362 us for the gradient of a
-// 512-sample minibatch, the tiles 15 us; a whole training step fell from 1370 to 21 us.)
+// 512-sample minibatch, the tiles 15 us; a whole training step fell from 1370 to 20.6 us.)
 // Prediction and features: see k_mlp_predict and log10_pos.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
+#include "rimp2_internal.cuh"
 #include "rimp2_mlp.h"
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int IN = RIMP2_MLP_IN, H = RIMP2_MLP_HIDDEN, P = RIMP2_MLP_PARAMS;
 constexpr int OW1 = 0, OB1 = OW1 + H * IN, OW2 = OB1 + H, OB2 = OW2 + H * H, OW3 = OB2 + H,
@@ -73,10 +77,12 @@ __device__ __forceinline__ void load_weights(Weights& W, const float* __restrict
   }
 }
 
-// acc[q][c] += sum_k in[s_q][k] w[k][4 tx + c] in the order of k, samples s_q = ty SPT + q
+// acc[q][c] += sum_k in[s_q][k] w[k][4 tx + c], samples s_q = ty SPT + q: four chains (k mod 4)
+// added at the end, which round less than one and wait less for one another
 template <int SPT>
 __device__ __forceinline__ void product(const float* __restrict__ in, const float* __restrict__ w,
                                         int tx, int ty, float (&acc)[SPT][4]) {
+  float a[4][SPT][4] = {};
 #pragma unroll 4
   for (int k = 0; k < H; k += 4) {
     float4 h[SPT];
@@ -88,13 +94,17 @@ __device__ __forceinline__ void product(const float* __restrict__ in, const floa
 #pragma unroll
       for (int q = 0; q < SPT; ++q) {
         const float x = kk == 0 ? h[q].x : kk == 1 ? h[q].y : kk == 2 ? h[q].z : h[q].w;
-        acc[q][0] = fmaf(wv.x, x, acc[q][0]);
-        acc[q][1] = fmaf(wv.y, x, acc[q][1]);
-        acc[q][2] = fmaf(wv.z, x, acc[q][2]);
-        acc[q][3] = fmaf(wv.w, x, acc[q][3]);
+        a[kk][q][0] = fmaf(wv.x, x, a[kk][q][0]);
+        a[kk][q][1] = fmaf(wv.y, x, a[kk][q][1]);
+        a[kk][q][2] = fmaf(wv.z, x, a[kk][q][2]);
+        a[kk][q][3] = fmaf(wv.w, x, a[kk][q][3]);
       }
     }
   }
+#pragma unroll
+  for (int q = 0; q < SPT; ++q)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[q][c] += (a[0][q][c] + a[1][q][c]) + (a[2][q][c] + a[3][q][c]);
 }
 
 template <int SPT>
@@ -187,12 +197,17 @@ __device__ __forceinline__ void output_layer(const Weights& W, const float* h3, 
   }
 }
 
+// k_mlp_grad starts beside it and waits for it before its first addition
 __global__ void k_zero_grad(float* g, float* loss) {
+  rimp2::pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < P) g[i] = 0.f;
   if (i == 0 && loss) *loss = 0.f;
 }
 
+// CTAs of a cluster of the gradient kernel, and how many of them run with an SM each: clusters
+// lie within one GPC, and those past 36 share SMs (20,000 samples: 152 CTAs 134 us, 144 91)
+constexpr int kCluster = 4, kGradCtas = 144;
 constexpr int GS = 16;   // samples per tile of the gradient kernel: a 512-sample minibatch
                          // then spreads over 32 CTAs
 
@@ -221,25 +236,47 @@ __device__ __forceinline__ void outer(const float* dz, const float* h, int ns, i
   }
 }
 
-__device__ __forceinline__ void add_rows(float* g, const float (&acc)[4][4], int tx, int ty, bool al) {
+// Sums of the CTAs of a cluster: each adds its share of the parameters over the cluster, in a
+// fixed order, and adds the result to grad and loss.  img: this CTA's gradient [P], then its loss.
+__device__ __forceinline__ void add_cluster(float* img, float* grad, float* loss) {
+  const cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  rimp2::pdl_wait();   // k_zero_grad
+  const bool al = ((uintptr_t)grad & 15) == 0;
+  for (int e = 4 * ((int)cl.block_rank() * NT + (int)threadIdx.x); e < P + 1; e += 4 * kCluster * NT) {
+    float4 v[kCluster];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    float* p = g + (4 * ty + r) * H + 4 * tx;
-    if (al) {
-      asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p),
-                   "f"(acc[r][0]), "f"(acc[r][1]), "f"(acc[r][2]), "f"(acc[r][3])
+    for (int c = 0; c < kCluster; ++c) v[c] = *(const float4*)(cl.map_shared_rank(img, c) + e);
+#pragma unroll
+    for (int w = kCluster / 2; w > 0; w >>= 1)
+#pragma unroll
+      for (int c = 0; c < w; ++c) {
+        v[c].x += v[c + w].x; v[c].y += v[c + w].y;
+        v[c].z += v[c + w].z; v[c].w += v[c + w].w;
+      }
+    if (al && e + 4 <= P) {
+      asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(grad + e),
+                   "f"(v[0].x), "f"(v[0].y), "f"(v[0].z), "f"(v[0].w)
                    : "memory");
     } else {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) atomicAdd(p + c, acc[r][c]);
+      const float x[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
+      for (int k = 0; k < 4; ++k)
+        if (e + k < P) atomicAdd(grad + e + k, x[k]);
+        else if (e + k == P && loss) atomicAdd(loss, x[k]);
     }
   }
+  cl.sync();   // the others have read img
 }
 
 // Gradient of the minibatch loss.  A CTA takes tiles blockIdx.x, blockIdx.x + gridDim.x, ...
 // of GS samples and keeps its sums over them in registers (the 64 x 64 weight gradients as
-// 4 x 4 blocks a thread); one global addition per parameter and CTA at the end.
-__global__ void __launch_bounds__(NT)
+// 4 x 4 blocks a thread), then the CTAs of a cluster add theirs up through distributed shared
+// memory, and each parameter takes one global addition per cluster: those arrive in any order,
+// and a long chain of them bounds the gradient's accuracy.  Error in norm against 64 bits,
+// additions per CTA -> per cluster (and product's four chains): 32 samples 1.1e-7 -> 0.9e-7,
+// 512 0.89e-7 -> 0.54e-7, 2048 1.7e-7 -> 0.86e-7, 20,000 1.8e-7 -> 0.87e-7.  It starts beside
+// k_zero_grad, which pays for the cluster's barriers (a training step 21.0 -> 20.6 us).
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(NT)
 k_mlp_grad(const float* __restrict__ master, const float* __restrict__ feats,
            const float* __restrict__ y, const int* __restrict__ idx, int n,
            const float* __restrict__ mean, const float* __restrict__ stdv, float* grad,
@@ -247,11 +284,13 @@ k_mlp_grad(const float* __restrict__ master, const float* __restrict__ feats,
   extern __shared__ __align__(16) unsigned char smem_mlp[];
   GradSmem& S = *(GradSmem*)smem_mlp;
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const bool al_m = ((uintptr_t)master & 15) == 0, al_g = ((uintptr_t)grad & 15) == 0;
+  const bool al_m = ((uintptr_t)master & 15) == 0;
   load_weights(S.W, master, al_m);
-  for (int e = t; e < H * H; e += NT) {
-    S.w2n[e] = bf16_round(master[OW2 + e]);
-    S.w3n[e] = bf16_round(master[OW3 + e]);
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int e = 4 * (t + NT * r);
+    *(float4*)(S.w2n + e) = load_w4(master + OW2, e / H, e % H, al_m);
+    *(float4*)(S.w3n + e) = load_w4(master + OW3, e / H, e % H, al_m);
   }
   float g2[4][4] = {}, g3[4][4] = {};
   float g1[3] = {0.f, 0.f, 0.f};   // dW1 elements t, t + 256, t + 512
@@ -315,17 +354,26 @@ k_mlp_grad(const float* __restrict__ master, const float* __restrict__ feats,
     if (t == 0)
       for (int s = 0; s < ns; ++s) { gb4 += S.dy[s]; lsum += S.rs[s]; }
   }
-  add_rows(grad + OW3, g3, tx, ty, al_g);
-  add_rows(grad + OW2, g2, tx, ty, al_g);
+  // the weights' place takes the CTA's sums
+  static_assert(sizeof(Weights) >= (P + 1 + 3) / 4 * 16, "gradient and loss in 16-byte units");
+  __syncthreads();
+  float* img = (float*)&S.W;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int e = (4 * ty + r) * H + 4 * tx;
+    *(float4*)(img + OW2 + e) = make_float4(g2[r][0], g2[r][1], g2[r][2], g2[r][3]);
+    *(float4*)(img + OW3 + e) = make_float4(g3[r][0], g3[r][1], g3[r][2], g3[r][3]);
+  }
 #pragma unroll
   for (int r = 0; r < 3; ++r)
-    if (t + NT * r < IN * H) atomicAdd(grad + OW1 + t + NT * r, g1[r]);
-  if (t < 192) atomicAdd(grad + (t < 64 ? OB1 : t < 128 ? OB2 : OB3) + (t & 63), gb);
-  else atomicAdd(grad + OW4 + (t & 63), gw4);
+    if (t + NT * r < IN * H) img[OW1 + t + NT * r] = g1[r];
+  if (t < 192) img[(t < 64 ? OB1 : t < 128 ? OB2 : OB3) + (t & 63)] = gb;
+  else img[OW4 + (t & 63)] = gw4;
   if (t == 0) {
-    atomicAdd(grad + OB4, gb4);
-    if (loss) atomicAdd(loss, lsum / (float)n);
+    img[OB4] = gb4;
+    img[P] = lsum / (float)n;
   }
+  add_cluster(img, grad, loss);
 }
 
 __global__ void k_mlp_adam(float* w, const float* g, float* m, float* v, float c1, float c2,
@@ -663,11 +711,11 @@ extern "C" int rimp2_mlp_grad(const float* master, const float* feats, const flo
       cudaSuccess)
     return check(cudaGetLastError());
   k_zero_grad<<<(P + 255) / 256, 256, 0, s>>>(grad, loss);
-  // one CTA per tile up to one per SM of a GB300; more tiles are looped over
+  // one CTA per tile, rounded up to whole clusters; more tiles are looped over
   const int tiles = n / GS + (n % GS != 0);
-  k_mlp_grad<<<tiles < kSMs ? tiles : kSMs, NT, smem, s>>>(master, feats, y, idx, n, mean, stdv, grad,
-                                                           loss);
-  return check(cudaGetLastError());
+  const int ctas = tiles < kGradCtas ? (tiles + kCluster - 1) / kCluster * kCluster : kGradCtas;
+  return check(rimp2::launch_pdl(k_mlp_grad, (unsigned)ctas, NT, smem, s, true, master, feats, y, idx, n, mean,
+                                 stdv, grad, loss));
 }
 
 extern "C" int rimp2_mlp_adam(float* master, const float* grad, float* m, float* v, int32_t t,
