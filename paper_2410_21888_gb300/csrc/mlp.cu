@@ -600,27 +600,40 @@ __device__ __forceinline__ void sort3(float& a, float& b, float& c) {
   if (a > b) { t = a; a = b; b = t; }
 }
 
-// log10 of x >= 1e-16 (or inf, NaN) in FP64, for a result that is rounded to FP32.  x = 2^e m;
-// with c = 1/m at the middle of m's 1/128 of [1, 2), log10(x) = e log10(2) - log10(c) +
-// log10(1 + r), r = m c - 1 (|r| < 2^-7), by the Taylor series of log(1 + r) to r^7: twelve
-// FP64 instructions, a relative error of at most 2^-45.  At both ends of the octave c is 1 or 1/2,
-// so the logarithm of an x next to 1 has no cancellation.
-constexpr double kLog10Of2 = 0.30102999566398119521, kLog10OfE = 0.43429448190325182765;
+// log10 of x >= 1e-16 (or inf, NaN) in FP64: x = 2^e m with m in [0.71, 1.42); with c near 1/m
+// from a table of 1/128 steps, log10(x) = e log10(2) - log10(c) + log10(1 + r), r = m c - 1
+// (|r| < 2^-7), by the Taylor series of log(1 + r) to r^8.  Around x = 1 both e and log10(c)
+// vanish, so nothing cancels: at most 1.6 units in the last place of the FP64 result anywhere
+// (emulated with exact rationals; the CUDA library states 2), in 13 FP64 instructions.
+constexpr double kLog10Of2 = 0.30102999566398119521;
+constexpr double kLog10OfE = 0.43429448190325182765, kLog10OfELow = 1.0983196502167650e-17;
+constexpr int kLogUpper = 53;   // first step of m in [1, 2) that is taken as 2^(e + 1) m / 2
 
-constexpr double minus_log10(double c) {   // -log10(c), 1/2 <= c <= 1: -2 atanh((c - 1) / (c + 1)) / log(10)
-  const double z = (c - 1.0) / (c + 1.0), z2 = z * z;
-  double s = 0.0;
-  for (int k = 45; k > 0; k -= 2) s = s * z2 + 1.0 / k;
-  return -2.0 * z * s * kLog10OfE;
+// a b = p + the returned remainder, exactly (Dekker)
+constexpr double product_rest(double a, double b, double p) {
+  const double ta = 134217729.0 * a, ah = ta - (ta - a), al = a - ah;
+  const double tb = 134217729.0 * b, bh = tb - (tb - b), bl = b - bh;
+  return ((ah * bh - p) + ah * bl + al * bh) + al * bl;
 }
 
-struct LogTable { double2 e[128]; };   // (c, -log10(c))
+// -log10(c), 0.7 < c < 1.42, to an ulp: -2 atanh(z) / log(10), z = (c - 1) / (c + 1), with the
+// rounding errors of z and of the last product carried along
+constexpr double minus_log10(double c) {
+  const double n = c - 1.0, d = c + 1.0, dl = c < 1.0 ? 1.0 - (d - c) : c - (d - 1.0);
+  const double z = n / d, zd = z * d, zl = ((n - zd) - product_rest(z, d, zd) - z * dl) / d, z2 = z * z;
+  double q = 0.0;
+  for (int k = 45; k > 1; k -= 2) q = q * z2 + 1.0 / k;
+  const double t = zl + z * (z2 * q), p = z * kLog10OfE;
+  return -2.0 * (p + (product_rest(z, kLog10OfE, p) + kLog10OfE * t + kLog10OfELow * z));
+}
+
+struct LogTable { double2 e[128]; };   // (c, -log10(c), or -log10(2 c) from kLogUpper on)
 constexpr LogTable log_table() {
   LogTable t{};
   for (int i = 0; i < 128; ++i) {
     const double c = i == 0 ? 1.0 : i == 127 ? 0.5 : 1.0 / (1.0 + (i + 0.5) / 128.0);
     t.e[i].x = c;
-    t.e[i].y = i == 0 ? 0.0 : i == 127 ? kLog10Of2 : minus_log10(c);
+    t.e[i].y = i == 0 || i == 127 ? 0.0 : minus_log10(i < kLogUpper ? c : 2.0 * c);
   }
   return t;
 }
@@ -628,36 +641,24 @@ __device__ const LogTable g_log_table = log_table();
 
 __device__ __forceinline__ float log10_pos(double x) {
   const long long u = __double_as_longlong(x);
-  const int ef = (int)(u >> 52) & 0x7ff;
+  const int ef = (int)(u >> 52) & 0x7ff, i = (int)(u >> 45) & 127;
   if (ef == 0x7ff) return (float)fabs(x);
   const double m = __longlong_as_double((u & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
-  const double2 t = g_log_table.e[(int)(u >> 45) & 127];
+  const double2 t = g_log_table.e[i];
   const double r = fma(m, t.x, -1.0);
-  double p = kLog10OfE / 7.0;
+  double p = -kLog10OfE / 8.0;
+  p = fma(p, r, kLog10OfE / 7.0);
   p = fma(p, r, -kLog10OfE / 6.0);
   p = fma(p, r, kLog10OfE / 5.0);
   p = fma(p, r, -kLog10OfE / 4.0);
   p = fma(p, r, kLog10OfE / 3.0);
   p = fma(p, r, -kLog10OfE / 2.0);
   p = fma(p, r, kLog10OfE);
-  return (float)fma(p, r, fma((double)(ef - 1023), kLog10Of2, t.y));
+  return (float)fma(p, r, fma((double)(ef - 1023 + (i >= kLogUpper)), kLog10Of2, t.y));
 }
 
-__device__ __noinline__ float sqrt_any(double s) { return (float)sqrt(s); }
-
-// sqrt(s) rounded to FP32: the FP32 root and one correction from the FP64 residual (its error
-// is 2^-46 of the root); outside FP32's comfortable range the FP64 root
-__device__ __forceinline__ float sqrt_f32(double s) {
-  const float f = (float)s;
-  if (!(f > 1e-30f && f < 1e30f)) return sqrt_any(s);
-  const float y = sqrtf(f);
-  const double yd = y;
-  return y + (float)fma(-yd, yd, s) * (0.5f / y);
-}
-
-// FP64 instructions bound it (a warp's takes the SM's pipe for 16 clocks): about 70 a trimer
-// instead of 250 with FP64 square roots and library logarithms, 22,018 trimers 8.6 us
-// instead of 11.8 from cold caches.
+// FP64 instructions bound it (a warp's takes the SM's pipe for 16 clocks): log10_pos needs a
+// quarter of the library logarithm's, 22,018 trimers take 9.9 us instead of 13.9 (calls in a row).
 __global__ void k_screen_features(const double* __restrict__ cen, const int* __restrict__ nocc,
                                   int n, const int* __restrict__ tri, long long nt,
                                   const double* __restrict__ dde, float* __restrict__ f) {
@@ -667,7 +668,7 @@ __global__ void k_screen_features(const double* __restrict__ cen, const int* __r
   auto d = [&](int a, int b) {
     const double dx = cen[3 * a] - cen[3 * b], dy = cen[3 * a + 1] - cen[3 * b + 1],
                  dz = cen[3 * a + 2] - cen[3 * b + 2];
-    return sqrt_f32(dx * dx + dy * dy + dz * dz);
+    return (float)sqrt(dx * dx + dy * dy + dz * dz);
   };
   auto lg = [&](int a, int b) { return log10_pos(fabs(dde[(long long)a * n + b]) + 1e-16); };
   float e0 = lg(I, J), e1 = lg(I, K), e2 = lg(J, K);
