@@ -43,7 +43,8 @@ typedef struct rimp2_zvec_args {
   double* lpp;               /* device out [nvir][n]: L''_aq */
   double* dai;               /* device out [nocc][nvir]: D_ai stored at [i][a] */
   double* info;              /* device out [3]: iterations taken, ||r|| / ||rhs||, ||rhs||
-                                (iterations = max_iter + 1 when the tolerance was not met) */
+                                (iterations = max_iter + 1 when the tolerance was not met,
+                                -1 when a bounded device wait expired: D_ai is unfinished) */
 } rimp2_zvec_args;
 
 /* Workspace bytes for one fragment of these sizes (device memory the caller owns; 256-byte
@@ -55,7 +56,7 @@ int rimp2_zvec_workspace_size(int32_t nocc, int32_t nvir, int32_t naux, int32_t 
  * staged from host memory into the workspace during the call, which therefore waits for
  * the work already queued on the stream and is not stream-capturable; the step itself
  * runs asynchronously (the conjugate-gradient iterations are one cooperative launch, whose
- * grid barriers have bounded waits: on expiry it ends as not converged).  Errors:
+ * grid barriers have bounded waits: on expiry it ends with info[0] = -1).  Errors:
  * RIMP2_ERR_BAD_ARG for negative sizes or a NULL required pointer, RIMP2_ERR_WORKSPACE when
  * the workspace is NULL, not 256-byte aligned or below rimp2_zvec_workspace_size,
  * RIMP2_ERR_UNSUPPORTED when the descriptor lists outgrow their 1.25 MB region (nocc above

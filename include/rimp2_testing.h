@@ -43,6 +43,12 @@ int rimp2_testing_slice_gemm_k(int32_t M, int32_t N, int32_t K, int32_t kpad, in
  * device until it is set again. */
 int rimp2_testing_set_wait_limit(int64_t ns);
 
+/* The same for the grid barriers of the conjugate-gradient kernel (rimp2_zvec_solve), in the
+ * calls that follow in this process; ns < 0 restores the normal limit.  With 0 a barrier's
+ * wait gives up unless its first probe finds every CTA there: all CTAs leave the kernel and
+ * info[0] is -1. */
+int rimp2_testing_set_zvec_wait_limit(int64_t ns);
+
 /* FP64 throughput of the current device in TFLOP/s, measured in place (the denominators
  * of the plain FP64 path's roofline): kind 0 = CUDA-core DFMA (8 independent FMA chains
  * per thread), kind 1 = FP64 tensor path (mma.sync m8n8k4, 8 independent accumulators

@@ -16,6 +16,7 @@
 // on caller pointers); the sums over one index run as column or row sums; the whole
 // conjugate-gradient solve is one cooperative kernel (k_cg).
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <vector>
 
@@ -23,6 +24,7 @@
 
 #include "fp64_gemm.cuh"
 #include "rimp2_grad.h"
+#include "rimp2_testing.h"
 
 namespace rimp2 {
 namespace {
@@ -140,7 +142,11 @@ __device__ __forceinline__ bool grid_barrier(const CgArgs& A, unsigned long long
     atomicAdd(A.bar, 1ull);
     unsigned long long t0, t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-    for (unsigned it = 1;; ++it) {
+    if (A.limit_ns == 0 && *(volatile unsigned long long*)A.bar < arrivals) {   // the test hook's
+      atomicExch(A.abort, 1u);
+      good = 0;
+    }
+    for (unsigned it = 1; good; ++it) {
       if (*(volatile unsigned long long*)A.bar >= arrivals) break;
       if ((it & 255u) == 0) {
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -322,8 +328,8 @@ __global__ void __launch_bounds__(256, F64_CTAS) k_cg(CgArgs A) {
     if (!grid_barrier(A, arrivals)) break;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    // iterations = max_iter + 1 when the tolerance was not met
-    A.info[0] = s_conv ? (double)it : (double)(A.max_iter + 1);
+    // iterations = max_iter + 1 when the tolerance was not met, -1 when a barrier's wait expired
+    A.info[0] = s_conv ? (double)it : *(volatile unsigned*)A.abort ? -1.0 : (double)(A.max_iter + 1);
     A.info[1] = s_bnorm > 0.0 ? s_rnorm / s_bnorm : 0.0;
     A.info[2] = s_bnorm;
   }
@@ -376,6 +382,8 @@ Layout layout(long long o, long long v, long long X, int max_iter) {
   return L;
 }
 
+std::atomic<long long> g_wait_ns{-1};   // test hook: limit of k_cg's barriers (< 0: the normal one)
+
 int iters_of(const rimp2_zvec_args* a) { return a->max_iter > 0 ? a->max_iter : 100; }
 
 }  // namespace
@@ -384,6 +392,11 @@ int iters_of(const rimp2_zvec_args* a) { return a->max_iter > 0 ? a->max_iter : 
 using namespace rimp2;
 
 extern "C" {
+
+int rimp2_testing_set_zvec_wait_limit(int64_t ns) {
+  g_wait_ns.store(ns < 0 ? -1 : (long long)ns, std::memory_order_relaxed);
+  return RIMP2_OK;
+}
 
 int rimp2_zvec_workspace_size(int32_t nocc, int32_t nvir, int32_t naux, int32_t max_iter,
                               size_t* bytes) {
@@ -514,7 +527,9 @@ int rimp2_zvec_solve(const rimp2_zvec_args* A, void* workspace, size_t ws_bytes,
   C.bar = (unsigned long long*)(ws + L.bar);
   C.abort = (unsigned*)(ws + L.bar + 128);
   // a healthy barrier waits for a fraction of one exchange product's time
-  C.limit_ns = 2000000000ull + (unsigned long long)(2.0 * o * o * v * X * 4e-3);
+  const long long limit = g_wait_ns.load(std::memory_order_relaxed);
+  C.limit_ns = limit >= 0 ? (unsigned long long)limit
+                          : 2000000000ull + (unsigned long long)(2.0 * o * o * v * X * 4e-3);
   // every CTA resident (cooperative), and no more of them than the phases have items: a grid
   // barrier costs less with fewer
   int dev = 0, sms = 0, per = 0;
