@@ -54,8 +54,8 @@ k_assemble_rows(const OutBlock* __restrict__ blocks, const Contrib* __restrict__
   const int2 it = items[blockIdx.x];
   const OutBlock b = blocks[it.x];
   const int lane = threadIdx.x & 31;
-  const long long rows = min((long long)b.n0 * b.n1, (long long)it.y + rows_per);
-  for (long long r = it.y + (threadIdx.x >> 5); r < rows; r += 8) {
+  const long long first = (long long)it.y * rows_per, rows = min((long long)b.n0 * b.n1, first + rows_per);
+  for (long long r = first + (threadIdx.x >> 5); r < rows; r += 8) {
     const int i = (int)(r / b.n1), a = (int)(r - (long long)i * b.n1);
     double* const row = out + b.out_off + (long long)i * b.ld0 + (long long)a * b.ld1;
     for (int q0 = lane; q0 < b.n2; q0 += 32 * kRun) {
@@ -99,7 +99,7 @@ k_assemble_rows(const OutBlock* __restrict__ blocks, const Contrib* __restrict__
 struct Table {
   std::vector<OutBlock> blocks;
   std::vector<Contrib> con;
-  std::vector<int2> items;   // (block, first row)
+  std::vector<int2> items;   // (block, group of rows_per rows: a block may hold 2^31 rows and more)
   int rows_per = 1;
   // device copies (inside the handle's buffer)
   const OutBlock* d_blocks = nullptr;
@@ -132,7 +132,7 @@ void finish_items(Table& t, int rows_per) {
   std::vector<int2> sorted;
   for (int b : order) {
     const long long rows = (long long)t.blocks[b].n0 * t.blocks[b].n1;
-    for (long long r = 0; r < rows; r += rows_per) sorted.push_back(make_int2(b, (int)r));
+    for (long long r = 0; r < rows; r += rows_per) sorted.push_back(make_int2(b, (int)(r / rows_per)));
   }
   // dealt in groups of about one wave of CTAs that all hold the same mix: rows with many
   // contributions are bound by FP64 additions, those with one by HBM
