@@ -144,8 +144,11 @@ def _require_cuda():
 def _stream_handle(stream) -> int:
     if stream is None:
         # the current stream's handle without a Stream object around it (0.3 us instead of 3,
-        # of the 25 that the host spends on a training step of 21 us)
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        # of the 25 that the host spends on a training step of 21 us), where torch has the call
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None:
+            return raw(torch.cuda.current_device())
+        stream = torch.cuda.current_stream()
     return int(stream.cuda_stream)
 
 
