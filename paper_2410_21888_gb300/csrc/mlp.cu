@@ -29,9 +29,9 @@ static_assert(OB4 + 1 == P, "parameter layout");
 static_assert(H == 64 && OW2 % 4 == 0 && OW3 % 4 == 0, "16-byte weight rows");
 
 constexpr int kSMs = 152;       // streaming multiprocessors of a GB300
-constexpr int NT = 256;         // threads: 16 unit groups (of 4) x 16 sample groups
-constexpr int LDH = H + 4;      // activation row stride: rows of a warp's two sample groups
-                                // start 4 banks apart
+constexpr int NT = 256;         // threads of the gradient kernel: 16 unit groups (of 4) x 16 samples
+constexpr int LDH = H + 4;      // activation row stride: the rows of a warp's two samples start
+                                // 4 banks apart
 constexpr int LDX = 12;         // standardised input row stride
 
 __device__ __forceinline__ float bf16_round(float x) {
@@ -77,124 +77,44 @@ __device__ __forceinline__ void load_weights(Weights& W, const float* __restrict
   }
 }
 
-// acc[q][c] += sum_k in[s_q][k] w[k][4 tx + c], samples s_q = ty SPT + q: four chains (k mod 4)
-// added at the end, which round less than one and wait less for one another
-template <int SPT>
+// acc[c] += sum_k in[k] w[k][4 tx + c], in: the thread's sample.  Four chains (k mod 4) added at
+// the end, which round less than one and wait less for one another
 __device__ __forceinline__ void product(const float* __restrict__ in, const float* __restrict__ w,
-                                        int tx, int ty, float (&acc)[SPT][4]) {
-  float a[4][SPT][4] = {};
+                                        int tx, float (&acc)[4]) {
+  float a[4][4] = {};
 #pragma unroll 4
   for (int k = 0; k < H; k += 4) {
-    float4 h[SPT];
-#pragma unroll
-    for (int q = 0; q < SPT; ++q) h[q] = *(const float4*)(in + (ty * SPT + q) * LDH + k);
+    const float4 h = *(const float4*)(in + k);
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
       const float4 wv = *(const float4*)(w + (k + kk) * H + 4 * tx);
-#pragma unroll
-      for (int q = 0; q < SPT; ++q) {
-        const float x = kk == 0 ? h[q].x : kk == 1 ? h[q].y : kk == 2 ? h[q].z : h[q].w;
-        a[kk][q][0] = fmaf(wv.x, x, a[kk][q][0]);
-        a[kk][q][1] = fmaf(wv.y, x, a[kk][q][1]);
-        a[kk][q][2] = fmaf(wv.z, x, a[kk][q][2]);
-        a[kk][q][3] = fmaf(wv.w, x, a[kk][q][3]);
-      }
+      const float x = kk == 0 ? h.x : kk == 1 ? h.y : kk == 2 ? h.z : h.w;
+      a[kk][0] = fmaf(wv.x, x, a[kk][0]);
+      a[kk][1] = fmaf(wv.y, x, a[kk][1]);
+      a[kk][2] = fmaf(wv.z, x, a[kk][2]);
+      a[kk][3] = fmaf(wv.w, x, a[kk][3]);
     }
   }
 #pragma unroll
-  for (int q = 0; q < SPT; ++q)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[q][c] += (a[0][q][c] + a[1][q][c]) + (a[2][q][c] + a[3][q][c]);
+  for (int c = 0; c < 4; ++c) acc[c] += (a[0][c] + a[1][c]) + (a[2][c] + a[3][c]);
 }
 
-template <int SPT>
-__device__ __forceinline__ void set_bias(const float* b, int tx, float (&acc)[SPT][4]) {
+__device__ __forceinline__ void set_bias(const float* b, int tx, float (&z)[4]) {
 #pragma unroll
-  for (int q = 0; q < SPT; ++q)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[q][c] = b[4 * tx + c];
+  for (int c = 0; c < 4; ++c) z[c] = b[4 * tx + c];
 }
 
-// h = SiLU(z) to shared memory and, for the backward pass, SiLU'(z) = s (1 + z (1 - s))
-template <int SPT, bool D>
-__device__ __forceinline__ void activate(const float (&z)[SPT][4], float* h, float* d, int tx,
-                                         int ty) {
+// h = SiLU(z) and d = SiLU'(z) = s (1 + z (1 - s)) to shared memory
+__device__ __forceinline__ void activate(const float (&z)[4], float* h, float* d) {
+  float hv[4], dv[4];
 #pragma unroll
-  for (int q = 0; q < SPT; ++q) {
-    float hv[4], dv[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const float s = sigm(z[q][c]);
-      hv[c] = z[q][c] * s;
-      dv[c] = s * (1.f + z[q][c] * (1.f - s));
-    }
-    *(float4*)(h + (ty * SPT + q) * LDH + 4 * tx) = make_float4(hv[0], hv[1], hv[2], hv[3]);
-    if (D) *(float4*)(d + (ty * SPT + q) * LDH + 4 * tx) = make_float4(dv[0], dv[1], dv[2], dv[3]);
+  for (int c = 0; c < 4; ++c) {
+    const float s = sigm(z[c]);
+    hv[c] = z[c] * s;
+    dv[c] = s * (1.f + z[c] * (1.f - s));
   }
-}
-
-// Standardised inputs of the tile's first ns samples (rows idx[s0 + s] of feats, or s0 + s)
-template <int S>
-__device__ __forceinline__ void load_inputs(const float* __restrict__ feats,
-                                            const int* __restrict__ idx, long long s0, int ns,
-                                            const float* __restrict__ mean,
-                                            const float* __restrict__ stdv, float* xs) {
-  for (int e = threadIdx.x; e < S * IN; e += NT) {
-    const int s = e / IN, i = e - s * IN;
-    float v = 0.f;
-    if (s < ns) {
-      const long long row = idx ? (long long)idx[s0 + s] : s0 + s;
-      v = (feats[row * IN + i] - mean[i]) / stdv[i];
-    }
-    xs[s * LDX + i] = v;
-  }
-}
-
-// Hidden layers 1..3 of the tile (z -> h, and SiLU' for the backward pass); h1 may be
-// overwritten by h3 (prediction)
-template <int SPT, bool D>
-__device__ __forceinline__ void hidden_layers(const Weights& W, const float* xs, float* h1, float* h2,
-                                              float* h3, float* d1, float* d2, float* d3, int tx,
-                                              int ty) {
-  float z[SPT][4];
-  set_bias<SPT>(W.b1, tx, z);
-#pragma unroll
-  for (int i = 0; i < IN; ++i) {
-    const float4 wv = *(const float4*)(W.w1t + i * H + 4 * tx);
-#pragma unroll
-    for (int q = 0; q < SPT; ++q) {
-      const float x = xs[(ty * SPT + q) * LDX + i];
-      z[q][0] = fmaf(wv.x, x, z[q][0]);
-      z[q][1] = fmaf(wv.y, x, z[q][1]);
-      z[q][2] = fmaf(wv.z, x, z[q][2]);
-      z[q][3] = fmaf(wv.w, x, z[q][3]);
-    }
-  }
-  activate<SPT, D>(z, h1, d1, tx, ty);
-  __syncthreads();
-  set_bias<SPT>(W.b2, tx, z);
-  product<SPT>(h1, W.w2t, tx, ty, z);
-  activate<SPT, D>(z, h2, d2, tx, ty);
-  __syncthreads();
-  set_bias<SPT>(W.b3, tx, z);
-  product<SPT>(h2, W.w3t, tx, ty, z);
-  activate<SPT, D>(z, h3, d3, tx, ty);
-  __syncthreads();
-}
-
-// Output layer: the 16 threads of a sample group sum their units of each sample
-template <int SPT>
-__device__ __forceinline__ void output_layer(const Weights& W, const float* h3, int tx, int ty,
-                                             float (&y)[SPT]) {
-#pragma unroll
-  for (int q = 0; q < SPT; ++q) {
-    const float4 h = *(const float4*)(h3 + (ty * SPT + q) * LDH + 4 * tx);
-    float s = W.w4[4 * tx] * h.x + W.w4[4 * tx + 1] * h.y + W.w4[4 * tx + 2] * h.z +
-              W.w4[4 * tx + 3] * h.w;
-#pragma unroll
-    for (int off = 8; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    y[q] = s + W.b4;
-  }
+  *(float4*)h = make_float4(hv[0], hv[1], hv[2], hv[3]);
+  *(float4*)d = make_float4(dv[0], dv[1], dv[2], dv[3]);
 }
 
 // k_mlp_grad starts beside it and waits for it before its first addition
@@ -206,7 +126,8 @@ __global__ void k_zero_grad(float* g, float* loss) {
 }
 
 // CTAs of a cluster of the gradient kernel, and how many of them run with an SM each: clusters
-// lie within one GPC, and those past 36 share SMs (20,000 samples: 152 CTAs 134 us, 144 91)
+// lie within one GPC, and those past 36 share SMs (a step of 20,000 samples: with 152 CTAs 134 us,
+// with 144 90)
 constexpr int kCluster = 4, kGradCtas = 144;
 constexpr int GS = 16;   // samples per tile of the gradient kernel: a 512-sample minibatch
                          // then spreads over 32 CTAs
@@ -268,6 +189,59 @@ __device__ __forceinline__ void add_cluster(float* img, float* grad, float* loss
   cl.sync();   // the others have read img
 }
 
+// Standardised inputs of the tile's first ns samples (rows idx[s0 + s] of feats, or s0 + s)
+__device__ __forceinline__ void load_inputs(const float* __restrict__ feats,
+                                            const int* __restrict__ idx, long long s0, int ns,
+                                            const float* __restrict__ mean,
+                                            const float* __restrict__ stdv, float* xs) {
+  for (int e = threadIdx.x; e < GS * IN; e += NT) {
+    const int s = e / IN, i = e - s * IN;
+    float v = 0.f;
+    if (s < ns) {
+      const long long row = idx ? (long long)idx[s0 + s] : s0 + s;
+      v = (feats[row * IN + i] - mean[i]) / stdv[i];
+    }
+    xs[s * LDX + i] = v;
+  }
+}
+
+// Hidden layers 1..3 of the tile (z -> h, and SiLU' for the backward pass): units 4 tx .. + 3 of
+// sample ty
+__device__ __forceinline__ void hidden_layers(GradSmem& S, int tx, int ty) {
+  const int row = ty * LDH, at = row + 4 * tx;
+  float z[4];
+  set_bias(S.W.b1, tx, z);
+#pragma unroll
+  for (int i = 0; i < IN; ++i) {
+    const float4 wv = *(const float4*)(S.W.w1t + i * H + 4 * tx);
+    const float x = S.xs[ty * LDX + i];
+    z[0] = fmaf(wv.x, x, z[0]);
+    z[1] = fmaf(wv.y, x, z[1]);
+    z[2] = fmaf(wv.z, x, z[2]);
+    z[3] = fmaf(wv.w, x, z[3]);
+  }
+  activate(z, S.h1 + at, S.d1 + at);
+  __syncthreads();
+  set_bias(S.W.b2, tx, z);
+  product(S.h1 + row, S.W.w2t, tx, z);
+  activate(z, S.h2 + at, S.d2 + at);
+  __syncthreads();
+  set_bias(S.W.b3, tx, z);
+  product(S.h2 + row, S.W.w3t, tx, z);
+  activate(z, S.h3 + at, S.d3 + at);
+  __syncthreads();
+}
+
+// Output layer: the 16 threads of a sample sum their units
+__device__ __forceinline__ float output_layer(const GradSmem& S, int tx, int ty) {
+  const float4 h = *(const float4*)(S.h3 + ty * LDH + 4 * tx);
+  const float* w = S.W.w4 + 4 * tx;
+  float s = w[0] * h.x + w[1] * h.y + w[2] * h.z + w[3] * h.w;
+#pragma unroll
+  for (int off = 8; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  return s + S.W.b4;
+}
+
 // Gradient of the minibatch loss.  A CTA takes tiles blockIdx.x, blockIdx.x + gridDim.x, ...
 // of GS samples and keeps its sums over them in registers (the 64 x 64 weight gradients as
 // 4 x 4 blocks a thread), then the CTAs of a cluster add theirs up through distributed shared
@@ -300,15 +274,14 @@ k_mlp_grad(const float* __restrict__ master, const float* __restrict__ feats,
   for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const int s0 = tile * GS, ns = min(GS, n - s0);
     __syncthreads();   // weights loaded; the previous tile is no longer read
-    load_inputs<GS>(feats, idx, s0, ns, mean, stdv, S.xs);
+    load_inputs(feats, idx, s0, ns, mean, stdv, S.xs);
     __syncthreads();
-    hidden_layers<1, true>(S.W, S.xs, S.h1, S.h2, S.h3, S.d1, S.d2, S.d3, tx, ty);
-    float yv[1];
-    output_layer<1>(S.W, S.h3, tx, ty, yv);
+    hidden_layers(S, tx, ty);
+    const float yv = output_layer(S, tx, ty);
     float dy = 0.f;
     if (ty < ns) {
       const int row = idx ? idx[s0 + ty] : s0 + ty;
-      const float r = yv[0] - y[row];
+      const float r = yv - y[row];
       dy = 2.f * r / (float)n;
       if (tx == 0) { S.rs[ty] = r * r; S.dy[ty] = dy; }
     }
@@ -321,20 +294,20 @@ k_mlp_grad(const float* __restrict__ master, const float* __restrict__ feats,
     __syncthreads();
     outer(S.d3, S.h2, ns, tx, ty, g3);
     {
-      float dh[1][4] = {};
-      product<1>(S.d3, S.w3n, tx, ty, dh);
+      float dh[4] = {};
+      product(S.d3 + ty * LDH, S.w3n, tx, dh);
       float4* p = (float4*)(S.d2 + ty * LDH + 4 * tx);
       v = *p;
-      *p = make_float4(dh[0][0] * v.x, dh[0][1] * v.y, dh[0][2] * v.z, dh[0][3] * v.w);
+      *p = make_float4(dh[0] * v.x, dh[1] * v.y, dh[2] * v.z, dh[3] * v.w);
     }
     __syncthreads();
     outer(S.d2, S.h1, ns, tx, ty, g2);
     {
-      float dh[1][4] = {};
-      product<1>(S.d2, S.w2n, tx, ty, dh);
+      float dh[4] = {};
+      product(S.d2 + ty * LDH, S.w2n, tx, dh);
       float4* p = (float4*)(S.d1 + ty * LDH + 4 * tx);
       v = *p;
-      *p = make_float4(dh[0][0] * v.x, dh[0][1] * v.y, dh[0][2] * v.z, dh[0][3] * v.w);
+      *p = make_float4(dh[0] * v.x, dh[1] * v.y, dh[2] * v.z, dh[3] * v.w);
     }
     __syncthreads();
     if (t < 192) {

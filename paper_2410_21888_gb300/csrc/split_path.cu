@@ -1087,7 +1087,6 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
   // amplitude kernel's scales)
   const int head = sp.fp8 ? SG_HEAD_FP8 : SG_HEAD_BF16;
   const int kTtAdd = -123 + head, kTAdd = -124 + head;
-  w.want_gamma = false;
   for (int idx : members) {
     const rimp2_frag& f = frags[idx];
     const Layout L = frag_layout(sp, f);
@@ -1117,7 +1116,6 @@ int split_build_wave(SplitPlan& sp, const rimp2_frag* frags, const std::vector<i
       const int nq = sp.fp8 ? B2Q<true> : B2Q<false>, nc = sp.fp8 ? B2C<true> : B2C<false>;
       b2t += (long long)((X + nq - 1) / nq) * ((RL + nc - 1) / nc);
       qbl += (long long)((X + 31) / 32) * ((ov + kColRows - 1) / kColRows);
-      w.want_gamma = true;
     }
     w.sfd.push_back(s);
     off += L.total;

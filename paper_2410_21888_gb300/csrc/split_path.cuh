@@ -78,7 +78,6 @@ struct SplitWave {
   bool sep_energy = false;   // energies by k_split_energy instead of the last amplitude CTAs
   std::vector<SplitProb> probs_s;   // P_ab / P_ij of small extents (slice-stacked kernel)
   long long tiles_v = 0, tiles_c = 0, tiles_g = 0, tiles_s = 0, rows = 0, b2_tiles = 0, qblks = 0;
-  bool want_gamma = false;
   int max_x = 0;       // largest naux of the wave
   int amp_lpr = 32;    // lanes per row of the amplitude kernel
   double mma_v = 0, mma_c = 0, mma_g = 0;   // tensor-core FLOPs issued per launch
