@@ -15,7 +15,7 @@
 //   * the next 16 K elements are loaded into registers while the current ones are
 //     multiplied from one of two shared-memory buffers (one barrier per 16).
 // Measured (energy, Gamma, P_ij, P_ab; fixed 64 x 64 tiles over whole P matrices before):
-// nocc=10 nvir=40 naux=150 1042 -> 131 us, nocc=29 nvir=117 naux=437 19.8 -> 15.0 ms, 64
+// nocc=10 nvir=40 naux=150 1042 -> 148 us (131 with the other kernels' work since), nocc=29 nvir=117 naux=437 19.8 -> 15.0 ms, 64
 // monomers (nocc 8..20) 87.8 -> 46.2 ms; V at nocc=50 nvir=250 naux=750 runs at 1.24 TFLOP/s
 // of issued FMAs, the rate of a register-only DFMA loop (1.25).
 #pragma once

@@ -839,8 +839,8 @@ k_split_gemm(const SplitProb* __restrict__ probs, const long long* __restrict__ 
         tc_fence_after();
         // levels from the highest down; the set is released as soon as level 0 is in
         // registers (its fold and the renormalisation run while the next MMAs do).  Up to
-        // 24 columns a thread, two register buffers: the loads of level l-1 are in flight
-        // while level l is folded (wider tiles would spill)
+        // 12 columns a thread (24 with 8 epilogue warps), two register buffers: the loads of
+        // level l-1 are in flight while level l is folded (wider tiles would spill)
         auto fold = [&](int l, float (&v)[NC]) {
           const float sc = __int_as_float((127 - LB * l) << 23);   // 2^(-LB l)
           const f2x sc2 = f2_pack(sc, sc);
@@ -1438,8 +1438,8 @@ SplitLaunch split_launch_config(int slices, int bk, int n_tile, bool fp8) {
   } else {
     c.bk = bk == 16 ? 16 : 32;
     // 64 columns when no width is asked for: with 5 or 6 slices a stage is then small
-    // enough for three stages in shared memory.  (The plan asks per launch: 48 for V,
-    // whose two accumulator sets then fit TMEM, 80 for Gamma, 64 for P_ab / P_ij.)
+    // enough for three stages in shared memory.  (The plan asks per launch: 48, 64 or 80
+    // for V by its work, 80 for Gamma, 64 for P_ab / P_ij.)
     const int widest = slices <= 5 ? 96 : (slices == 6 ? 80 : 64);
     c.n_tile_max = (n_tile == 48 || n_tile == 64 || n_tile == 80 || n_tile == 96)
                        ? std::min(n_tile, widest) : 64;

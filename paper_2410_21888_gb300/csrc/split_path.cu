@@ -650,7 +650,6 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, unsigned amp_ctas, int s
   const int row = warp * GROUPS + lane / LPR, a = a0 + row, c0 = 4 * (lane % LPR);
   const int yq = 4 * (tid % (ROWS / 4)), yb = tid / (ROWS / 4);
 
-  // the next step's direct and transposed elements; their offsets advance within a j block
   // this CTA's share of the outputs that the contractions accumulate into
   {
     const long long ctas = (long long)strips * jranges * o, me = (long long)(blockIdx.x - F.pair_begin);
@@ -660,6 +659,7 @@ k_amp_split(const SplitFragDev* __restrict__ f, int nf, unsigned amp_ctas, int s
     for (long long e = me * 256 + tid; e < nv; e += ctas * 256) bs.pab[F.pab_off + e] = 0.0;
     for (long long e = me * 256 + tid; e < ng; e += ctas * 256) __stcs(bs.gamma + F.gamma_off + e, 0.0);
   }
+  // the next step's direct and transposed elements; their offsets advance within a j block
   float4 dh, dl, xh, xl;
   long long id = 0, ix = 0;
   const long long xstep = (long long)C * ldt;
