@@ -207,11 +207,11 @@ int rimp2_workspace_size(const rimp2_plan* plan, size_t* bytes);
  * hold rimp2_workspace_size() bytes; its contents are scratch.  Host-side validation
  * errors return before anything is launched.
  *
- * Two calls of one plan on the same inputs give the same bits for the energies and e_pair,
- * and for Gamma (FP64 path: always; split modes: while nocc x nvir, nvir rounded up to
- * whole digit rows, is below about 40,000: at most two K slabs then meet in an element).
- * P_ij and P_ab, and Gamma above that, are sums of FP64 atomics: equal up to the order
- * of their additions. */
+ * Two calls of one plan on the same inputs (autotune's trials apart) give the same bits for
+ * the energies and e_pair, and for Gamma (FP64 path: always; split modes: while nocc x nvir,
+ * nvir rounded up to whole digit rows, is below about 40,000: at most two K slabs then meet
+ * in an element).  P_ij and P_ab, and Gamma above that, are sums of FP64 atomics: equal up
+ * to the order of their additions. */
 int rimp2_energy_grad(rimp2_plan* plan, const rimp2_batch* batch, void* workspace,
                       size_t ws_bytes, void* stream);
 
